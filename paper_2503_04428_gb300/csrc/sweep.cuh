@@ -1017,43 +1017,48 @@ struct Sweep {
 };
 
 // Block-wide reductions into the control block, then the last-CTA commit.
+// (The maximum of the non-negative speeds is taken on their bit patterns:
+// integer compares, where an FP64 compare would occupy the FP64 pipe.)
 template <int NT>
-__device__ void finish_step(Ctrl* ctrl, double smax, int err, unsigned long long fb,
-                            unsigned long long it, unsigned long long mlp, long long step,
-                            double dt) {
-  __shared__ double red_s[NT / 32];
+__device__ void finish_step(Ctrl* ctrl, double speed, int err, unsigned long long fb,
+                            unsigned long long it, double dt) {
+  __shared__ unsigned long long red_s[NT / 32];
   __shared__ int red_e[NT / 32];
-  __shared__ unsigned long long red_f[NT / 32], red_i[NT / 32], red_m[NT / 32];
+  __shared__ unsigned long long red_f[NT / 32], red_i[NT / 32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  unsigned long long smax = dbits(speed);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    smax = fmax(smax, __shfl_xor_sync(0xffffffffu, smax, o));
-    const int e2 = __shfl_xor_sync(0xffffffffu, err, o);
-    err = err ? err : e2;
-    fb += __shfl_xor_sync(0xffffffffu, fb, o);
-    it += __shfl_xor_sync(0xffffffffu, it, o);
-    mlp += __shfl_xor_sync(0xffffffffu, mlp, o);
+    const unsigned long long s2 = __shfl_xor_sync(0xffffffffu, smax, o);
+    smax = smax > s2 ? smax : s2;
+  }
+  if (__any_sync(0xffffffffu, err != 0 || fb != 0 || it != 0)) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const int e2 = __shfl_xor_sync(0xffffffffu, err, o);
+      err = err ? err : e2;
+      fb += __shfl_xor_sync(0xffffffffu, fb, o);
+      it += __shfl_xor_sync(0xffffffffu, it, o);
+    }
   }
   if (lane == 0) {
     red_s[wid] = smax;
     red_e[wid] = err;
     red_f[wid] = fb;
     red_i[wid] = it;
-    red_m[wid] = mlp;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int w = 1; w < NT / 32; ++w) {
-      smax = fmax(smax, red_s[w]);
+      smax = smax > red_s[w] ? smax : red_s[w];
       err = err ? err : red_e[w];
       fb += red_f[w];
       it += red_i[w];
-      mlp += red_m[w];
     }
-    if (smax > 0.0) atomicMax(&ctrl->smax_next, dbits(smax));
+    const long long step = ((volatile Ctrl*)ctrl)->step;  // (constant until the commit below)
+    if (smax) atomicMax(&ctrl->smax_next, smax);
     if (fb) atomicAdd(&ctrl->fallbacks, fb);
     if (it) atomicAdd(&ctrl->iters, it);
-    if (mlp) atomicAdd(&ctrl->mlp, mlp);
     if (err) {
       if (atomicCAS(&ctrl->status, 0, err) == 0) ctrl->err_step = step;
     }
@@ -1077,23 +1082,15 @@ __device__ void finish_step(Ctrl* ctrl, double smax, int err, unsigned long long
   }
 }
 
-// Common step prologue: read the control block, decide dt.  Returns false
-// when the launch must do nothing (earlier failure, or t_end reached).
-__device__ __forceinline__ bool step_begin(const Ctrl* ctrl, double dt_host, double cfl,
-                                           double t_end, double& dt, double& t, long long& step,
-                                           int& cur) {
-  const volatile Ctrl* vc = ctrl;
-  if (vc->status != 0) return false;
-  t = vc->t;
-  step = vc->step;
-  cur = vc->cur;
-  if (dt_host > 0.0) {
-    dt = dt_host;
-  } else {
-    dt = cfl / vc->smax_cur;
-    if (t_end > 0.0) dt = fmin(dt, t_end - t);
-  }
-  return dt > 0.0;
+// Time step of a launch: the host's dt, or the CFL step clipped to t_end (0
+// or less: nothing to do).  One thread computes it for the CTA: an FP64
+// operation costs a warp 19 cycles of an SM's FP64 pipe whatever its active
+// lanes, so a division in every warp kept that pipe a quarter busy.
+__device__ __forceinline__ double step_dt(const volatile Ctrl* vc, double dt_host, double cfl, double t_end) {
+  if (dt_host > 0.0) return dt_host;
+  double dt = cfl / vc->smax_cur;
+  if (t_end > 0.0) dt = fmin(dt, t_end - vc->t);
+  return dt;
 }
 
 template <typename T, int DIM, int NSX, int RS, int MODE>
@@ -1102,10 +1099,20 @@ __global__ void __launch_bounds__(SweepShape<T, DIM, NSX>::NT,
     sweep_kernel(const SweepArgs<T> args) {
   using S = SweepShape<T, DIM, NSX>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  double dtd, t;
-  long long step;
-  int cur;
-  if (!step_begin(args.ctrl, args.dt_host, args.cfl, args.t_end, dtd, t, step, cur)) return;
+  // dt (and the heating factor) come from thread 0 and are read after the
+  // barrier that ends the staging; a launch behind a failed one (dt 0)
+  // writes nothing.
+  __shared__ double s_dt;
+  __shared__ T s_hfac;
+  const volatile Ctrl* vc = args.ctrl;
+  const int cur = vc->cur;
+  if (threadIdx.x == 0) {
+    s_dt = vc->status != 0 ? 0.0 : step_dt(vc, args.dt_host, args.cfl, args.t_end);
+    if (args.heating == HEAT_NI56) {
+      const double t = vc->t;
+      s_hfac = (T)(args.ni_lambda * (args.ni_a * exp(-t / args.ni_tni) + args.ni_qco * exp(-t / args.ni_tco)));
+    }
+  }
 
   Sweep<T, DIM, NSX, RS, MODE> sw(args, reinterpret_cast<T*>(smem_raw));
   if (sw.tsum)
@@ -1114,13 +1121,13 @@ __global__ void __launch_bounds__(SweepShape<T, DIM, NSX>::NT,
   sw.y0 = blockIdx.y * S::TY;
   sw.stage_geometry();  // (read after the first barrier below)
   sw.n2 = DIM == 3 ? args.n[2] : 1;
-  sw.dt = (T)dtd;
-  sw.half_dt = T(0.5) * sw.dt;
   sw.Uin = cur ? args.B : args.A;
   sw.Uout = cur ? args.Aw : args.B;
-  if (args.heating == HEAT_NI56) {
-    sw.hfac = (T)(args.ni_lambda * (args.ni_a * exp(-t / args.ni_tni) + args.ni_qco * exp(-t / args.ni_tco)));
-  }
+  auto set_dt = [&]() {
+    sw.dt = (T)s_dt;
+    sw.half_dt = T(0.5) * sw.dt;
+    sw.hfac = args.heating == HEAT_NI56 ? s_hfac : T(0);
+  };
 
   if constexpr (DIM == 3) {
     const int z0 = blockIdx.z * args.zchunk;
@@ -1128,6 +1135,8 @@ __global__ void __launch_bounds__(SweepShape<T, DIM, NSX>::NT,
     sw.z1 = z1;
     for (int q = z0 - 2; q <= z0; ++q) sw.load_plane(q);
     __syncthreads();
+    if (!(s_dt > 0.0)) return;
+    set_dt();
     sw.template predictor<PRED_ZHI>(z0 - 1);
     __syncthreads();
     // Plane k: its face states, then its x/y faces and the z face below it;
@@ -1148,6 +1157,8 @@ __global__ void __launch_bounds__(SweepShape<T, DIM, NSX>::NT,
     sw.z1 = 1;
     sw.load_plane(0);
     __syncthreads();
+    if (!(s_dt > 0.0)) return;
+    set_dt();
     sw.template predictor<PRED_ALL>(0);
     __syncthreads();
     sw.template faces<true, false>(0);
@@ -1183,7 +1194,7 @@ __global__ void __launch_bounds__(SweepShape<T, DIM, NSX>::NT,
     if (threadIdx.x < S::NV) args.tot_part[threadIdx.x * ncta + cta] = sw.tsum[threadIdx.x * S::NI];
   }
   finish_step<S::NT>(args.ctrl, (double)sw.smax, sw.err, sw.n_fallback,
-                     (MODE & 1) ? (unsigned long long)sw.t_iters : sw.n_iters, 0ull, step, dtd);
+                     (MODE & 1) ? (unsigned long long)sw.t_iters : sw.n_iters, s_dt);
 }
 
 template <typename T, int DIM, int NSX, int RS, int MODE>
