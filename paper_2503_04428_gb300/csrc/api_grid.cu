@@ -113,7 +113,7 @@ static int upload_d(hydro_ctx* h, const std::vector<double>& v, double** out) {
 
 // Index of each geometry array inside hydro_ctx::geo.
 enum {
-  G_IDXC0 = 0, G_IDXC1, G_IDXC2, G_HW0, G_HW1, G_HW2, G_IW0, G_IW1, G_IW2, G_IR, G_IS,
+  G_SQ0 = 0, G_SQ1, G_SQ2, G_SF0, G_SF1, G_SF2, G_IW0, G_IW1, G_IW2, G_IR, G_IS,
   G_AF, G_INVA, G_GA, G_QR, G_GR, G_GPT, G_BF, G_INVB, G_ZC, G_GT, G_QT, G_INVC, G_COUNT
 };
 static_assert(G_COUNT <= (int)(sizeof(((hydro_ctx*)nullptr)->geo) / sizeof(void*)),
@@ -166,9 +166,9 @@ static int build_geometry(hydro_ctx* h) {
       }
     }
     const int m = (int)ax[d].w.size();
-    std::vector<double> idxc(m, 0.0), hw(m), iw(m);
+    // (the outermost ghosts need no slope)
+    std::vector<double> idxc(m, 0.0), sq(m, 1.0), sf(m, 0.0), iw(m);
     for (int k = 0; k < m; ++k) {
-      hw[k] = 0.5 * ax[d].w[k];
       iw[k] = 1.0 / ax[d].w[k];
       if (k > 0) {
         const double cm = ax[d].lo[k - 1] + 0.5 * ax[d].w[k - 1];
@@ -176,9 +176,13 @@ static int build_geometry(hydro_ctx* h) {
         idxc[k] = 1.0 / (c0 - cm);
       }
     }
+    for (int k = 1; k + 1 < m; ++k) {
+      sq[k] = idxc[k + 1] / idxc[k];
+      sf[k] = 0.5 * ax[d].w[k] * idxc[k];
+    }
     int st;
-    if ((st = upload<T>(h, idxc, &g[G_IDXC0 + d]))) return st;
-    if ((st = upload<T>(h, hw, &g[G_HW0 + d]))) return st;
+    if ((st = upload<T>(h, sq, &g[G_SQ0 + d]))) return st;
+    if ((st = upload<T>(h, sf, &g[G_SF0 + d]))) return st;
     if ((st = upload<T>(h, iw, &g[G_IW0 + d]))) return st;
   }
   // spherical width factors (ext)
@@ -311,8 +315,8 @@ template <typename T>
 static Geom<T> geom_of(const hydro_ctx* h) {
   Geom<T> g;
   for (int d = 0; d < 3; ++d) {
-    g.inv_dxc[d] = (const T*)h->geo[G_IDXC0 + d];
-    g.hw[d] = (const T*)h->geo[G_HW0 + d];
+    g.sq[d] = (const T*)h->geo[G_SQ0 + d];
+    g.sf[d] = (const T*)h->geo[G_SF0 + d];
     g.inv_w[d] = (const T*)h->geo[G_IW0 + d];
   }
   g.inv_r = (const T*)h->geo[G_IR];

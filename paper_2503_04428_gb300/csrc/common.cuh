@@ -45,8 +45,8 @@ struct Ctrl {
 // (n entries) or interior face (n+1 entries).
 template <typename T>
 struct Geom {
-  const T* inv_dxc[3];  // ext: 1/(x_i - x_{i-1})
-  const T* hw[3];       // ext: half coordinate width
+  const T* sq[3];       // ext: (x_i - x_{i-1})/(x_{i+1} - x_i), the slopes' ratio of spacings
+  const T* sf[3];       // ext: half coordinate width / (x_i - x_{i-1})
   const T* inv_w[3];    // ext: 1/coordinate width
   const T* inv_r;       // ext axis 0: 1/r_i (spherical)
   const T* inv_s;       // ext axis 1: 1/s_j, s_j = (sin th_- + sin th_+)/2 (spherical)

@@ -38,12 +38,58 @@ struct Gas {
   T pow_c;    // 2 gamma/(gamma - 1)
 };
 
-// Square roots.  The FP32 bulk takes x rsqrt(x) (about 3 ulp; x > 0 on every
-// path that uses it): the correctly rounded sqrtf sequence cost 2-3 % of the
-// FP32 step's instructions.
+// FP64 on this part: one warp instruction occupies an SM's FP64 pipe for 19
+// cycles (measured; DFMA, DADD, DMUL and the compares alike, whatever the
+// active lanes), an integer instruction an ALU for about half a cycle.  So
+// the FP64 forms below count FP64 operations: signs and orders are read from
+// the bit patterns, and reciprocals and square roots take one third-order
+// step (error e -> O(e^3); Householder, The Numerical Treatment of a Single
+// Nonlinear Equation, 1970) from the documented PTX approximations, whose
+// relative error is below 2^-18: 3 and 5 FP64 operations against 4.5 and 7.5
+// of the correctly rounded ones, with errors of about 1 ulp.
+
+// 1/x (FP32: the fast 2-ulp form; FP64: x normal, |x| < 2^1021).
+template <typename T> __device__ __forceinline__ T rcp(T x);
+template <> __device__ __forceinline__ float rcp<float>(float x) { return __fdividef(1.0f, x); }
+template <> __device__ __forceinline__ double rcp<double>(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  double e = fma(-x, r, 1.0);
+  e = fma(e, e, e);
+  return fma(r, e, r);
+}
+
+// Square roots of positive x.  The FP32 bulk takes x rsqrt(x) (about 3 ulp):
+// the correctly rounded sqrtf sequence cost 2-3 % of the FP32 step's
+// instructions.
 template <typename T> __device__ __forceinline__ T dsqrt(T x);
-template <> __device__ __forceinline__ double dsqrt<double>(double x) { return sqrt(x); }
 template <> __device__ __forceinline__ float dsqrt<float>(float x) { return x * rsqrtf(x); }
+template <> __device__ __forceinline__ double dsqrt<double>(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double s = x * y;            // sqrt(x) (1 + d), x y^2 = 1 - e
+  const double e = fma(-s, y, 1.0);
+  return fma(s, e * fma(0.375, e, 0.5), s);
+}
+
+// x > 0 (false for NaN).
+__device__ __forceinline__ bool is_pos(float x) { return x > 0.0f; }
+__device__ __forceinline__ bool is_pos(double x) {
+  return (unsigned long long)__double_as_longlong(x) - 1ull < 0x7ff0000000000000ull;
+}
+// x >= 0 up to the sign of zero (-0 counts as negative).
+__device__ __forceinline__ bool is_nonneg(float x) { return x >= 0.0f; }
+__device__ __forceinline__ bool is_nonneg(double x) { return __double2hiint(x) >= 0; }
+// The smaller and the larger of two numbers (neither NaN).
+__device__ __forceinline__ long long order_key(double x) {
+  const long long b = __double_as_longlong(x);
+  return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ float min_of(float a, float b) { return fminf(a, b); }
+__device__ __forceinline__ float max_of(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ double min_of(double a, double b) { return order_key(a) < order_key(b) ? a : b; }
+__device__ __forceinline__ double max_of(double a, double b) { return order_key(a) < order_key(b) ? b : a; }
+
 // Powers (x > 0) as exp2(y log2 x): a few ulp (FP64: relative 1e-15 at the
 // exponents of the exact solver), against the accurate pow/powf, whose
 // extended-precision logarithm is several times longer and dominated the
@@ -53,11 +99,11 @@ template <> __device__ __forceinline__ double dpow<double>(double x, double y) {
 template <> __device__ __forceinline__ float dpow<float>(float x, float y) { return exp2f(y * log2f(x)); }
 
 // Quotient of the state conversions, wave speeds and the exact solver
-// (pressure functions, guess, Newton step, sampling): correctly rounded in
-// FP64, the fast 2-ulp division in FP32 (the FP32 bulk's rounding error is
-// ~1e-7 per operation either way, and Newton corrects its own iterates; the
-// IEEE sequence is several times longer).
-template <typename T> __device__ __forceinline__ T qdiv(T a, T b) { return a / b; }
+// (pressure functions, guess, Newton step, sampling): a times the reciprocal
+// above (FP32: the fast 2-ulp division; the FP32 bulk's rounding error is
+// ~1e-7 per operation either way, and Newton corrects its own iterates).
+// FP64: b normal, |b| < 2^1021; 4 FP64 operations against 7.5.
+template <typename T> __device__ __forceinline__ T qdiv(T a, T b) { return a * rcp<T>(b); }
 template <> __device__ __forceinline__ float qdiv<float>(float a, float b) { return __fdividef(a, b); }
 
 template <typename T> __device__ __forceinline__ T temp_tol();
@@ -146,6 +192,12 @@ struct GasRad : Gas<T> {
   }
 };
 
+// The larger of two non-negative numbers (FP64: by their bit patterns).
+__device__ __forceinline__ float larger_speed(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ double larger_speed(double a, double b) {
+  return __double_as_longlong(a) < __double_as_longlong(b) ? b : a;
+}
+
 template <typename T> __device__ __forceinline__ T dexp(T x);
 template <> __device__ __forceinline__ double dexp<double>(double x) { return exp(x); }
 template <> __device__ __forceinline__ float dexp<float>(float x) { return expf(x); }
@@ -159,7 +211,7 @@ template <> __device__ __forceinline__ float dlog<float>(float x) { return logf(
 template <typename T, int D, int NSX, typename G>
 __device__ __forceinline__ void to_prim(const T* U, T* W, const G& gas) {
   const T rho = U[0];
-  const T ir = qdiv(T(1), rho);
+  const T ir = rcp<T>(rho);
   T ke = T(0);
 #pragma unroll
   for (int d = 0; d < D; ++d) {
@@ -183,7 +235,7 @@ template <typename T, int D, int NSX, typename G>
 __device__ __forceinline__ void to_prim_ct(const T* U, T* W, T& c2, T& t, const G& gas, T t0 = T(0),
                                            int* its = nullptr) {
   const T rho = U[0];
-  const T ir = qdiv(T(1), rho);
+  const T ir = rcp<T>(rho);
   T ke = T(0);
 #pragma unroll
   for (int d = 0; d < D; ++d) {
@@ -199,7 +251,7 @@ __device__ __forceinline__ void to_prim_ct(const T* U, T* W, T& c2, T& t, const 
 template <typename T, int D, int NSX, typename G>
 __device__ __forceinline__ void to_prim_c2(const T* U, T* W, T& c2, const G& gas) {
   const T rho = U[0];
-  const T ir = qdiv(T(1), rho);
+  const T ir = rcp<T>(rho);
   T ke = T(0);
 #pragma unroll
   for (int d = 0; d < D; ++d) {
@@ -276,17 +328,39 @@ __device__ __forceinline__ void phys_flux(const T* W, T* F, const G& gas) {
 // Slope limiters of Eq. 17 (minmod, van Leer, van Albada; 0 = first order),
 // applied to the one-sided differences dm, dp; zero when they differ in sign.
 // ---------------------------------------------------------------------------
+// minmod: the argument of smaller magnitude where the signs agree.  FP32:
+// the hardware minimum of magnitudes that carries the product's sign,
+// clamped at 0, with dm's sign put back (3 instructions).  FP64: signs and
+// magnitudes compared as integers (no FP64 operation).
+__device__ __forceinline__ float minmod(float dm, float dp) {
+  float m;
+  asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(m) : "f"(dm), "f"(dp));
+  return __int_as_float(__float_as_int(fmaxf(m, 0.0f)) | (__float_as_int(dm) & 0x80000000));
+}
+__device__ __forceinline__ double minmod(double dm, double dp) {
+  const unsigned long long bm = (unsigned long long)__double_as_longlong(dm) & 0x7fffffffffffffffull;
+  const unsigned long long bp = (unsigned long long)__double_as_longlong(dp) & 0x7fffffffffffffffull;
+  const double m = bm < bp ? dm : dp;
+  return (__double2hiint(dm) ^ __double2hiint(dp)) < 0 ? 0.0 : m;
+}
+// The product of two slopes is taken as positive from here on (FP64: the
+// quotients below need a normal divisor; slopes of less than ~1e-145 do not
+// matter).
+__device__ __forceinline__ bool slopes_agree(float pr) { return pr > 0.0f; }
+__device__ __forceinline__ bool slopes_agree(double pr) { return __double2hiint(pr) > 0x01d00000; }  // > 2^-994
+
+// Homogeneous of degree 1: limit(k, s a, s b) = s limit(k, a, b) for s > 0.
 template <typename T>
 __device__ __forceinline__ T limit(int kind, T dm, T dp) {
+  if (kind == LIM_MINMOD) return minmod(dm, dp);
   const T pr = dm * dp;
-  if (kind == LIM_FIRST || !(pr > T(0))) return T(0);
-  if (kind == LIM_MINMOD) return dm > T(0) ? fmin(dm, dp) : fmax(dm, dp);
+  if (kind == LIM_FIRST || !slopes_agree(pr)) return T(0);
   if (kind == LIM_VANLEER) return qdiv(T(2) * pr, dm + dp);
   return qdiv(pr * (dm + dp), dm * dm + dp * dp);
 }
 
 // ---------------------------------------------------------------------------
-// HLL with Davis wave-speed bounds.
+// Approximate Riemann solvers.
 // ---------------------------------------------------------------------------
 // Flux through a face normal to DIR and the conserved state of a primitive
 // state whose internal energy per volume e is already known.
@@ -315,167 +389,109 @@ __device__ __forceinline__ void flux_cons_e(const T* W, T e, T* F, T* U) {
   }
 }
 
-// HLL for the gas + radiation EoS: one temperature solve per side gives e
-// and the Eq. 7 sound speed.
-// (TL, TR > 0: the face states' temperatures, known to the caller; no solve)
-template <typename T, int D, int NSX, int DIR, typename G>
-__device__ __forceinline__ void riemann_hll_rad(const T* WL, const T* WR, T* F, const G& gas, T TL = T(0),
-                                                T TR = T(0)) {
-  constexpr int NV = 2 + D + NSX;
-  T eL, c2L, eR, c2R;
-  if (TL > T(0)) gas.from_t(WL[0], TL, eL, c2L);
-  else gas.from_p(WL[0], WL[1 + D], eL, c2L);
-  if (TR > T(0)) gas.from_t(WR[0], TR, eR, c2R);
-  else gas.from_p(WR[0], WR[1 + D], eR, c2R);
-  const T cL = dsqrt(c2L), cR = dsqrt(c2R);
-  const T SL = fmin(WL[1 + DIR] - cL, WR[1 + DIR] - cR);
-  const T SR = fmax(WL[1 + DIR] + cL, WR[1 + DIR] + cR);
-  T FL[NV], FR[NV], UL[NV], UR[NV];
-  flux_cons_e<T, D, NSX, DIR>(WL, eL, FL, UL);
-  flux_cons_e<T, D, NSX, DIR>(WR, eR, FR, UR);
-  if (SL >= T(0)) {
+// HLL flux of two states with known internal energies and sound speeds,
+// Davis speeds S_L, S_R.  With S_L clamped to <= 0 and S_R to >= 0 (the
+// supersonic cases included), F = a F_L + b F_R + c (U_R - U_L) with a =
+// S_R/(S_R - S_L), b = -S_L/(S_R - S_L), c = S_L S_R/(S_R - S_L); and since
+// F = u U + P (0, n, u), each side's conserved state enters with one factor
+// k_L = a u_L - c, k_R = b u_R + c: about 45 operations instead of the ~75 of
+// forming both fluxes and both conserved states.
+template <typename T, int D, int NSX, int DIR>
+__device__ __forceinline__ void hll_flux(const T* WL, const T* WR, T eL, T eR, T cL, T cR, T* F) {
+  const T uL = WL[1 + DIR], uR = WR[1 + DIR], pL = WL[1 + D], pR = WR[1 + D];
+  T SL = min_of(uL - cL, uR - cR), SR = max_of(uL + cL, uR + cR);
+  SL = is_nonneg(SL) ? T(0) : SL;
+  SR = is_nonneg(SR) ? SR : T(0);
+  const T inv = rcp<T>(SR - SL);
+  const T a = SR * inv, b = -SL * inv, c = (SL * SR) * inv;
+  const T auL = a * uL, buR = b * uR;
+  const T kL = auL - c, kR = buR + c;
+  const T mL = WL[0] * kL, mR = WR[0] * kR;
+  T vL = T(0), vR = T(0);
 #pragma unroll
-    for (int v = 0; v < NV; ++v) F[v] = FL[v];
-    return;
+  for (int d = 0; d < D; ++d) {
+    vL += WL[1 + d] * WL[1 + d];
+    vR += WR[1 + d] * WR[1 + d];
+    F[1 + d] = mL * WL[1 + d] + mR * WR[1 + d];
   }
-  if (SR <= T(0)) {
+  F[0] = mL + mR;
+  F[1 + DIR] += a * pL + b * pR;
+  F[1 + D] = (kL * eL + auL * pL) + (kR * eR + buR * pR) + T(0.5) * (mL * vL + mR * vR);
 #pragma unroll
-    for (int v = 0; v < NV; ++v) F[v] = FR[v];
-    return;
-  }
-  const T inv = qdiv(T(1), SR - SL);
-  const T sLR = SL * SR;
-#pragma unroll
-  for (int v = 0; v < NV; ++v) F[v] = (SR * FL[v] - SL * FR[v] + sLR * (UR[v] - UL[v])) * inv;
+  for (int s = 0; s < NSX; ++s) F[2 + D + s] = mL * WL[2 + D + s] + mR * WR[2 + D + s];
 }
 
-// HLLC for the gas + radiation EoS (the star states need only E, p, rho, u).
-template <typename T, int D, int NSX, int DIR, typename G>
-__device__ __forceinline__ void riemann_hllc_rad(const T* WL, const T* WR, T* F, const G& gas, T TL = T(0),
-                                                 T TR = T(0)) {
-  constexpr int NV = 2 + D + NSX;
-  const T rL = WL[0], rR = WR[0], uL = WL[1 + DIR], uR = WR[1 + DIR];
-  const T pL = WL[1 + D], pR = WR[1 + D];
-  T eL, c2L, eR, c2R;
-  if (TL > T(0)) gas.from_t(rL, TL, eL, c2L);
-  else gas.from_p(rL, pL, eL, c2L);
-  if (TR > T(0)) gas.from_t(rR, TR, eR, c2R);
-  else gas.from_p(rR, pR, eR, c2R);
-  const T cL = dsqrt(c2L), cR = dsqrt(c2R);
-  const T SL = fmin(uL - cL, uR - cR);
-  const T SR = fmax(uL + cL, uR + cR);
-  T Fk[NV], Uk[NV];
-  if (SL >= T(0)) {
-    flux_cons_e<T, D, NSX, DIR>(WL, eL, F, Uk);
-    return;
-  }
-  if (SR <= T(0)) {
-    flux_cons_e<T, D, NSX, DIR>(WR, eR, F, Uk);
-    return;
-  }
-  const T aL = rL * (SL - uL), aR = rR * (SR - uR);
+// HLLC flux of two states with known internal energies and sound speeds: the
+// contact is restored; star states keep their side's tangential velocities
+// and scalars.  The flux is that of the state on the face: V (rho, rho u_t,
+// rho V, E + P, rho f) + (0, n P, 0), with V, rho, P, E those of the side
+// where the flow is supersonic and of its star state (V = S*, rho* = rho (S -
+// u)/(S - S*), P* = P + rho (S - u)(S* - u)) otherwise: two quotients instead
+// of the four of F + S (U* - U).
+template <typename T, int D, int NSX, int DIR>
+__device__ __forceinline__ void hllc_flux(const T* WL, const T* WR, T eL, T eR, T cL, T cR, T* F) {
+  const T uL = WL[1 + DIR], uR = WR[1 + DIR], pL = WL[1 + D], pR = WR[1 + D];
+  const T SL = min_of(uL - cL, uR - cR), SR = max_of(uL + cL, uR + cR);
+  const T aL = WL[0] * (SL - uL), aR = WR[0] * (SR - uR);
   const T Ss = qdiv(pR - pL + uL * aL - uR * aR, aL - aR);
-  const bool left = Ss >= T(0);
-  T W[NV];
+  const bool supL = is_nonneg(SL), supR = !is_pos(SR);
+  const bool left = supL || (!supR && is_nonneg(Ss));  // the side of the contact
+  T W[2 + D + NSX];
 #pragma unroll
-  for (int v = 0; v < NV; ++v) W[v] = left ? WL[v] : WR[v];
-  const T S = left ? SL : SR;
-  const T a = left ? aL : aR;
+  for (int v = 0; v < 2 + D + NSX; ++v) W[v] = left ? WL[v] : WR[v];
+  const T S = left ? SL : SR, a = left ? aL : aR, e = left ? eL : eR;  // a = rho (S - u)
   const T rho = W[0], un = W[1 + DIR], p = W[1 + D];
-  flux_cons_e<T, D, NSX, DIR>(W, left ? eL : eR, Fk, Uk);
-  const T fac = qdiv(a, S - Ss);
-  T Us[NV];
-  Us[0] = fac;
+  T v2 = T(0);
 #pragma unroll
-  for (int d = 0; d < D; ++d) Us[1 + d] = fac * W[1 + d];
-  Us[1 + DIR] = fac * Ss;
-  Us[1 + D] = fac * (qdiv(Uk[1 + D], rho) + (Ss - un) * (Ss + qdiv(p, a)));
+  for (int d = 0; d < D; ++d) v2 += W[1 + d] * W[1 + d];
+  const T E = e + T(0.5) * rho * v2;
+  const T inv = rcp<T>(S - Ss);
+  const bool sup = left ? supL : supR;
+  const T V = sup ? un : Ss;
+  const T pS = sup ? p : p + a * (Ss - un);
+  const T rS = sup ? rho : a * inv;
+  const T ES = sup ? E : (E * (S - un) - p * un + pS * Ss) * inv;
+  const T m = rS * V;
+  F[0] = m;
 #pragma unroll
-  for (int s = 0; s < NSX; ++s) Us[2 + D + s] = fac * W[2 + D + s];
+  for (int d = 0; d < D; ++d) F[1 + d] = m * W[1 + d];
+  F[1 + DIR] = m * V + pS;
+  F[1 + D] = V * (ES + pS);
 #pragma unroll
-  for (int v = 0; v < NV; ++v) F[v] = Fk[v] + S * (Us[v] - Uk[v]);
+  for (int s = 0; s < NSX; ++s) F[2 + D + s] = m * W[2 + D + s];
+}
+
+// Internal energy and sound speed of a face state: from its temperature t
+// where the caller knows it (gas + radiation, t > 0), else from (rho, P).
+template <typename T, typename G>
+__device__ __forceinline__ void face_e_c(const G& gas, T rho, T p, T t, T& e, T& c) {
+  T c2;
+  if constexpr (G::RAD) {
+    if (t > T(0)) gas.from_t(rho, t, e, c2);
+    else gas.from_p(rho, p, e, c2);
+  } else {
+    e = p * gas.igm1;
+    c2 = qdiv(gas.g * p, rho);
+  }
+  c = dsqrt(c2);
+}
+
+// HLL and HLLC with Davis wave-speed bounds (TL, TR: the face states'
+// temperatures, gas + radiation).
+template <typename T, int D, int NSX, int DIR, typename G>
+__device__ __forceinline__ void riemann_hll(const T* WL, const T* WR, T* F, const G& gas, T TL = T(0), T TR = T(0)) {
+  T eL, eR, cL, cR;
+  face_e_c<T>(gas, WL[0], WL[1 + D], TL, eL, cL);
+  face_e_c<T>(gas, WR[0], WR[1 + D], TR, eR, cR);
+  hll_flux<T, D, NSX, DIR>(WL, WR, eL, eR, cL, cR, F);
 }
 
 template <typename T, int D, int NSX, int DIR, typename G>
-__device__ __forceinline__ void riemann_hll(const T* WL, const T* WR, T* F, const G& gas) {
-  if constexpr (G::RAD) {
-    riemann_hll_rad<T, D, NSX, DIR>(WL, WR, F, gas);
-    return;
-  }
-  constexpr int NV = 2 + D + NSX;
-  const T cL = dsqrt(qdiv(gas.g * WL[1 + D], WL[0]));
-  const T cR = dsqrt(qdiv(gas.g * WR[1 + D], WR[0]));
-  const T SL = fmin(WL[1 + DIR] - cL, WR[1 + DIR] - cR);
-  const T SR = fmax(WL[1 + DIR] + cL, WR[1 + DIR] + cR);
-  T FL[NV], FR[NV];
-  if (SL >= T(0)) {
-    phys_flux<T, D, NSX, DIR>(WL, F, gas);
-    return;
-  }
-  if (SR <= T(0)) {
-    phys_flux<T, D, NSX, DIR>(WR, F, gas);
-    return;
-  }
-  T UL[NV], UR[NV];
-  phys_flux<T, D, NSX, DIR>(WL, FL, gas);
-  phys_flux<T, D, NSX, DIR>(WR, FR, gas);
-  to_cons<T, D, NSX>(WL, UL, gas);
-  to_cons<T, D, NSX>(WR, UR, gas);
-  const T inv = qdiv(T(1), SR - SL);
-  const T sLR = SL * SR;
-#pragma unroll
-  for (int v = 0; v < NV; ++v) F[v] = (SR * FL[v] - SL * FR[v] + sLR * (UR[v] - UL[v])) * inv;
-}
-
-// ---------------------------------------------------------------------------
-// HLLC: the contact is restored; star states keep their side's tangential
-// velocities and scalars.  Branches: SL>=0 -> F_L; S*>=0 -> F*_L; SR>0 -> F*_R;
-// otherwise F_R.
-// ---------------------------------------------------------------------------
-template <typename T, int D, int NSX, int DIR, typename G>
-__device__ __forceinline__ void riemann_hllc(const T* WL, const T* WR, T* F, const G& gas) {
-  if constexpr (G::RAD) {
-    riemann_hllc_rad<T, D, NSX, DIR>(WL, WR, F, gas);
-    return;
-  }
-  constexpr int NV = 2 + D + NSX;
-  const T rL = WL[0], rR = WR[0], uL = WL[1 + DIR], uR = WR[1 + DIR];
-  const T pL = WL[1 + D], pR = WR[1 + D];
-  const T cL = dsqrt(qdiv(gas.g * pL, rL)), cR = dsqrt(qdiv(gas.g * pR, rR));
-  const T SL = fmin(uL - cL, uR - cR);
-  const T SR = fmax(uL + cL, uR + cR);
-  if (SL >= T(0)) {
-    phys_flux<T, D, NSX, DIR>(WL, F, gas);
-    return;
-  }
-  if (SR <= T(0)) {
-    phys_flux<T, D, NSX, DIR>(WR, F, gas);
-    return;
-  }
-  const T aL = rL * (SL - uL), aR = rR * (SR - uR);
-  const T Ss = qdiv(pR - pL + uL * aL - uR * aR, aL - aR);
-  // pick the side of the contact
-  const bool left = Ss >= T(0);
-  T W[NV];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) W[v] = left ? WL[v] : WR[v];
-  const T S = left ? SL : SR;
-  const T a = left ? aL : aR;  // rho_K (S_K - u_K)
-  const T rho = W[0], un = W[1 + DIR], p = W[1 + D];
-  T Fk[NV], Uk[NV];
-  phys_flux<T, D, NSX, DIR>(W, Fk, gas);
-  to_cons<T, D, NSX>(W, Uk, gas);
-  const T fac = qdiv(a, S - Ss);
-  T Us[NV];
-  Us[0] = fac;
-#pragma unroll
-  for (int d = 0; d < D; ++d) Us[1 + d] = fac * W[1 + d];
-  Us[1 + DIR] = fac * Ss;
-  Us[1 + D] = fac * (qdiv(Uk[1 + D], rho) + (Ss - un) * (Ss + qdiv(p, a)));
-#pragma unroll
-  for (int s = 0; s < NSX; ++s) Us[2 + D + s] = fac * W[2 + D + s];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) F[v] = Fk[v] + S * (Us[v] - Uk[v]);
+__device__ __forceinline__ void riemann_hllc(const T* WL, const T* WR, T* F, const G& gas, T TL = T(0), T TR = T(0)) {
+  T eL, eR, cL, cR;
+  face_e_c<T>(gas, WL[0], WL[1 + D], TL, eL, cL);
+  face_e_c<T>(gas, WR[0], WR[1 + D], TR, eR, cR);
+  hllc_flux<T, D, NSX, DIR>(WL, WR, eL, eR, cL, cR, F);
 }
 
 // ---------------------------------------------------------------------------

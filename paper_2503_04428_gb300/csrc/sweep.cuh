@@ -82,8 +82,8 @@ struct SweepShape {
   static constexpr size_t rad_elems = (size_t)2 * NFX + 2 * NFY + 3 * NFZ + (size_t)WP * WPL;
   // the x and y geometry factors of the CTA's cells, staged once per CTA
   // (GX_N arrays over the TX + 2 predictor columns, GY_N over the TY + 2 rows)
-  enum { GX_IDM, GX_IDP, GX_HW, GX_IW, GX_IR, GX_AF, GX_INVA, GX_GA, GX_QR, GX_GR, GX_G, GX_N };
-  enum { GY_IDM, GY_IDP, GY_HW, GY_IW, GY_IS, GY_BF, GY_INVB, GY_ZC, GY_GT, GY_QT, GY_N };
+  enum { GX_SQ, GX_SF, GX_IW, GX_IR, GX_AF, GX_INVA, GX_GA, GX_QR, GX_GR, GX_G, GX_N };
+  enum { GY_SQ, GY_SF, GY_IW, GY_IS, GY_BF, GY_INVB, GY_ZC, GY_GT, GY_QT, GY_N };
   static constexpr size_t geo_elems = (size_t)GX_N * (TX + 2) + (DIM >= 2 ? (size_t)GY_N * (TY + 2) : 0);
   __host__ __device__ static constexpr size_t smem_bytes_for(int mode) {
     return (smem_elems + ((mode & 2) ? dual_elems : 0) + ((mode & 1) ? rad_elems : 0) + geo_elems) * sizeof(T);
@@ -235,14 +235,12 @@ struct Sweep {
     for (int p = threadIdx.x; p < TX + 2; p += NT) {
       const int gi = x0 - 1 + p;              // >= -1
       const int ge = min(gi, n0 + 1) + 2;     // extended (ghost) index
-      const int gp = min(gi, n0) + 3;         // the face above, extended
       const int gc = min(max(gi, 0), n0 - 1);  // interior cell
       const int gf = min(max(gi, 0), n0);      // interior face
       T* g = GXs + p;
       constexpr int st = TX + 2;
-      g[S::GX_IDM * st] = a.geo.inv_dxc[0][ge];
-      g[S::GX_IDP * st] = a.geo.inv_dxc[0][gp];
-      g[S::GX_HW * st] = a.geo.hw[0][ge];
+      g[S::GX_SQ * st] = a.geo.sq[0][ge];
+      g[S::GX_SF * st] = a.geo.sf[0][ge];
       g[S::GX_IW * st] = a.geo.inv_w[0][ge];
       g[S::GX_IR * st] = a.spherical ? a.geo.inv_r[ge] : T(1);
       g[S::GX_AF * st] = a.geo.Af[gf];
@@ -256,14 +254,12 @@ struct Sweep {
       for (int p = threadIdx.x; p < TY + 2; p += NT) {
         const int gj = y0 - 1 + p;
         const int ge = min(gj, n1 + 1) + 2;
-        const int gp = min(gj, n1) + 3;
         const int gc = min(max(gj, 0), n1 - 1);
         const int gf = min(max(gj, 0), n1);
         T* g = GYs + p;
         constexpr int st = TY + 2;
-        g[S::GY_IDM * st] = a.geo.inv_dxc[1][ge];
-        g[S::GY_IDP * st] = a.geo.inv_dxc[1][gp];
-        g[S::GY_HW * st] = a.geo.hw[1][ge];
+        g[S::GY_SQ * st] = a.geo.sq[1][ge];
+        g[S::GY_SF * st] = a.geo.sf[1][ge];
         g[S::GY_IW * st] = a.geo.inv_w[1][ge];
         g[S::GY_IS * st] = a.spherical ? a.geo.inv_s[ge] : T(1);
         g[S::GY_BF * st] = a.geo.Bf[gf];
@@ -401,25 +397,23 @@ struct Sweep {
   template <int DIR>
   __device__ __forceinline__ void faces_of(const T* Wm, const T* Wc, const T* Wp, int l, T* Wlo,
                                            T* Whi) const {
-    T idm, idp, h;
+    // the limiters are homogeneous: (dm idm, dp idp) -> idm limit(dm, dp q)
+    T q, f;
     if constexpr (DIR == 0) {
-      idm = gx(S::GX_IDM, l);
-      idp = gx(S::GX_IDP, l);
-      h = gx(S::GX_HW, l);
+      q = gx(S::GX_SQ, l);
+      f = gx(S::GX_SF, l);
     } else if constexpr (DIR == 1) {
-      idm = gy(S::GY_IDM, l);
-      idp = gy(S::GY_IDP, l);
-      h = gy(S::GY_HW, l);
+      q = gy(S::GY_SQ, l);
+      f = gy(S::GY_SF, l);
     } else {
-      idm = a.geo.inv_dxc[DIR][l + 2];
-      idp = a.geo.inv_dxc[DIR][l + 3];
-      h = a.geo.hw[DIR][l + 2];
+      q = a.geo.sq[DIR][l + 2];
+      f = a.geo.sf[DIR][l + 2];
     }
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-      const T sig = limit<T>(a.limiter, (Wc[v] - Wm[v]) * idm, (Wp[v] - Wc[v]) * idp);
-      Wlo[v] = Wc[v] - h * sig;
-      Whi[v] = Wc[v] + h * sig;
+      const T sig = limit<T>(a.limiter, Wc[v] - Wm[v], (Wp[v] - Wc[v]) * q);
+      Wlo[v] = Wc[v] - f * sig;
+      Whi[v] = Wc[v] + f * sig;
     }
   }
 
@@ -466,7 +460,7 @@ struct Sweep {
       a.grad.from_e_t(rho, u[1 + DIM] - T(0.5) * ke, w[1 + DIM], c2, t, *tp, &k);
 #pragma unroll
       for (int s = 0; s < NSX; ++s) w[2 + DIM + s] = u[2 + DIM + s] * ir;
-      if (!(w[0] > T(0)) || !(w[1 + DIM] > T(0))) {
+      if (!is_pos(w[0]) || !is_pos(w[1 + DIM])) {
 #pragma unroll
         for (int v = 0; v < NV; ++v) w[v] = Wc[v];
         t = a.grad.temp_p(Wc[0], Wc[1 + DIM], *tp, &k);
@@ -479,7 +473,7 @@ struct Sweep {
 #pragma unroll
       for (int v = 0; v < NV; ++v) u[v] = p[v * st] + dU[v];
       to_prim<T, DIM, NSX>(u, w, gas());
-      if (!(w[0] > T(0)) || !(w[1 + DIM] > T(0))) {
+      if (!is_pos(w[0]) || !is_pos(w[1 + DIM])) {
 #pragma unroll
         for (int v = 0; v < NV; ++v) w[v] = Wc[v];
         if (owned) ++n_fallback;
@@ -527,8 +521,8 @@ struct Sweep {
     }
   }
 
-  // a3 + a4 for plane gz: the predictor increment dU = dt/2 sum_d
-  // (F_d(W_lo) - F_d(W_hi))/h_d of every needed cell, and its predicted face
+  // a3 + a4 for plane gz: the predictor increment dU = sum_d
+  // (F_d(W_lo) - F_d(W_hi)) dt/(2 h_d) of every needed cell, and its predicted face
   // states.  PRED_ALL: tile plus halo, every face state of the plane;
   // PRED_ZHI / PRED_ZLO: tile cells only, the upper / lower z state.
   template <int PM>
@@ -585,7 +579,7 @@ struct Sweep {
         if (xlo) XTR[ixlo] = tl;
         if (xhi) XTL[ixhi] = th;
       }
-      const T ih = inv_h(0, px, py, gz);
+      const T ih = inv_h(0, px, py, gz) * half_dt;
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         dU[v] += (Fl[v] - Fh[v]) * ih;
@@ -610,7 +604,7 @@ struct Sweep {
         if (ylo) YTR[iylo] = tl;
         if (yhi) YTL[iyhi] = th;
       }
-      const T ih = inv_h(1, px, py, gz);
+      const T ih = inv_h(1, px, py, gz) * half_dt;
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         dU[v] += (Fl[v] - Fh[v]) * ih;
@@ -635,7 +629,7 @@ struct Sweep {
         if (zlo) ZTR[iz] = tl;
         if (zhi) ZTL[(gz & 1) * NFZ + iz] = th;
       }
-      const T ih = inv_h(2, px, py, gz);
+      const T ih = inv_h(2, px, py, gz) * half_dt;
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         dU[v] += (Fl[v] - Fh[v]) * ih;
@@ -643,8 +637,6 @@ struct Sweep {
         if (zhi) zhp[v * NFZ + iz] = Ph[v];
       }
     }
-#pragma unroll
-    for (int v = 0; v < NV; ++v) dU[v] = half_dt * dU[v];
     if constexpr (DIM < 3) {
       if (t < NI) {
 #pragma unroll
@@ -702,14 +694,10 @@ struct Sweep {
   template <int DIR>
   __device__ __forceinline__ void riemann_fixed(const T* WL, const T* WR, T* F, bool owned, T TL = T(0),
                                                 T TR = T(0)) {
-    if constexpr (EOS == 1 && RS == RS_HLL) {
-      riemann_hll_rad<T, DIM, NSX, DIR>(WL, WR, F, a.grad, TL, TR);
-    } else if constexpr (EOS == 1 && RS == RS_HLLC) {
-      riemann_hllc_rad<T, DIM, NSX, DIR>(WL, WR, F, a.grad, TL, TR);
-    } else if constexpr (RS == RS_HLL) {
-      riemann_hll<T, DIM, NSX, DIR>(WL, WR, F, gas());
+    if constexpr (RS == RS_HLL) {
+      riemann_hll<T, DIM, NSX, DIR>(WL, WR, F, gas(), TL, TR);
     } else if constexpr (RS == RS_HLLC) {
-      riemann_hllc<T, DIM, NSX, DIR>(WL, WR, F, gas());
+      riemann_hllc<T, DIM, NSX, DIR>(WL, WR, F, gas(), TL, TR);
     } else {
       int it = 0, kind = 0;
       const int st = riemann_exact<T, DIM, NSX, DIR>(WL, WR, F, a.gas, T(0), it, kind);
@@ -844,7 +832,7 @@ struct Sweep {
         for (int v = 0; v < NV; ++v) Uh[v] = Uo[v] + dUo[v];
         to_prim<T, DIM, NSX>(Uh, Wh, gas());
         to_prim<T, DIM, NSX>(Uo, Wo, gas());
-        P = (Wh[0] > T(0) && Wh[1 + DIM] > T(0)) ? Wh[1 + DIM] : Wo[1 + DIM];
+        P = (is_pos(Wh[0]) && is_pos(Wh[1 + DIM])) ? Wh[1 + DIM] : Wo[1 + DIM];
       }
       T Tth = P, Tph = P;
       if constexpr (DIM >= 2) Tth = tth;
@@ -966,7 +954,7 @@ struct Sweep {
 #pragma unroll
     for (int v = 0; v < NV; ++v) finite = finite && isfinite(Un[v]);
     if (!finite) err = err ? err : ST_NONFINITE;
-    else if (!(Wn[0] > T(0)) || !(Wn[1 + DIM] > T(0))) err = err ? err : ST_NEG;
+    else if (!is_pos(Wn[0]) || !is_pos(Wn[1 + DIM])) err = err ? err : ST_NEG;
     const T cs = dsqrt(c2n);
     T sp = T(0);
 #pragma unroll
@@ -982,7 +970,7 @@ struct Sweep {
       }
       sp += (fabs(ud) + cs) * ih;
     }
-    smax = fmax(smax, sp);
+    smax = larger_speed(smax, sp);
 #pragma unroll
     for (int v = 0; v < NV; ++v)
       if (v < nvact) Uout[(long long)v * a.ncell + c] = Un[v];
