@@ -93,8 +93,8 @@ typedef struct {
   long long mlp_faces;     /* exact solver: faces whose guess came from the MLP */
   double t;                /* simulation time (grid handles) */
   double last_dt;
-  int tile_x, tile_y, zchunk, threads;  /* launch shape chosen by the autotuner */
-  double tuned_us_per_step;            /* autotuner's best measured step time */
+  int tile_x, tile_y, zchunk, threads;  /* launch shape of the last step (batched: the autotuner's) */
+  double tuned_us_per_step;            /* batched autotuner's best measured step time; 0 for grids */
   /* Batched exact solver, owned faces that ran Newton (not two identical
    * states) and their iterations, by category: [0] started from Toro's guess,
    * [1] from the network's guess, both in the handle's precision; [2] FP32

@@ -1,7 +1,7 @@
 // api_grid.cu -- C ABI of the grid solver (include/hydro.h): handle lifetime,
 // geometry set-up, state transfer and validation, the step loop (one fused
 // sweep launch per step, optionally preceded by the monopole kernels), CUDA
-// graph capture of the device-dt step, the z-chunk autotuner and totals.
+// graph capture of the device-dt step and totals.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -407,7 +407,7 @@ static SweepArgs<T> sweep_args(hydro_ctx* h, double dt_host, double cfl, double 
   a.dt_host = dt_host;
   a.cfl = cfl;
   a.t_end = t_end;
-  a.zchunk = h->zchunk;
+  a.zchunk = 1;  // (planned at the launch)
   a.ctrl = ctrl;
   a.geo = geom_of<T>(h);
   a.xaxis = h->xaxis;
@@ -422,6 +422,16 @@ static SweepArgs<T> sweep_args(hydro_ctx* h, double dt_host, double cfl, double 
   for (int d = 0; d < 3; ++d) a.dvol[d] = h->dvol[d];
   a.dvz32 = reinterpret_cast<const float2*>(h->dvz32);
   return a;
+}
+
+// The plain 3D step: FP32 with HLL or HLLC marches (march3.cuh); FP64, which
+// is bound by the FP64 pipe, and the exact solver take the general sweep.
+static cudaError_t step3(const SweepArgs<double>& a, int nsx, int rs, cudaStream_t s, LaunchShape* sh) {
+  return sweep_dispatch<double, 3>(a, nsx, rs, s, sh);
+}
+static cudaError_t step3(const SweepArgs<float>& a, int nsx, int rs, cudaStream_t s, LaunchShape* sh) {
+  return rs == RS_EXACT ? sweep_dispatch<float, 3>(a, nsx, rs, s, sh)
+                        : march3_dispatch(a, nsx, rs, s, sh);
 }
 
 template <typename T>
@@ -441,33 +451,31 @@ static int launch_step_t(hydro_ctx* h, double dt_host, double cfl, double t_end,
   }
   SweepArgs<T> a = sweep_args<T>(h, dt_host, cfl, t_end, ctrl);
   cudaError_t e;
-  int* tx = &h->tile_x;
-  int* ty = &h->tile_y;
-  int* nt = &h->threads;
+  LaunchShape* const sh = &h->shape;
   const int dual = h->eps_dual > 0.0;
   if (h->eos_rad) {
     switch (h->dim) {
-      case 1: e = sweep_dispatch_rad<T, 1>(a, h->nsx, h->riemann, dual, h->stream, tx, ty, nt); break;
-      case 2: e = sweep_dispatch_rad<T, 2>(a, h->nsx, h->riemann, dual, h->stream, tx, ty, nt); break;
-      default: e = sweep_dispatch_rad<T, 3>(a, h->nsx, h->riemann, dual, h->stream, tx, ty, nt); break;
+      case 1: e = sweep_dispatch_rad<T, 1>(a, h->nsx, h->riemann, dual, h->stream, sh); break;
+      case 2: e = sweep_dispatch_rad<T, 2>(a, h->nsx, h->riemann, dual, h->stream, sh); break;
+      default: e = sweep_dispatch_rad<T, 3>(a, h->nsx, h->riemann, dual, h->stream, sh); break;
     }
   } else if (h->xaxis >= 0 || h->maxis >= 0) {
     switch (h->dim) {
-      case 1: e = sweep_dispatch_xm<T, 1>(a, h->nsx, h->riemann, h->stream, tx, ty, nt); break;
-      case 2: e = sweep_dispatch_xm<T, 2>(a, h->nsx, h->riemann, h->stream, tx, ty, nt); break;
-      default: e = sweep_dispatch_xm<T, 3>(a, h->nsx, h->riemann, h->stream, tx, ty, nt); break;
+      case 1: e = sweep_dispatch_xm<T, 1>(a, h->nsx, h->riemann, h->stream, sh); break;
+      case 2: e = sweep_dispatch_xm<T, 2>(a, h->nsx, h->riemann, h->stream, sh); break;
+      default: e = sweep_dispatch_xm<T, 3>(a, h->nsx, h->riemann, h->stream, sh); break;
     }
   } else if (dual) {
     switch (h->dim) {
-      case 1: e = sweep_dispatch_dual<T, 1>(a, h->nsx, h->riemann, h->stream, tx, ty, nt); break;
-      case 2: e = sweep_dispatch_dual<T, 2>(a, h->nsx, h->riemann, h->stream, tx, ty, nt); break;
-      default: e = sweep_dispatch_dual<T, 3>(a, h->nsx, h->riemann, h->stream, tx, ty, nt); break;
+      case 1: e = sweep_dispatch_dual<T, 1>(a, h->nsx, h->riemann, h->stream, sh); break;
+      case 2: e = sweep_dispatch_dual<T, 2>(a, h->nsx, h->riemann, h->stream, sh); break;
+      default: e = sweep_dispatch_dual<T, 3>(a, h->nsx, h->riemann, h->stream, sh); break;
     }
   } else {
     switch (h->dim) {
-      case 1: e = sweep_dispatch<T, 1>(a, h->nsx, h->riemann, h->stream, tx, ty, nt); break;
-      case 2: e = sweep_dispatch<T, 2>(a, h->nsx, h->riemann, h->stream, tx, ty, nt); break;
-      default: e = sweep_dispatch<T, 3>(a, h->nsx, h->riemann, h->stream, tx, ty, nt); break;
+      case 1: e = sweep_dispatch<T, 1>(a, h->nsx, h->riemann, h->stream, sh); break;
+      case 2: e = sweep_dispatch<T, 2>(a, h->nsx, h->riemann, h->stream, sh); break;
+      default: e = step3(a, h->nsx, h->riemann, h->stream, sh); break;
     }
   }
   if (e != cudaSuccess) return cuda_fail(e, "sweep launch");
@@ -548,88 +556,6 @@ std::string device_key() {
   for (auto& ch : name)
     if (ch == ' ') ch = '_';
   return name + "_sm" + std::to_string(p.major) + std::to_string(p.minor);
-}
-
-// Autotuner of the 3D z-chunk: each candidate runs on a scratch control
-// block (so the committed state is untouched; outputs land in the
-// non-current buffer) and is timed with CUDA events.
-static int autotune_grid(hydro_ctx* h, double cfl) {
-  if (h->tuned) return HYDRO_OK;
-  h->tuned = true;
-  if (h->dim < 3) return HYDRO_OK;
-  std::ostringstream key;
-  key << "grid_d" << h->dim << "_p" << h->precision << "_r" << h->riemann << "_ns" << h->ns
-      << (h->eos_rad ? "_rad" : "") << (h->eps_dual > 0.0 ? "_dual" : "") << "_n"
-      << h->n[0] << "x" << h->n[1] << "x" << h->n[2] << "_" << device_key();
-  int cached;
-  double us;
-  if (tune_cache_get(key.str(), &cached, &us)) {
-    h->zchunk = cached;
-    h->tuned_us = us;
-    return HYDRO_OK;
-  }
-  int st = read_ctrl(h);
-  if (st) return st;
-  Ctrl* scratch = nullptr;
-  HCK(cudaMalloc(&scratch, sizeof(Ctrl)));
-  Ctrl base = *h->ctrl_host;
-  base.status = 0;
-  base.done = 0;
-  base.smax_next = 0;
-  cudaEvent_t e0, e1;
-  cudaEventCreate(&e0);
-  cudaEventCreate(&e1);
-  // Powers of two, then (once the first launch has set the tile shape)
-  // chunk lengths that make the CTA count just fill whole waves of the SMs.
-  std::vector<int> cands = {4, 8, 16, 32, 64};
-  double best = 1e300;
-  int best_z = h->zchunk;
-  double dt = base.smax_cur > 0.0 ? cfl / base.smax_cur : 1e-12;
-  int nsm = 0, dev = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  bool waves_added = false;
-  for (size_t ci = 0; ci < cands.size(); ++ci) {
-    if (!waves_added && h->tile_x > 0 && h->tile_y > 0 && nsm > 0) {
-      waves_added = true;
-      const long long plane = (long long)((h->n[0] + h->tile_x - 1) / h->tile_x) *
-                              ((h->n[1] + h->tile_y - 1) / h->tile_y);
-      for (int w = 1; w <= 16; ++w) {
-        const long long nch = (long long)w * nsm / plane;
-        if (nch < 1) continue;
-        const int z = (int)((h->n[2] + nch - 1) / nch);
-        if (z >= 2 && z <= h->n[2] && std::find(cands.begin(), cands.end(), z) == cands.end())
-          cands.push_back(z);
-      }
-    }
-    const int zc = cands[ci];
-    if (zc > h->n[2]) continue;
-    h->zchunk = zc;
-    const int reps = 3;
-    float ms = 0.f;
-    for (int r = 0; r < reps + 1; ++r) {
-      cudaMemcpyAsync(scratch, &base, sizeof(Ctrl), cudaMemcpyHostToDevice, h->stream);
-      if (r == 1) cudaEventRecord(e0, h->stream);
-      if ((st = launch_step(h, dt, cfl, 0.0, scratch))) break;
-    }
-    if (st) break;
-    cudaEventRecord(e1, h->stream);
-    cudaEventSynchronize(e1);
-    cudaEventElapsedTime(&ms, e0, e1);
-    const double t = 1000.0 * ms / reps;
-    if (t < best) {
-      best = t;
-      best_z = zc;
-    }
-  }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  cudaFree(scratch);
-  if (st) return st;
-  h->zchunk = best_z;
-  h->tuned_us = best;
-  tune_cache_put(key.str(), best_z, best);
-  return HYDRO_OK;
 }
 
 template <typename T>
@@ -751,7 +677,6 @@ int hydro_create(const hydro_grid* grid, int coords, const hydro_eos* eos, int r
     if (d < h->dim) h->faces[d].assign(grid->faces[d], grid->faces[d] + grid->n[d] + 1);
   }
   h->ncell = (long long)h->n[0] * h->n[1] * h->n[2];
-  h->zchunk = std::min(32, h->n[2]);
   h->faces_per_step = (long long)(h->n[0] + 1) * h->n[1] * h->n[2];
   if (h->dim >= 2) h->faces_per_step += (long long)h->n[0] * (h->n[1] + 1) * h->n[2];
   if (h->dim == 3) h->faces_per_step += (long long)h->n[0] * h->n[1] * (h->n[2] + 1);
@@ -779,7 +704,6 @@ int hydro_set_dual_energy(hydro_t h, double eps) {
     set_error("hydro_set_dual_energy: not built with the moving grid or the slabs");
     return HYDRO_ERR_UNSUPPORTED;
   }
-  if ((eps > 0.0) != (h->eps_dual > 0.0)) h->tuned = false;  // another kernel: tune again
   h->eps_dual = eps;
   if (h->graph) {
     cudaGraphExecDestroy(h->graph);
@@ -803,7 +727,6 @@ int hydro_set_eos_radiation(hydro_t h, double R_gas, double a_rad) {
   h->eos_rad = 1;
   h->R_gas = R_gas;
   h->a_rad = a_rad;
-  h->tuned = false;
   if (h->graph) {
     cudaGraphExecDestroy(h->graph);
     h->graph = nullptr;
@@ -1121,7 +1044,6 @@ int hydro_run(hydro_t h, int nsteps, double cfl, double t_end, double* t_out) {
     return HYDRO_OK;
   }
   int st;
-  if ((st = autotune_grid(h, cfl))) return st;
   if (!h->graph || h->graph_cfl != cfl || h->graph_tend != t_end) {
     if (h->graph) {
       cudaGraphExecDestroy(h->graph);
@@ -1157,8 +1079,8 @@ int hydro_set_step_totals(hydro_t h, int on) {
   }
   if (on && !h->step_tot_part) {
     // partials for the most CTAs any launch shape gives (tiles of at least
-    // 16 x 8 cells, z chunks of at least one plane)
-    const long long ctas = (long long)((h->n[0] + 15) / 16) * ((h->n[1] + 7) / 8) * h->n[2];
+    // 16 x 6 cells, z chunks of at least one plane)
+    const long long ctas = (long long)((h->n[0] + 15) / 16) * ((h->n[1] + 5) / 6) * h->n[2];
     int st = h->arena.alloc((void**)&h->step_tot_part, sizeof(double) * h->nv * ctas);
     if (st) return st;
   }
@@ -1175,10 +1097,7 @@ int hydro_step_totals(hydro_t h, double* out_nv) {
   if (!h || h->batched || !out_nv) return arg_error("hydro_step_totals: bad argument");
   if (!h->step_tot || !h->step_tot_ok)
     return arg_error("hydro_step_totals: no step with totals since they were turned on or the state was set");
-  const long long ctas = (long long)((h->n[0] + h->tile_x - 1) / h->tile_x) *
-                         (h->dim >= 2 ? (h->n[1] + h->tile_y - 1) / h->tile_y : 1) *
-                         (h->dim == 3 ? (h->n[2] + h->zchunk - 1) / h->zchunk : 1);
-  totals_final_kernel<<<1, 32, 0, h->stream>>>(h->step_tot_part, (int)ctas, h->nv, h->tot_out);
+  totals_final_kernel<<<1, 32, 0, h->stream>>>(h->step_tot_part, (int)h->shape.ctas, h->nv, h->tot_out);
   HCK(cudaGetLastError());
   HCK(cudaMemcpyAsync(out_nv, h->tot_out, sizeof(double) * h->nv, cudaMemcpyDeviceToHost, h->stream));
   HCK(cudaStreamSynchronize(h->stream));
@@ -1220,11 +1139,10 @@ int hydro_stats(hydro_t h, hydro_stats_t* out) {
   out->mlp_faces = (long long)h->ctrl_host->mlp;
   out->t = h->ctrl_host->t;
   out->last_dt = h->ctrl_host->last_dt;
-  out->tile_x = h->tile_x;
-  out->tile_y = h->tile_y;
-  out->zchunk = h->zchunk;
-  out->threads = h->threads;
-  out->tuned_us_per_step = h->tuned_us;
+  out->tile_x = h->shape.tx;
+  out->tile_y = h->shape.ty;
+  out->zchunk = h->shape.zchunk;
+  out->threads = h->shape.threads;
   return HYDRO_OK;
 }
 

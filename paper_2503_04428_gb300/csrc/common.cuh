@@ -6,6 +6,7 @@
 #include <mutex>
 #include <map>
 #include <set>
+#include <tuple>
 #include <utility>
 
 #include "physics.cuh"
@@ -88,7 +89,7 @@ struct SweepArgs {
   double dt_host;         // > 0: use this dt; otherwise CFL on the device
   double cfl;
   double t_end;           // > 0: clip dt so t does not pass t_end
-  int zchunk;             // planes per CTA along axis 2 (3D)
+  int zchunk;             // planes per CTA along axis 2 (3D general sweep)
   Ctrl* ctrl;
   Geom<T> geo;
   // domain decomposition: the axis whose sides may be BC_EXCHANGED (-1 none)
@@ -114,21 +115,69 @@ struct SweepArgs {
   const float2* dvz32;    // dvol[2][k] as an FP32 pair (hi, lo) with hi + lo = dvol[2][k] to ~2^-48
 };
 
+// The shape a step was launched with.
+struct LaunchShape {
+  int tx = 0, ty = 0;    // owned cells of a CTA's tile
+  int zchunk = 0;        // planes of axis 2 per CTA (persistent CTAs: their share, rounded up)
+  int threads = 0;
+  long long ctas = 0;
+};
+
+// Planes per CTA of a march along axis 2 over `tiles` columns of n2 planes
+// with room for `slots` CTAs at a time: the length (at most zmax) whose
+// makespan is least, a CTA that takes z planes `per` at a time costing z/per
+// steps (rounded up) plus `extra` for its partial planes and its start.
+// Measured: FP64 Sedov 128^3 (64 tiles, 152 slots, per 1, extra 1.5) 2.98 ms
+// at 56 planes (128 CTAs of 56 and 64 of 16 on the free slots: 57.5), 3.13 at
+// 19 = 3 waves of 20.5, 3.28 at 8 = 7 of 9.5, 3.39 at 64 = 1 of 65.5, 3.53 at
+// 16 = 4 of 17.5.  A rule rather than a timed trial, so that
+// equal handles take equal chunks and the sums of the totals, grouped by CTA,
+// are the same bits.
+inline int plan_zchunk(long long tiles, int n2, long long slots, int per, double extra, int zmax) {
+  struct Plan {
+    long long tiles = 0, slots = 0;
+    int n2 = 0, per = 0, zmax = 0, z = 0;
+  };
+  static thread_local Plan last;
+  if (last.tiles == tiles && last.n2 == n2 && last.slots == slots && last.per == per && last.zmax == zmax) return last.z;
+  double least = 1e300;
+  const int top = n2 < zmax ? n2 : zmax, stride = (top + 255) / 256;
+  int best = top;
+  for (int z = top; z >= 1; z -= stride) {
+    const int chunks = (n2 + z - 1) / z, rest = n2 - (chunks - 1) * z;
+    const double full = (z + per - 1) / per + extra, part = (rest + per - 1) / per + extra;
+    // the full chunks run in waves; the last, shorter ones fill the slots that come free
+    const long long nfull = tiles * (chunks - 1), waves = nfull / slots, busy = nfull % slots;
+    double end = (waves + (busy ? 1 : 0)) * full;
+    long long left = tiles;
+    for (double t = waves * full; left > 0; t += part) {
+      left -= slots - busy;
+      if (t >= (waves + 1) * full - 1e-9) left -= busy;
+      end = t + part > end ? t + part : end;
+    }
+    if (end < least * 0.999) {
+      least = end;
+      best = z;
+    }
+  }
+  last = {tiles, slots, n2, per, zmax, best};
+  return best;
+}
+
 template <typename T, int DIM>
-cudaError_t sweep_dispatch(const SweepArgs<T>& a, int nsx, int rs, cudaStream_t s, int* tx, int* ty,
-                           int* nt);
+cudaError_t sweep_dispatch(const SweepArgs<T>& a, int nsx, int rs, cudaStream_t s, LaunchShape* sh);
+// The FP32 3D step of the plain ideal gas with HLL or HLLC (march3.cuh).
+cudaError_t march3_dispatch(const SweepArgs<float>& a, int nsx, int rs, cudaStream_t s, LaunchShape* sh);
 // The same with the dual-energy correction (Sect. 2.5).
 template <typename T, int DIM>
-cudaError_t sweep_dispatch_dual(const SweepArgs<T>& a, int nsx, int rs, cudaStream_t s, int* tx, int* ty,
-                                int* nt);
+cudaError_t sweep_dispatch_dual(const SweepArgs<T>& a, int nsx, int rs, cudaStream_t s, LaunchShape* sh);
 // A slab of a decomposed grid or a moving grid (ideal gas, no dual energy).
 template <typename T, int DIM>
-cudaError_t sweep_dispatch_xm(const SweepArgs<T>& a, int nsx, int rs, cudaStream_t s, int* tx, int* ty,
-                              int* nt);
+cudaError_t sweep_dispatch_xm(const SweepArgs<T>& a, int nsx, int rs, cudaStream_t s, LaunchShape* sh);
 // The gas + radiation EoS (HLL and HLLC only), with or without dual energy.
 template <typename T, int DIM>
-cudaError_t sweep_dispatch_rad(const SweepArgs<T>& a, int nsx, int rs, int dual, cudaStream_t s, int* tx,
-                               int* ty, int* nt);
+cudaError_t sweep_dispatch_rad(const SweepArgs<T>& a, int nsx, int rs, int dual, cudaStream_t s,
+                               LaunchShape* sh);
 
 // Raise the dynamic shared-memory limit of kernel `fn` to at least `bytes`
 // on the current device.  The attribute is a property of the kernel on one
@@ -147,6 +196,26 @@ inline cudaError_t smem_attr_once(const void* fn, int bytes) {
   e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e == cudaSuccess) done[{dev, fn}] = bytes;
   return e;
+}
+
+// CTAs of kernel `fn` that the current device holds at a time, looked up once
+// per (device, kernel, shared memory).
+inline cudaError_t kernel_slots(const void* fn, int threads, size_t smem, long long* slots) {
+  static std::mutex mu;
+  static std::map<std::tuple<int, const void*, size_t>, long long> known;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lock(mu);
+  auto it = known.find({dev, fn, smem});
+  if (it == known.end()) {
+    int sms = 0, occ = 0;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, smem)) != cudaSuccess) return e;
+    it = known.insert({{dev, fn, smem}, (long long)sms * (occ > 0 ? occ : 1)}).first;
+  }
+  *slots = it->second;
+  return cudaSuccess;
 }
 
 // Bits of a non-negative double, for an ordered atomicMax.

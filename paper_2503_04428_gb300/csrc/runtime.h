@@ -83,11 +83,7 @@ struct hydro_ctx {
   // per-CTA partials [nv][ctas]
   bool step_tot = false, step_tot_ok = false;
   double* step_tot_part = nullptr;
-  // launch shape
-  int zchunk = 32;
-  int tile_x = 0, tile_y = 0, threads = 0;
-  double tuned_us = 0.0;
-  bool tuned = false;
+  hydro::LaunchShape shape;  // of the last step launched
   // domain decomposition (Sect. 3.3.1): exchanged sides of axis xaxis, the
   // two face coordinates beyond each (nearest first), their halo buffers
   // [nv][2][cross section] on the device, and the monopole's inner mass

@@ -137,6 +137,33 @@ __device__ __forceinline__ int map_axis(int g, int n, int lo, int hi, bool& flip
   return g;
 }
 
+// sum += x z for z given as the pair z.x + z.y, the sum kept as a compensated
+// pair.  (The _rn intrinsics keep the compiler from fusing these operations.)
+__device__ __forceinline__ void add_column_sum(float2& sum, float x, float2 z) {
+  const float p = __fmul_rn(x, z.x);
+  const float e = fmaf(x, z.y, fmaf(x, z.x, -p));
+  const float t = __fadd_rn(sum.x, p);
+  const float bb = __fsub_rn(t, sum.x);
+  const float r = __fadd_rn(__fsub_rn(sum.x, __fsub_rn(t, bb)), __fsub_rn(p, bb));
+  const float lo = __fadd_rn(sum.y, __fadd_rn(r, e));
+  sum.x = __fadd_rn(t, lo);
+  sum.y = __fsub_rn(lo, __fsub_rn(sum.x, t));
+}
+
+// The CTA's totals of its NI owners' sums [v][owner], by a tree in a fixed
+// order per variable (so the result does not depend on scheduling), left in
+// sums[v][0].
+template <int NV, int NI, int NT>
+__device__ void reduce_totals(double* sums) {
+  for (int w = pow2_ceil(NI) / 2; w > 0; w >>= 1) {
+    for (int q = threadIdx.x; q < NV * w; q += NT) {
+      const int v = q / w, o = q - v * w;
+      if (o + w < NI) sums[v * NI + o] += sums[v * NI + o + w];
+    }
+    __syncthreads();
+  }
+}
+
 // Which face states a predictor pass writes.
 enum { PRED_ALL = 0, PRED_ZHI = 1, PRED_ZLO = 2 };
 
@@ -909,25 +936,12 @@ struct Sweep {
         // pair hi + lo.  Each product is split exactly by an FMA, the sum
         // kept as an unevaluated pair (TwoSum, then renormalised), so each
         // term costs ~2^-48 of the sum; the column's sum is multiplied by
-        // dvol[0] dvol[1] in FP64 at the end of the CTA.  (The _rn
-        // intrinsics keep the compiler from fusing these operations.)
+        // dvol[0] dvol[1] in FP64 at the end of the CTA.
         const float2 z = a.dvz32[gz];
         float2* ts = reinterpret_cast<float2*>(tsum);
 #pragma unroll
         for (int v = 0; v < NV; ++v)
-          if (v < nvact) {
-            const float x = Un[v];
-            const float p = __fmul_rn(x, z.x);
-            const float e = fmaf(x, z.y, fmaf(x, z.x, -p));
-            float2 sv = ts[v * NI + o];
-            const float t = __fadd_rn(sv.x, p);
-            const float bb = __fsub_rn(t, sv.x);
-            const float r = __fadd_rn(__fsub_rn(sv.x, __fsub_rn(t, bb)), __fsub_rn(p, bb));
-            const float lo = __fadd_rn(sv.y, __fadd_rn(r, e));
-            sv.x = __fadd_rn(t, lo);
-            sv.y = __fsub_rn(lo, __fsub_rn(sv.x, t));
-            ts[v * NI + o] = sv;
-          }
+          if (v < nvact) add_column_sum(ts[v * NI + o], (float)Un[v], z);
       } else {
         // FP64 sums of U dV
         double dV = a.dvol[0][gi];
@@ -1081,9 +1095,20 @@ __device__ __forceinline__ double step_dt(const volatile Ctrl* vc, double dt_hos
   return dt;
 }
 
+// CTAs per SM that an instantiation's registers are sized for.  The FP32 3D
+// forms of the radiation EoS and the exact solver wait on their Newton chains:
+// two CTAs of 96 registers instead of one of 130-144 (wedge with radiation
+// 512 x 96^2 8.22 -> 5.6 ms per 5 steps, exact 101 x 67 x 53 2.15 -> 1.49 ms
+// per 10 steps, both with the chunks of plan_zchunk).
+template <typename T, int DIM, int NSX, int RS, int MODE>
+__host__ __device__ constexpr int sweep_ctas() {
+  if (RS == RS_EXACT || (MODE & 1)) return DIM == 3 && sizeof(T) == 4 ? 2 : 1;
+  return SweepShape<T, DIM, NSX>::MB;
+}
+
 template <typename T, int DIM, int NSX, int RS, int MODE>
 __global__ void __launch_bounds__(SweepShape<T, DIM, NSX>::NT,
-                                  (RS == RS_EXACT || (MODE & 1)) ? 1 : SweepShape<T, DIM, NSX>::MB)
+                                  sweep_ctas<T, DIM, NSX, RS, MODE>())
     sweep_kernel(const SweepArgs<T> args) {
   using S = SweepShape<T, DIM, NSX>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1167,16 +1192,7 @@ __global__ void __launch_bounds__(SweepShape<T, DIM, NSX>::NT,
       }
       __syncthreads();
     }
-    // the CTA's totals: the owners' sums by a tree in a fixed order, per
-    // variable, so the result does not depend on scheduling
-    constexpr int P2 = pow2_ceil(S::NI);
-    for (int w = P2 / 2; w > 0; w >>= 1) {
-      for (int q = threadIdx.x; q < S::NV * w; q += S::NT) {
-        const int v = q / w, o = q - v * w;
-        if (o + w < S::NI) sw.tsum[v * S::NI + o] += sw.tsum[v * S::NI + o + w];
-      }
-      __syncthreads();
-    }
+    reduce_totals<S::NV, S::NI, S::NT>(sw.tsum);
     const long long ncta = (long long)gridDim.x * gridDim.y * gridDim.z;
     const long long cta = blockIdx.x + gridDim.x * ((long long)blockIdx.y + (long long)gridDim.y * blockIdx.z);
     if (threadIdx.x < S::NV) args.tot_part[threadIdx.x * ncta + cta] = sw.tsum[threadIdx.x * S::NI];
@@ -1185,45 +1201,62 @@ __global__ void __launch_bounds__(SweepShape<T, DIM, NSX>::NT,
                      (MODE & 1) ? (unsigned long long)sw.t_iters : sw.n_iters, s_dt);
 }
 
-template <typename T, int DIM, int NSX, int RS, int MODE>
-cudaError_t launch_sweep(const SweepArgs<T>& a, cudaStream_t s) {
+// Launch one instantiation and report the launch's shape.
+template <typename T, int DIM, int NSX, int RS, int MODE = 0>
+cudaError_t launch_sweep(const SweepArgs<T>& args, cudaStream_t s, LaunchShape* sh) {
   using S = SweepShape<T, DIM, NSX>;
+  SweepArgs<T> a = args;
+  const void* fn = (const void*)sweep_kernel<T, DIM, NSX, RS, MODE>;
   const size_t smem = a.tot_part ? S::tot_offset(MODE) + S::tot_bytes : S::smem_bytes_for(MODE);
-  cudaError_t e = smem_attr_once((const void*)sweep_kernel<T, DIM, NSX, RS, MODE>, (int)smem);
+  cudaError_t e = smem_attr_once(fn, (int)smem);
   if (e != cudaSuccess) return e;
-  dim3 grid((a.n[0] + S::TX - 1) / S::TX, DIM >= 2 ? (a.n[1] + S::TY - 1) / S::TY : 1,
-            DIM == 3 ? (a.n[2] + a.zchunk - 1) / a.zchunk : 1);
+  dim3 grid((a.n[0] + S::TX - 1) / S::TX, DIM >= 2 ? (a.n[1] + S::TY - 1) / S::TY : 1, 1);
+  a.zchunk = 1;
+  if (DIM == 3) {
+    // (planned for the launch without totals, so that both take the same chunks)
+    long long slots;
+    if ((e = kernel_slots(fn, S::NT, S::smem_bytes_for(MODE), &slots)) != cudaSuccess) return e;
+    a.zchunk = plan_zchunk((long long)grid.x * grid.y, a.n[2], slots, 1, 1.5, a.n[2]);
+    grid.z = (a.n[2] + a.zchunk - 1) / a.zchunk;
+  }
+  sh->tx = S::TX;
+  sh->ty = S::TY;
+  sh->zchunk = a.zchunk;
+  sh->threads = S::NT;
+  sh->ctas = (long long)grid.x * grid.y * grid.z;
   sweep_kernel<T, DIM, NSX, RS, MODE><<<grid, S::NT, smem, s>>>(a);
   return cudaGetLastError();
-}
-
-// Launch one instantiation and report its tile shape and threads per CTA.
-template <typename T, int DIM, int NSX, int RS, int MODE = 0>
-cudaError_t launch_sweep_shape(const SweepArgs<T>& a, cudaStream_t s, int* tx, int* ty, int* nt) {
-  using S = SweepShape<T, DIM, NSX>;
-  *tx = S::TX;
-  *ty = S::TY;
-  *nt = S::NT;
-  return launch_sweep<T, DIM, NSX, RS, MODE>(a, s);
 }
 
 // Instantiate the dispatcher of one (precision, dimension) pair and MODE
 // (ideal gas: 0, ideal gas + dual energy: 2).
 #define HYDRO_SWEEP_DISPATCH_MODE(NAME, T, DIM, MODE)                                         \
   template <>                                                                                 \
-  cudaError_t NAME<T, DIM>(const SweepArgs<T>& a, int nsx, int rs, cudaStream_t s, int* tx,   \
-                           int* ty, int* nt) {                                                \
+  cudaError_t NAME<T, DIM>(const SweepArgs<T>& a, int nsx, int rs, cudaStream_t s,            \
+                           LaunchShape* sh) {                                                 \
     switch (nsx * 4 + rs) {                                                                   \
-      case 0: return launch_sweep_shape<T, DIM, 0, RS_HLL, MODE>(a, s, tx, ty, nt);           \
-      case 1: return launch_sweep_shape<T, DIM, 0, RS_HLLC, MODE>(a, s, tx, ty, nt);          \
-      case 2: return launch_sweep_shape<T, DIM, 0, RS_EXACT, MODE>(a, s, tx, ty, nt);         \
-      case 4: return launch_sweep_shape<T, DIM, 1, RS_HLL, MODE>(a, s, tx, ty, nt);           \
-      case 5: return launch_sweep_shape<T, DIM, 1, RS_HLLC, MODE>(a, s, tx, ty, nt);          \
-      case 6: return launch_sweep_shape<T, DIM, 1, RS_EXACT, MODE>(a, s, tx, ty, nt);         \
-      case 12: return launch_sweep_shape<T, DIM, 3, RS_HLL, MODE>(a, s, tx, ty, nt);          \
-      case 13: return launch_sweep_shape<T, DIM, 3, RS_HLLC, MODE>(a, s, tx, ty, nt);         \
-      case 14: return launch_sweep_shape<T, DIM, 3, RS_EXACT, MODE>(a, s, tx, ty, nt);        \
+      case 0: return launch_sweep<T, DIM, 0, RS_HLL, MODE>(a, s, sh);                  \
+      case 1: return launch_sweep<T, DIM, 0, RS_HLLC, MODE>(a, s, sh);                 \
+      case 2: return launch_sweep<T, DIM, 0, RS_EXACT, MODE>(a, s, sh);                \
+      case 4: return launch_sweep<T, DIM, 1, RS_HLL, MODE>(a, s, sh);                  \
+      case 5: return launch_sweep<T, DIM, 1, RS_HLLC, MODE>(a, s, sh);                 \
+      case 6: return launch_sweep<T, DIM, 1, RS_EXACT, MODE>(a, s, sh);                \
+      case 12: return launch_sweep<T, DIM, 3, RS_HLL, MODE>(a, s, sh);                 \
+      case 13: return launch_sweep<T, DIM, 3, RS_HLLC, MODE>(a, s, sh);                \
+      case 14: return launch_sweep<T, DIM, 3, RS_EXACT, MODE>(a, s, sh);               \
       default: return cudaErrorInvalidValue;                                                  \
+    }                                                                                         \
+  }
+// The exact solver alone (the FP32 3D form, whose HLL and HLLC steps march).
+#define HYDRO_SWEEP_DISPATCH_EXACT(T, DIM)                                                    \
+  template <>                                                                                 \
+  cudaError_t sweep_dispatch<T, DIM>(const SweepArgs<T>& a, int nsx, int rs, cudaStream_t s,  \
+                                     LaunchShape* sh) {                                       \
+    if (rs != RS_EXACT) return cudaErrorInvalidValue;                                         \
+    switch (nsx) {                                                                            \
+      case 0: return launch_sweep<T, DIM, 0, RS_EXACT, 0>(a, s, sh);                   \
+      case 1: return launch_sweep<T, DIM, 1, RS_EXACT, 0>(a, s, sh);                   \
+      default: return launch_sweep<T, DIM, 3, RS_EXACT, 0>(a, s, sh);                  \
     }                                                                                         \
   }
 #define HYDRO_SWEEP_DISPATCH(T, DIM) HYDRO_SWEEP_DISPATCH_MODE(sweep_dispatch, T, DIM, 0)
@@ -1235,20 +1268,20 @@ cudaError_t launch_sweep_shape(const SweepArgs<T>& a, cudaStream_t s, int* tx, i
 #define HYDRO_SWEEP_DISPATCH_RAD(T, DIM)                                                      \
   template <>                                                                                 \
   cudaError_t sweep_dispatch_rad<T, DIM>(const SweepArgs<T>& a, int nsx, int rs, int dual,    \
-                                         cudaStream_t s, int* tx, int* ty, int* nt) {         \
+                                         cudaStream_t s, LaunchShape* sh) {                   \
     switch ((nsx * 4 + rs) * 2 + (dual ? 1 : 0)) {                                            \
-      case 0: return launch_sweep_shape<T, DIM, 0, RS_HLL, 1>(a, s, tx, ty, nt);              \
-      case 1: return launch_sweep_shape<T, DIM, 0, RS_HLL, 3>(a, s, tx, ty, nt);              \
-      case 2: return launch_sweep_shape<T, DIM, 0, RS_HLLC, 1>(a, s, tx, ty, nt);             \
-      case 3: return launch_sweep_shape<T, DIM, 0, RS_HLLC, 3>(a, s, tx, ty, nt);             \
-      case 8: return launch_sweep_shape<T, DIM, 1, RS_HLL, 1>(a, s, tx, ty, nt);              \
-      case 9: return launch_sweep_shape<T, DIM, 1, RS_HLL, 3>(a, s, tx, ty, nt);              \
-      case 10: return launch_sweep_shape<T, DIM, 1, RS_HLLC, 1>(a, s, tx, ty, nt);            \
-      case 11: return launch_sweep_shape<T, DIM, 1, RS_HLLC, 3>(a, s, tx, ty, nt);            \
-      case 24: return launch_sweep_shape<T, DIM, 3, RS_HLL, 1>(a, s, tx, ty, nt);             \
-      case 25: return launch_sweep_shape<T, DIM, 3, RS_HLL, 3>(a, s, tx, ty, nt);             \
-      case 26: return launch_sweep_shape<T, DIM, 3, RS_HLLC, 1>(a, s, tx, ty, nt);            \
-      case 27: return launch_sweep_shape<T, DIM, 3, RS_HLLC, 3>(a, s, tx, ty, nt);            \
+      case 0: return launch_sweep<T, DIM, 0, RS_HLL, 1>(a, s, sh);                     \
+      case 1: return launch_sweep<T, DIM, 0, RS_HLL, 3>(a, s, sh);                     \
+      case 2: return launch_sweep<T, DIM, 0, RS_HLLC, 1>(a, s, sh);                    \
+      case 3: return launch_sweep<T, DIM, 0, RS_HLLC, 3>(a, s, sh);                    \
+      case 8: return launch_sweep<T, DIM, 1, RS_HLL, 1>(a, s, sh);                     \
+      case 9: return launch_sweep<T, DIM, 1, RS_HLL, 3>(a, s, sh);                     \
+      case 10: return launch_sweep<T, DIM, 1, RS_HLLC, 1>(a, s, sh);                   \
+      case 11: return launch_sweep<T, DIM, 1, RS_HLLC, 3>(a, s, sh);                   \
+      case 24: return launch_sweep<T, DIM, 3, RS_HLL, 1>(a, s, sh);                    \
+      case 25: return launch_sweep<T, DIM, 3, RS_HLL, 3>(a, s, sh);                    \
+      case 26: return launch_sweep<T, DIM, 3, RS_HLLC, 1>(a, s, sh);                   \
+      case 27: return launch_sweep<T, DIM, 3, RS_HLLC, 3>(a, s, sh);                   \
       default: return cudaErrorInvalidValue;                                                  \
     }                                                                                         \
   }
