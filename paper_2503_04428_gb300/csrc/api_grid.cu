@@ -258,16 +258,17 @@ static int build_geometry(hydro_ctx* h) {
   if ((st = upload_d(h, a, &h->dvol[0]))) return st;
   if ((st = upload_d(h, b, &h->dvol[1]))) return st;
   if ((st = upload_d(h, c, &h->dvol[2]))) return st;
-  {
-    // the axis-2 factors split into FP32 pairs for the FP32 form's
-    // compensated in-step totals
-    std::vector<float> hl(2 * c.size());
-    for (size_t k = 0; k < c.size(); ++k) {
-      hl[2 * k] = (float)c[k];
-      hl[2 * k + 1] = (float)(c[k] - (double)hl[2 * k]);
+  for (int d = 1; d < 3; ++d) {
+    // the axis-1 and axis-2 factors split into FP32 pairs for the FP32
+    // form's compensated in-step totals
+    const std::vector<double>& f = d == 1 ? b : c;
+    std::vector<float> hl(2 * f.size());
+    for (size_t k = 0; k < f.size(); ++k) {
+      hl[2 * k] = (float)f[k];
+      hl[2 * k + 1] = (float)(f[k] - (double)hl[2 * k]);
     }
-    if (!h->dvz32 && (st = h->arena.alloc((void**)&h->dvz32, hl.size() * sizeof(float)))) return st;
-    HCK(cudaMemcpy(h->dvz32, hl.data(), hl.size() * sizeof(float), cudaMemcpyHostToDevice));
+    if (!h->dv32[d] && (st = h->arena.alloc((void**)&h->dv32[d], hl.size() * sizeof(float)))) return st;
+    HCK(cudaMemcpy(h->dv32[d], hl.data(), hl.size() * sizeof(float), cudaMemcpyHostToDevice));
   }
   if ((st = upload_d(h, rc, &h->rc_d))) return st;
   double bsum = 0.0, csum = 0.0;
@@ -420,18 +421,21 @@ static SweepArgs<T> sweep_args(hydro_ctx* h, double dt_host, double cfl, double 
   a.ir_new = mv_sph && h->dim >= 2 ? (const T*)h->irn_d : nullptr;
   a.tot_part = h->step_tot ? h->step_tot_part : nullptr;
   for (int d = 0; d < 3; ++d) a.dvol[d] = h->dvol[d];
-  a.dvz32 = reinterpret_cast<const float2*>(h->dvz32);
+  for (int d = 0; d < 3; ++d) a.dv32[d] = reinterpret_cast<const float2*>(h->dv32[d]);
   return a;
 }
 
-// The plain 3D step: FP32 with HLL or HLLC marches (march3.cuh); FP64, which
-// is bound by the FP64 pipe, and the exact solver take the general sweep.
-static cudaError_t step3(const SweepArgs<double>& a, int nsx, int rs, cudaStream_t s, LaunchShape* sh) {
-  return sweep_dispatch<double, 3>(a, nsx, rs, s, sh);
+// The plain 2D and 3D steps: FP32 with HLL or HLLC marches (march2.cuh,
+// march3.cuh); FP64, which is bound by the FP64 pipe, and the exact solver
+// take the general sweep.
+template <int DIM>
+static cudaError_t plain_step(const SweepArgs<double>& a, int nsx, int rs, cudaStream_t s, LaunchShape* sh) {
+  return sweep_dispatch<double, DIM>(a, nsx, rs, s, sh);
 }
-static cudaError_t step3(const SweepArgs<float>& a, int nsx, int rs, cudaStream_t s, LaunchShape* sh) {
-  return rs == RS_EXACT ? sweep_dispatch<float, 3>(a, nsx, rs, s, sh)
-                        : march3_dispatch(a, nsx, rs, s, sh);
+template <int DIM>
+static cudaError_t plain_step(const SweepArgs<float>& a, int nsx, int rs, cudaStream_t s, LaunchShape* sh) {
+  if (rs == RS_EXACT) return sweep_dispatch<float, DIM>(a, nsx, rs, s, sh);
+  return DIM == 2 ? march2_dispatch(a, nsx, rs, s, sh) : march3_dispatch(a, nsx, rs, s, sh);
 }
 
 template <typename T>
@@ -474,8 +478,8 @@ static int launch_step_t(hydro_ctx* h, double dt_host, double cfl, double t_end,
   } else {
     switch (h->dim) {
       case 1: e = sweep_dispatch<T, 1>(a, h->nsx, h->riemann, h->stream, sh); break;
-      case 2: e = sweep_dispatch<T, 2>(a, h->nsx, h->riemann, h->stream, sh); break;
-      default: e = step3(a, h->nsx, h->riemann, h->stream, sh); break;
+      case 2: e = plain_step<2>(a, h->nsx, h->riemann, h->stream, sh); break;
+      default: e = plain_step<3>(a, h->nsx, h->riemann, h->stream, sh); break;
     }
   }
   if (e != cudaSuccess) return cuda_fail(e, "sweep launch");
@@ -1078,9 +1082,10 @@ int hydro_set_step_totals(hydro_t h, int on) {
     return HYDRO_ERR_UNSUPPORTED;
   }
   if (on && !h->step_tot_part) {
-    // partials for the most CTAs any launch shape gives (tiles of at least
-    // 16 x 6 cells, z chunks of at least one plane)
-    const long long ctas = (long long)((h->n[0] + 15) / 16) * ((h->n[1] + 5) / 6) * h->n[2];
+    // partials for the most CTAs any launch shape gives: tiles of at least
+    // 16 x 6 cells and one plane, or warps of 28 columns and one row, 4 a CTA
+    const long long ctas = std::max((long long)((h->n[0] + 15) / 16) * ((h->n[1] + 5) / 6) * h->n[2],
+                                    ((long long)((h->n[0] + 27) / 28) * h->n[1] + 3) / 4);
     int st = h->arena.alloc((void**)&h->step_tot_part, sizeof(double) * h->nv * ctas);
     if (st) return st;
   }

@@ -112,7 +112,7 @@ struct SweepArgs {
   // blockIdx.z)); null: not accumulated
   double* tot_part;
   const double* dvol[3];  // dV of cell (i, j, k) = dvol[0][i] dvol[1][j] dvol[2][k] (FP64)
-  const float2* dvz32;    // dvol[2][k] as an FP32 pair (hi, lo) with hi + lo = dvol[2][k] to ~2^-48
+  const float2* dv32[3];  // axes 1 and 2: dvol as FP32 pairs (hi, lo) with hi + lo = dvol to ~2^-48
 };
 
 // The shape a step was launched with.
@@ -168,6 +168,8 @@ template <typename T, int DIM>
 cudaError_t sweep_dispatch(const SweepArgs<T>& a, int nsx, int rs, cudaStream_t s, LaunchShape* sh);
 // The FP32 3D step of the plain ideal gas with HLL or HLLC (march3.cuh).
 cudaError_t march3_dispatch(const SweepArgs<float>& a, int nsx, int rs, cudaStream_t s, LaunchShape* sh);
+// The FP32 2D step of the plain ideal gas with HLL or HLLC (march2.cuh).
+cudaError_t march2_dispatch(const SweepArgs<float>& a, int nsx, int rs, cudaStream_t s, LaunchShape* sh);
 // The same with the dual-energy correction (Sect. 2.5).
 template <typename T, int DIM>
 cudaError_t sweep_dispatch_dual(const SweepArgs<T>& a, int nsx, int rs, cudaStream_t s, LaunchShape* sh);

@@ -30,29 +30,11 @@
 #pragma once
 #include <algorithm>
 
+#include "march.cuh"
 #include "pair.cuh"
 #include "sweep.cuh"
 
 namespace hydro {
-
-__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-// Asynchronous 4-byte copies to shared memory (PTX cp.async), waited for in
-// groups: at most N groups still in flight after copies_wait<N>.
-__device__ __forceinline__ void copy4_async(unsigned dst, const float* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void copies_wait() {
-  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
-
-// The element `bytes` bytes after a (uniform) address.
-template <typename P>
-__device__ __forceinline__ P* at_byte(P* p, unsigned bytes) {
-  using C = std::conditional_t<std::is_const_v<P>, const char, char>;
-  return reinterpret_cast<P*>(reinterpret_cast<C*>(p) + bytes);
-}
 
 // Rows of warps per CTA, one CTA per SM: as many as leave the step its
 // registers without spills (NV = 5: 16 rows of 128 registers 9.75 ms, 12 of
@@ -106,14 +88,7 @@ __global__ void __launch_bounds__(March3Shape<NSX, SPH>::NT, March3Shape<NSX, SP
   const int cur = vc->cur;
   const float* const Uin = cur ? a.B : a.A;
   float* const Uout = cur ? a.Aw : a.B;
-  if (threadIdx.x == 0) {
-    s_dt = vc->status != 0 ? 0.0 : step_dt(vc, a.dt_host, a.cfl, a.t_end);
-    s_hfac = 0.f;
-    if (a.heating == HEAT_NI56) {
-      const double t = vc->t;
-      s_hfac = (float)(a.ni_lambda * (a.ni_a * exp(-t / a.ni_tni) + a.ni_qco * exp(-t / a.ni_tco)));
-    }
-  }
+  if (threadIdx.x == 0) step_start(a, s_dt, s_hfac);
   int tid = threadIdx.x;
   asm volatile("" : "+r"(tid));  // (kept in a register: re-reading the special register costs more)
   const int lane = tid & 31, row = tid >> 5;
@@ -456,37 +431,13 @@ __global__ void __launch_bounds__(March3Shape<NSX, SPH>::NT, March3Shape<NSX, SP
             const bool w0 = lown, w1 = lown && i - 1 < lenb;  // the halves written
             if (w0) {
               copies_wait<1>();  // the own cells' state (all but the plane just fetched)
-              f2 Uo[NV], Un[NV], Wn[NV];
+              f2 Uo[NV], Un[NV];
 #pragma unroll
               for (int v = 0; v < NV; ++v) Uo[v] = own_u[v * NT];
-#pragma unroll
-              for (int v = 0; v < NV; ++v) Un[v] = fma2(dt, acc[v], Uo[v]);
-              if (a.gravity == GRAV_UNIFORM) {
-                f2 work = both(0.f);
-#pragma unroll
-                for (int d = 0; d < 3; ++d) {
-                  const f2 g = both(a.g0[d]);
-                  Un[1 + d] = fma2(dt * Uo[0], g, Un[1 + d]);
-                  work = fma2(Uo[1 + d], g, work);
-                }
-                Un[4] = fma2(dt, work, Un[4]);
-              } else if (a.gravity != GRAV_NONE) {
-                const f2 g = gx[S::GX_G * 33];  // point mass or monopole
-                Un[1] = fma2(dt * Uo[0], g, Un[1]);
-                Un[4] = fma2(dt, Uo[1] * g, Un[4]);
-              }
-              if (a.heating == HEAT_CONST) {
-                Un[4] = fma2(dt, both(a.heat_q), Un[4]);
-              } else if (a.heating == HEAT_NI56) {
-                f2 rf = both(0.f);
-#pragma unroll
-                for (int s = 0; s < NSX; ++s)
-                  if (s == a.ni_index) rf = Uo[5 + s];
-                Un[4] = fma2(dt * both(s_hfac), rf, Un[4]);
-              }
+              new_state2<3, NSX>(a, dt, gx[S::GX_G * 33], s_hfac, Uo, acc, Un);
               if (tsum) {
                 float2* ts = tsum + (row - 1) * TX + lane - 1;
-                const float2 t0 = a.dvz32[z0 + i - 1], t1 = a.dvz32[w1 ? zb + i - 1 : z0 + i - 1];
+                const float2 t0 = a.dv32[2][z0 + i - 1], t1 = a.dv32[2][w1 ? zb + i - 1 : z0 + i - 1];
 #pragma unroll
                 for (int v = 0; v < NV; ++v)
                   if (active(v)) {
@@ -494,36 +445,15 @@ __global__ void __launch_bounds__(March3Shape<NSX, SPH>::NT, March3Shape<NSX, SP
                     if (w1) add_column_sum(ts[v * NI], hi(Un[v]), t1);
                   }
               }
-              to_prim2<3, NSX>(Un, Wn, gas);
-              const f2 cs = sound2(Wn[0], Wn[4], gas);
-              f2 ihy = gy[S::GY_IW * (R + 1)], ihz = gz(S::GZ_IW, i - 1);
+              f2 ih[3] = {gx[S::GX_IW * 33], gy[S::GY_IW * (R + 1)], gz(S::GZ_IW, i - 1)};
               if constexpr (SPH) {
-                ihy = ihy * gx[S::GX_IR * 33];
-                ihz = ihz * (gx[S::GX_IR * 33] * gy[S::GY_IS * (R + 1)]);
+                ih[1] = ih[1] * gx[S::GX_IR * 33];
+                ih[2] = ih[2] * (gx[S::GX_IR * 33] * gy[S::GY_IS * (R + 1)]);
               }
-              auto absolute = [](f2 x) { return make_f2(fabsf(lo(x)), fabsf(hi(x))); };
-              const f2 sp = fma2(absolute(Wn[3]) + cs, ihz,
-                                 fma2(absolute(Wn[2]) + cs, ihy, (absolute(Wn[1]) + cs) * gx[S::GX_IW * 33]));
-              f2 nul = both(0.f);  // 0 unless a value is infinite or NaN
-#pragma unroll
-              for (int v = 0; v < NV; ++v) nul = fma2(Un[v], both(0.f), nul);
               float* const dst = Uout + (z0 + i - 1) * plane;
               store(dst, std::integral_constant<int, 0>(), Un);
-              smax = fmaxf(smax, lo(sp));
-              if (w1) {
-                store(dst + len * plane, std::integral_constant<int, 1>(), Un);
-                smax = fmaxf(smax, hi(sp));
-              }
-              auto check = [&](float n, float rho, float p) {
-                if (!(n == 0.f)) err = err ? err : ST_NONFINITE;
-                else if (!(rho > 0.f) || !(p > 0.f)) err = err ? err : ST_NEG;
-              };
-              const bool bad0 = !(lo(nul) == 0.f && lo(Wn[0]) > 0.f && lo(Wn[4]) > 0.f);
-              const bool bad1 = !(hi(nul) == 0.f && hi(Wn[0]) > 0.f && hi(Wn[4]) > 0.f);
-              if (bad0 || (w1 && bad1)) {
-                if (bad0) check(lo(nul), lo(Wn[0]), lo(Wn[4]));
-                if (w1 && bad1) check(hi(nul), hi(Wn[0]), hi(Wn[4]));
-              }
+              if (w1) store(dst + len * plane, std::integral_constant<int, 1>(), Un);
+              check_state2<3, NSX>(gas, Un, ih, w1, smax, err);
             }
           }
           f2 cz = gz(S::GZ_IC, i);

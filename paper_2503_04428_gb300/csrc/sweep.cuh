@@ -937,7 +937,7 @@ struct Sweep {
         // kept as an unevaluated pair (TwoSum, then renormalised), so each
         // term costs ~2^-48 of the sum; the column's sum is multiplied by
         // dvol[0] dvol[1] in FP64 at the end of the CTA.
-        const float2 z = a.dvz32[gz];
+        const float2 z = a.dv32[2][gz];
         float2* ts = reinterpret_cast<float2*>(tsum);
 #pragma unroll
         for (int v = 0; v < NV; ++v)
@@ -1247,7 +1247,7 @@ cudaError_t launch_sweep(const SweepArgs<T>& args, cudaStream_t s, LaunchShape* 
       default: return cudaErrorInvalidValue;                                                  \
     }                                                                                         \
   }
-// The exact solver alone (the FP32 3D form, whose HLL and HLLC steps march).
+// The exact solver alone (the FP32 2D and 3D forms, whose HLL and HLLC steps march).
 #define HYDRO_SWEEP_DISPATCH_EXACT(T, DIM)                                                    \
   template <>                                                                                 \
   cudaError_t sweep_dispatch<T, DIM>(const SweepArgs<T>& a, int nsx, int rs, cudaStream_t s,  \

@@ -1,6 +1,6 @@
-// Fused sweep kernels: float state, 2D grids (all scalar counts and Riemann solvers).
+// Fused sweep kernels: float state, 2D grids with the exact Riemann solver (all scalar counts).
 #include "sweep.cuh"
 
 namespace hydro {
-HYDRO_SWEEP_DISPATCH(float, 2)
+HYDRO_SWEEP_DISPATCH_EXACT(float, 2)
 }  // namespace hydro

@@ -1,11 +1,12 @@
-"""The FP32 3D marching step (csrc/march3.cuh) at the edges of its tiles, halves and chunks.
+"""The FP32 marching steps (csrc/march3.cuh, march2.cuh) at the edges of their tiles, halves and chunks.
 
 One step of each grid against the oracle, at the per-step bars of
 tests/parity.py: sizes at and around the owned columns of a warp (30) and the
-owned rows of a CTA (14, 10 and 8 for 0, 1 and 2-3 scalars), the smallest
-axes, odd plane counts (the high half of a pair then misses its last plane),
-every boundary kind and both coordinate systems; and many steps of the same
-runs give the same bits.
+owned rows of a CTA (14, 10 and 8 for 0, 1 and 2-3 scalars) in 3D, the owned
+columns of a warp (28) and the longest run of rows (2 x 64) in 2D, the
+smallest axes, odd counts (the high half of a pair then misses its last plane
+or row), every boundary kind and both coordinate systems; and repeated runs
+give the same bits.
 """
 import numpy as np
 import pytest
@@ -39,6 +40,26 @@ def test_spherical_sizes(hydro_lib, n, riemann):
     _one_step(hydro_lib, case)
 
 
+SIZES2 = [(2, 2), (27, 3), (28, 4), (29, 5), (57, 64), (3, 131), (84, 129), (30, 257)]
+
+
+@pytest.mark.parametrize("k", range(len(SIZES2)))
+@pytest.mark.parametrize("ns", [0, 1, 2, 3])
+def test_2d_sizes(hydro_lib, k, ns):
+    case = wl.smooth_random(2, list(SIZES2[k]), ns, seed=60 + k, bc=BCS[(k + ns) % 4][:2],
+                            riemann=[O.HLL, O.HLLC][(k + ns) % 2], limiter=[O.MINMOD, O.VANLEER, O.VANALBADA][k % 3])
+    case["sources"] = dict(gravity=O.GRAV_UNIFORM, g0=(0.1, -0.2, 0.0))
+    _one_step(hydro_lib, case)
+
+
+@pytest.mark.parametrize("n", [(2, 2), (29, 7), (56, 130)])
+@pytest.mark.parametrize("riemann", [O.HLL, O.HLLC])
+def test_2d_spherical_sizes(hydro_lib, n, riemann):
+    case = wl.sphere_state(*n, n_scalars=1, dim=2, riemann=riemann)
+    case["sources"] = dict(gravity=O.GRAV_POINT, G=0.01, Mc=2.0)
+    _one_step(hydro_lib, case)
+
+
 def _one_step(hydro_lib, case):
     case["U"] = case["U"].astype(np.float32).astype(np.float64)
     ref = O.solver_from_case(case)
@@ -49,7 +70,7 @@ def _one_step(hydro_lib, case):
         g = hydro_lib.Grid.from_case(case, 32)
         g.set_step_totals(True)
         g.step(dt)
-        check(ref.get_state(), g.get_state(), 3, case["gamma"], 32)
+        check(ref.get_state(), g.get_state(), case["dim"], case["gamma"], 32)
         g.run(4, 0.4)
         out.append((g.get_state(), g.step_totals()))
         g.close()
