@@ -1083,8 +1083,8 @@ int hydro_set_step_totals(hydro_t h, int on) {
   }
   if (on && !h->step_tot_part) {
     // partials for the most CTAs any launch shape gives: tiles of at least
-    // 16 x 6 cells and one plane, or warps of 28 columns and one row, 4 a CTA
-    const long long ctas = std::max((long long)((h->n[0] + 15) / 16) * ((h->n[1] + 5) / 6) * h->n[2],
+    // 8 x 8 (2D) or 16 x 8 (3D) cells and one plane, or warps of 28 columns and one row, 4 a CTA
+    const long long ctas = std::max((long long)((h->n[0] + 7) / 8) * ((h->n[1] + 7) / 8) * h->n[2],
                                     ((long long)((h->n[0] + 27) / 28) * h->n[1] + 3) / 4);
     int st = h->arena.alloc((void**)&h->step_tot_part, sizeof(double) * h->nv * ctas);
     if (st) return st;

@@ -22,46 +22,34 @@
 // registers until that plane's upper z flux is known.  Each state value is
 // read from HBM once per CTA (halo re-reads hit L2) and written once.
 #pragma once
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace hydro {
 
 // Tile shape per (precision, dimension, scalar slots) and the CTAs per SM
-// the register budget is sized for (MB; the exact solver, whose Newton
-// iteration needs more registers, always gets one CTA's budget).  The CTA has one thread per
-// predictor cell (the tile plus a one-cell halo without corners), rounded up
-// to whole warps.
-template <typename T, int DIM, int NSX>
-struct TileCfg;
-// float
-template <> struct TileCfg<float, 1, 0> { static constexpr int TX = 254, TY = 1, MB = 1; };
-template <> struct TileCfg<float, 1, 1> { static constexpr int TX = 254, TY = 1, MB = 1; };
-template <> struct TileCfg<float, 1, 3> { static constexpr int TX = 254, TY = 1, MB = 1; };
-template <> struct TileCfg<float, 2, 0> { static constexpr int TX = 32, TY = 16, MB = 1; };
-template <> struct TileCfg<float, 2, 1> { static constexpr int TX = 32, TY = 16, MB = 1; };
-template <> struct TileCfg<float, 2, 3> { static constexpr int TX = 32, TY = 8, MB = 1; };
-template <> struct TileCfg<float, 3, 0> { static constexpr int TX = 16, TY = 16, MB = 3; };
-template <> struct TileCfg<float, 3, 1> { static constexpr int TX = 16, TY = 16, MB = 2; };
-template <> struct TileCfg<float, 3, 3> { static constexpr int TX = 16, TY = 16, MB = 2; };
-// double
-template <> struct TileCfg<double, 1, 0> { static constexpr int TX = 254, TY = 1, MB = 1; };
-template <> struct TileCfg<double, 1, 1> { static constexpr int TX = 254, TY = 1, MB = 1; };
-template <> struct TileCfg<double, 1, 3> { static constexpr int TX = 254, TY = 1, MB = 1; };
-template <> struct TileCfg<double, 2, 0> { static constexpr int TX = 32, TY = 8, MB = 1; };
-template <> struct TileCfg<double, 2, 1> { static constexpr int TX = 32, TY = 8, MB = 1; };
-template <> struct TileCfg<double, 2, 3> { static constexpr int TX = 32, TY = 8, MB = 1; };
-template <> struct TileCfg<double, 3, 0> { static constexpr int TX = 16, TY = 16, MB = 1; };
-template <> struct TileCfg<double, 3, 1> { static constexpr int TX = 16, TY = 16, MB = 1; };
-template <> struct TileCfg<double, 3, 3> { static constexpr int TX = 16, TY = 8, MB = 1; };
+// the register budget is sized for (MB; see sweep_ctas).  The CTA has one
+// thread per predictor cell (the tile plus a one-cell halo without corners),
+// rounded up to whole warps.  SMALL: the 1D and 2D tiles of grids whose large
+// tiles would leave SMs idle (see small_tile): 28 cells and their halo fill
+// one warp, 8 x 8 three.
+template <typename T, int DIM, int NSX, bool SMALL>
+struct TileCfg {
+  static constexpr int TX = DIM == 1 ? (SMALL ? 28 : 254) : (SMALL ? 8 : 16);
+  static constexpr int TY = DIM == 1 ? 1 : SMALL ? 8 : (DIM == 3 && NSX == 3 && sizeof(T) == 8) ? 8 : 16;
+  // (FP32 3D without scalars: three CTAs of 64 registers)
+  static constexpr int MB = DIM == 1 || SMALL ? 1 : DIM == 2 ? 2 : sizeof(T) == 8 ? 1 : NSX == 0 ? 3 : 2;
+};
 
 // The smallest power of two >= n (n >= 1).
 __host__ __device__ constexpr int pow2_ceil(int n) { return n <= 1 ? 1 : 2 * pow2_ceil((n + 1) / 2); }
 
-template <typename T, int DIM, int NSX>
+template <typename T, int DIM, int NSX, bool SMALL = false>
 struct SweepShape {
   static constexpr int NV = 2 + DIM + NSX;
-  static constexpr int TX = TileCfg<T, DIM, NSX>::TX;
-  static constexpr int TY = TileCfg<T, DIM, NSX>::TY;
+  static constexpr int TX = TileCfg<T, DIM, NSX, SMALL>::TX;
+  static constexpr int TY = TileCfg<T, DIM, NSX, SMALL>::TY;
   static constexpr int HY = DIM >= 2 ? 2 : 0;              // primitive halo along axis 1
   static constexpr int EX = TX + 4, EY = TY + 2 * HY;      // primitive plane extents
   static constexpr int QY = DIM >= 2 ? 1 : 0;              // predictor halo along axis 1
@@ -70,7 +58,7 @@ struct SweepShape {
   static constexpr int NH = 2 * TY + (DIM >= 2 ? 2 * TX : 0);  // halo predictor cells
   static constexpr int NP = NI + NH;                        // predictor cells
   static constexpr int NT = (NP + 31) / 32 * 32;            // threads per CTA
-  static constexpr int MB = TileCfg<T, DIM, NSX>::MB;       // resident CTAs per SM (register budget)
+  static constexpr int MB = TileCfg<T, DIM, NSX, SMALL>::MB;       // resident CTAs per SM (register budget)
   static constexpr int WPL = EX * EY;
   static constexpr int NFX = (TX + 1) * TY;
   static constexpr int NFY = DIM >= 2 ? TX * (TY + 1) : 0;
@@ -171,14 +159,14 @@ enum { PRED_ALL = 0, PRED_ZHI = 1, PRED_ZLO = 2 };
 // (Sect. 2.5); bit 2: a slab of a decomposed grid or a moving grid (exchanged
 // ghosts, moving faces; ideal gas only).  Each combination is its own
 // instantiation, so the plain step carries none of the optional work.
-template <typename T, int DIM, int NSX, int RS, int MODE>
+template <typename T, int DIM, int NSX, int RS, int MODE, bool SMALL>
 struct Sweep {
   static constexpr int EOS = MODE & 1;
   static constexpr bool DUAL = (MODE & 2) != 0;
   static constexpr bool XM = (MODE & 4) != 0;
   // in-step totals as compensated FP32 column sums (FP32, 3D) instead of FP64 sums per cell
   static constexpr bool COLSUM = sizeof(T) == 4 && DIM == 3;
-  using S = SweepShape<T, DIM, NSX>;
+  using S = SweepShape<T, DIM, NSX, SMALL>;
   static constexpr int NV = S::NV, TX = S::TX, TY = S::TY, EX = S::EX, EY = S::EY, HY = S::HY,
                        QY = S::QY, NT = S::NT, NI = S::NI, NP = S::NP, NFX = S::NFX,
                        NFY = S::NFY, NFZ = S::NFZ;
@@ -331,7 +319,7 @@ struct Sweep {
       else sz = map_axis(gz, a.n[2], a.bc[2][0], a.bc[2][1], fz);
     }
     const int slot = wslot(gz);
-    const int nvact = 2 + DIM + a.ns;
+    const int nvact = NSX < 3 ? NV : 2 + DIM + a.ns;
     // a staged region inside the domain on every axis: no ghost mapping
     const bool inner = !XM && x0 >= 2 && x0 + TX + 2 <= n0 &&
                        (DIM < 2 || (y0 >= HY && y0 + TY + HY <= n1)) && (DIM < 3 || (gz >= 0 && gz < a.n[2]));
@@ -840,7 +828,7 @@ struct Sweep {
   // momentum flux of the upper z face (3D).
   __device__ void close_cell(int gz, int i, int j, int gi, int gj, T fzt3) {
     const int n0 = a.n[0], n1 = a.n[1];
-    const int nvact = 2 + DIM + a.ns;
+    const int nvact = NSX < 3 ? NV : 2 + DIM + a.ns;
     const long long c = ((long long)gz * n1 + gj) * n0 + gi;
     T Uo[NV], Un[NV];
 #pragma unroll
@@ -1100,17 +1088,18 @@ __device__ __forceinline__ double step_dt(const volatile Ctrl* vc, double dt_hos
 // two CTAs of 96 registers instead of one of 130-144 (wedge with radiation
 // 512 x 96^2 8.22 -> 5.6 ms per 5 steps, exact 101 x 67 x 53 2.15 -> 1.49 ms
 // per 10 steps, both with the chunks of plan_zchunk).
-template <typename T, int DIM, int NSX, int RS, int MODE>
+template <typename T, int DIM, int NSX, int RS, int MODE, bool SMALL>
 __host__ __device__ constexpr int sweep_ctas() {
-  if (RS == RS_EXACT || (MODE & 1)) return DIM == 3 && sizeof(T) == 4 ? 2 : 1;
+  if (SMALL) return 1;
+  if (RS == RS_EXACT || (MODE & 1)) return DIM >= 2 && sizeof(T) == 4 ? 2 : 1;
   return SweepShape<T, DIM, NSX>::MB;
 }
 
-template <typename T, int DIM, int NSX, int RS, int MODE>
-__global__ void __launch_bounds__(SweepShape<T, DIM, NSX>::NT,
-                                  sweep_ctas<T, DIM, NSX, RS, MODE>())
+template <typename T, int DIM, int NSX, int RS, int MODE, bool SMALL>
+__global__ void __launch_bounds__(SweepShape<T, DIM, NSX, SMALL>::NT,
+                                  sweep_ctas<T, DIM, NSX, RS, MODE, SMALL>())
     sweep_kernel(const SweepArgs<T> args) {
-  using S = SweepShape<T, DIM, NSX>;
+  using S = SweepShape<T, DIM, NSX, SMALL>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   // dt (and the heating factor) come from thread 0 and are read after the
   // barrier that ends the staging; a launch behind a failed one (dt 0)
@@ -1127,7 +1116,7 @@ __global__ void __launch_bounds__(SweepShape<T, DIM, NSX>::NT,
     }
   }
 
-  Sweep<T, DIM, NSX, RS, MODE> sw(args, reinterpret_cast<T*>(smem_raw));
+  Sweep<T, DIM, NSX, RS, MODE, SMALL> sw(args, reinterpret_cast<T*>(smem_raw));
   if (sw.tsum)
     for (int q = threadIdx.x; q < S::NI * S::NV; q += S::NT) sw.tsum[q] = 0.0;  // (read after later barriers)
   sw.x0 = blockIdx.x * S::TX;
@@ -1202,11 +1191,11 @@ __global__ void __launch_bounds__(SweepShape<T, DIM, NSX>::NT,
 }
 
 // Launch one instantiation and report the launch's shape.
-template <typename T, int DIM, int NSX, int RS, int MODE = 0>
-cudaError_t launch_sweep(const SweepArgs<T>& args, cudaStream_t s, LaunchShape* sh) {
-  using S = SweepShape<T, DIM, NSX>;
+template <typename T, int DIM, int NSX, int RS, int MODE, bool SMALL>
+cudaError_t launch_tiled(const SweepArgs<T>& args, cudaStream_t s, LaunchShape* sh) {
+  using S = SweepShape<T, DIM, NSX, SMALL>;
   SweepArgs<T> a = args;
-  const void* fn = (const void*)sweep_kernel<T, DIM, NSX, RS, MODE>;
+  const void* fn = (const void*)sweep_kernel<T, DIM, NSX, RS, MODE, SMALL>;
   const size_t smem = a.tot_part ? S::tot_offset(MODE) + S::tot_bytes : S::smem_bytes_for(MODE);
   cudaError_t e = smem_attr_once(fn, (int)smem);
   if (e != cudaSuccess) return e;
@@ -1224,8 +1213,36 @@ cudaError_t launch_sweep(const SweepArgs<T>& args, cudaStream_t s, LaunchShape* 
   sh->zchunk = a.zchunk;
   sh->threads = S::NT;
   sh->ctas = (long long)grid.x * grid.y * grid.z;
-  sweep_kernel<T, DIM, NSX, RS, MODE><<<grid, S::NT, smem, s>>>(a);
+  sweep_kernel<T, DIM, NSX, RS, MODE, SMALL><<<grid, S::NT, smem, s>>>(a);
   return cudaGetLastError();
+}
+
+// Whether a 1D or 2D grid takes the small tiles: an SM's time goes with the
+// threads of the CTAs it gets (FP64: with its warps, whatever their active
+// lanes, from four warps on; fewer leave schedulers idle), so the shape whose
+// busiest SM has fewer threads wins.  FP64 Sod, 1000 cells: 36 one-warp CTAs
+// on 36 SMs instead of 4 of 8 warps on 4.
+template <typename T, int DIM, int NSX>
+bool small_tile(const int* n, int sms) {
+  auto busiest = [&](long long tx, long long ty, long long threads) {
+    const long long tiles = (n[0] + tx - 1) / tx * ((n[1] + ty - 1) / ty);
+    return std::max(128ll, (tiles + sms - 1) / sms * threads);
+  };
+  using L = SweepShape<T, DIM, NSX, false>;
+  using M = SweepShape<T, DIM, NSX, true>;
+  return busiest(M::TX, M::TY, M::NT) < busiest(L::TX, L::TY, L::NT);
+}
+
+template <typename T, int DIM, int NSX, int RS, int MODE = 0>
+cudaError_t launch_sweep(const SweepArgs<T>& a, cudaStream_t s, LaunchShape* sh) {
+  if constexpr (DIM < 3 && MODE == 0) {
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    if (small_tile<T, DIM, NSX>(a.n, sms)) return launch_tiled<T, DIM, NSX, RS, MODE, true>(a, s, sh);
+  }
+  return launch_tiled<T, DIM, NSX, RS, MODE, false>(a, s, sh);
 }
 
 // Instantiate the dispatcher of one (precision, dimension) pair and MODE
