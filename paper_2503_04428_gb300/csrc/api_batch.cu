@@ -463,7 +463,7 @@ static int mlp_gradient(cudaStream_t s, const float* W, const float* X, const fl
   mlp_grad_kernel<<<nblocks, 256, sizeof(MlpSmem), s>>>(W, X, Y, idx, first, count, (float)(1.0 / count),
                                                         partial, loss_partial);
   HCK(cudaGetLastError());
-  mlp_reduce_kernel<<<(MLP_NPARAM + 255) / 256, 256, 0, s>>>(partial, nblocks, grad, loss_partial, loss_acc);
+  mlp_reduce_kernel<<<MLP_RED_GRID, 32 * MLP_RED, 0, s>>>(partial, nblocks, grad, loss_partial, loss_acc, 1, 0);
   HCK(cudaGetLastError());
   return HYDRO_OK;
 }
@@ -1083,7 +1083,7 @@ int hydro_mlp_train(hydro_t h, const double* faces6, const double* log_pstar, lo
       const int nblk = (int)((bsz_use + MLP_SB - 1) / MLP_SB);
       mlp_grad_kernel<<<nblk, 256, sizeof(MlpSmem), s>>>(bs->w, X, Y, idx, first, bsz_use,
                                                          (float)(1.0 / bsz_use), part, lpart);
-      mlp_reduce_adam_kernel<<<(MLP_NPARAM + 255) / 256, 256, 0, s>>>(part, nblk, lpart, lacc, bs->w, bs->m,
+      mlp_reduce_adam_kernel<<<MLP_RED_GRID, 32 * MLP_RED, 0, s>>>(part, nblk, lpart, lacc, bs->w, bs->m,
                                                                       bs->v, step, lr_t, 0.9, 0.999, 1e-8);
       if (cudaGetLastError() != cudaSuccess) { st = HYDRO_ERR_CUDA; break; }
     }
@@ -1297,23 +1297,6 @@ static int noalloc_scratch(void** out) {
   return HYDRO_OK;
 }
 
-// grad[p] = sum of the partials of parameter p (fixed order, FP64);
-// loss = sum of the loss partials / n.
-__global__ void noalloc_reduce_kernel(const float* partial, const double* loss_partial, int nblocks, long n,
-                                      double* grad, double* loss) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p < MLP_NPARAM) {
-    double a = 0.0;
-    for (int b = 0; b < nblocks; ++b) a += (double)partial[(long long)b * MLP_NPARAM + p];
-    grad[p] = a;
-  }
-  if (p == 0) {
-    double l = 0.0;
-    for (int b = 0; b < nblocks; ++b) l += loss_partial[b];
-    *loss = l / (double)n;
-  }
-}
-
 }  // namespace hydro
 
 extern "C" int hydro_mlp_loss_grad_device(const float* weights, const float* x6, const float* target, long n,
@@ -1336,8 +1319,7 @@ extern "C" int hydro_mlp_loss_grad_device(const float* weights, const float* x6,
   mlp_grad_kernel<<<nblocks, 256, sizeof(MlpSmem), s>>>(weights, x6, target, nullptr, 0, n, (float)(1.0 / n),
                                                         partial, loss_partial);
   HCK(cudaGetLastError());
-  hydro::noalloc_reduce_kernel<<<(MLP_NPARAM + 255) / 256, 256, 0, s>>>(partial, loss_partial, nblocks, n,
-                                                                       grad_out, loss_out);
+  mlp_reduce_kernel<<<MLP_RED_GRID, 32 * MLP_RED, 0, s>>>(partial, nblocks, grad_out, loss_partial, loss_out, n, 1);
   HCK(cudaGetLastError());
   return HYDRO_OK;
 }
