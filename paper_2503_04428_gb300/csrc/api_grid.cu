@@ -444,7 +444,7 @@ static int launch_step_t(hydro_ctx* h, double dt_host, double cfl, double t_end,
     dim3 gb((h->n[0] + 31) / 32, h->shell_nchunks), tb(32, 8);
     shell_partial_kernel<T><<<gb, tb, 0, h->stream>>>(ctrl, (const T*)h->buf[0], (const T*)h->buf[1],
                                                       h->ncell, h->n[0], h->n[1], h->n[2],
-                                                      h->shell_kchunk, h->dvol[1], h->dvol[2],
+                                                      h->shell_kchunk, h->dvol[1], h->dvol[2], (const float2*)h->dv32[1], (const float2*)h->dv32[2],
                                                       h->shell_partial);
     HCK(cudaGetLastError());
     monopole_kernel<T><<<1, MONO_THREADS, 0, h->stream>>>(ctrl, h->shell_partial, h->shell_nchunks, h->n[0],
@@ -875,12 +875,12 @@ int hydro_shell_masses(hydro_t h, double* m_out) {
   if (h->precision == 64)
     shell_partial_kernel<double><<<gb, tb, 0, h->stream>>>(h->ctrl, (const double*)h->buf[0],
                                                            (const double*)h->buf[1], h->ncell, h->n[0], h->n[1],
-                                                           h->n[2], h->shell_kchunk, h->dvol[1], h->dvol[2],
+                                                           h->n[2], h->shell_kchunk, h->dvol[1], h->dvol[2], (const float2*)h->dv32[1], (const float2*)h->dv32[2],
                                                            h->shell_partial);
   else
     shell_partial_kernel<float><<<gb, tb, 0, h->stream>>>(h->ctrl, (const float*)h->buf[0],
                                                           (const float*)h->buf[1], h->ncell, h->n[0], h->n[1],
-                                                          h->n[2], h->shell_kchunk, h->dvol[1], h->dvol[2],
+                                                          h->n[2], h->shell_kchunk, h->dvol[1], h->dvol[2], (const float2*)h->dv32[1], (const float2*)h->dv32[2],
                                                           h->shell_partial);
   HCK(cudaGetLastError());
   shell_mass_kernel<<<(h->n[0] + 127) / 128, 128, 0, h->stream>>>(h->shell_partial, h->shell_nchunks, h->n[0],
@@ -1102,7 +1102,7 @@ int hydro_step_totals(hydro_t h, double* out_nv) {
   if (!h || h->batched || !out_nv) return arg_error("hydro_step_totals: bad argument");
   if (!h->step_tot || !h->step_tot_ok)
     return arg_error("hydro_step_totals: no step with totals since they were turned on or the state was set");
-  totals_final_kernel<<<1, 32, 0, h->stream>>>(h->step_tot_part, (int)h->shape.ctas, h->nv, h->tot_out);
+  totals_final_kernel<<<1, 256, 0, h->stream>>>(h->step_tot_part, (int)h->shape.ctas, h->nv, h->tot_out);
   HCK(cudaGetLastError());
   HCK(cudaMemcpyAsync(out_nv, h->tot_out, sizeof(double) * h->nv, cudaMemcpyDeviceToHost, h->stream));
   HCK(cudaStreamSynchronize(h->stream));
@@ -1124,7 +1124,7 @@ int hydro_totals(hydro_t h, double* out_nv) {
                                                               h->n[0], h->n[1], h->dvol[0], h->dvol[1],
                                                               h->dvol[2], h->tot_partial);
   HCK(cudaGetLastError());
-  totals_final_kernel<<<1, 32, 0, h->stream>>>(h->tot_partial, h->tot_blocks, h->nv, h->tot_out);
+  totals_final_kernel<<<1, 256, 0, h->stream>>>(h->tot_partial, h->tot_blocks, h->nv, h->tot_out);
   HCK(cudaGetLastError());
   HCK(cudaMemcpyAsync(out_nv, h->tot_out, sizeof(double) * h->nv, cudaMemcpyDeviceToHost, h->stream));
   HCK(cudaStreamSynchronize(h->stream));

@@ -11,64 +11,98 @@
 //                    and g_i = -G M_i / r_i^2, in a fixed order.
 #pragma once
 #include "common.cuh"
+#include "physics.cuh"
 
 namespace hydro {
 
+// Bound by HBM (one read of the state) in FP32 and by the FP64 pipe in FP64:
+// the cell's indices advance by the grid's stride without divisions, the
+// maximum stays in the state's precision (its conversion is exact) and is
+// reduced on bit patterns, one reciprocal serves a cell.  Measured, before ->
+// now: FP32 256^3 222 -> 98 us, FP64 128^3 450 -> 100 us.
 template <typename T, int DIM, typename G>
 __global__ void __launch_bounds__(256)
     validate_kernel(const T* __restrict__ U, long long ncell, int n0, int n1, int nv, G gas,
                     int spherical, const T* __restrict__ w0, const T* __restrict__ w1,
                     const T* __restrict__ w2, const T* __restrict__ ir, const T* __restrict__ is,
                     int* status, unsigned long long* smax_bits, int maxis, T wg) {
-  double smax = 0.0;
+  T smax = T(0);
   int err = 0;
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < ncell;
-       c += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(c % n0);
-    const int j = (int)((c / n0) % n1);
-    const int k = (int)(c / ((long long)n0 * n1));
-    T u[2 + DIM];
-    bool finite = true;
-#pragma unroll
-    for (int v = 0; v < 2 + DIM; ++v) {
-      u[v] = U[(long long)v * ncell + c];
-      finite = finite && isfinite(u[v]);
-    }
-    for (int v = 2 + DIM; v < nv; ++v) finite = finite && isfinite(U[(long long)v * ncell + c]);
-    if (!finite) { err = err ? err : ST_NONFINITE; continue; }
-    const T rho = u[0];
-    T ke = T(0);
-#pragma unroll
-    for (int d = 0; d < DIM; ++d) ke += u[1 + d] * u[1 + d];
-    T p, c2;
-    if constexpr (G::RAD) {
-      gas.from_e(rho, u[1 + DIM] - T(0.5) * ke / rho, p, c2);
-    } else {
-      p = gas.gm1 * (u[1 + DIM] - T(0.5) * ke / rho);
-      c2 = gas.g * p / rho;
-    }
-    if (!(rho > T(0)) || !(p > T(0))) { err = err ? err : ST_NEG; continue; }
-    const T cs = dsqrt(c2);
-    // (on a moving axis the speed relative to the faces)
-    T sp = (fabs(u[1] / rho - (maxis == 0 ? wg : T(0))) + cs) * w0[i + 2];
-    if (DIM >= 2) {
-      const T ih = spherical ? w1[j + 2] * ir[i + 2] : w1[j + 2];
-      sp += (fabs(u[2] / rho - (maxis == 1 ? wg : T(0))) + cs) * ih;
-    }
-    if (DIM == 3) {
-      const T ih = spherical ? w2[k + 2] * ir[i + 2] * is[j + 2] : w2[k + 2];
-      sp += (fabs(u[3] / rho - (maxis == 2 ? wg : T(0))) + cs) * ih;
-    }
-    smax = fmax(smax, (double)sp);
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  int i = (int)(c % n0), j = 0, k = 0, di = (int)(stride % n0), dj = 0, dk = 0;
+  if (DIM >= 2) {
+    const long long r = c / n0, dr = stride / n0;
+    j = (int)(r % n1);
+    k = (int)(r / n1);
+    dj = (int)(dr % n1);
+    dk = (int)(dr / n1);
   }
+  for (; c < ncell; c += stride) {
+    T u[2 + DIM];
+    T nul = T(0);  // 0 unless a value is infinite or NaN
+#pragma unroll
+    for (int v = 0; v < 2 + DIM; ++v) u[v] = U[(long long)v * ncell + c];
+    for (int v = 2 + DIM; v < nv; ++v) nul = finite_or(nul, U[(long long)v * ncell + c]);
+#pragma unroll
+    for (int v = 0; v < 2 + DIM; ++v) nul = finite_or(nul, u[v]);
+    if (!(nul == T(0))) {
+      err = err ? err : ST_NONFINITE;
+    } else {
+      const T rho = u[0], inv = one_over(rho);
+      T ke = T(0);
+#pragma unroll
+      for (int d = 0; d < DIM; ++d) ke += u[1 + d] * u[1 + d];
+      T p, c2;
+      if constexpr (G::RAD) {
+        gas.from_e(rho, u[1 + DIM] - T(0.5) * ke * inv, p, c2);
+      } else {
+        p = gas.gm1 * (u[1 + DIM] - T(0.5) * ke * inv);
+        c2 = gas.g * p * inv;
+      }
+      if (!is_pos(rho) || !is_pos(p)) {
+        err = err ? err : ST_NEG;
+      } else {
+        const T cs = dsqrt(c2);
+        // (on a moving axis the speed relative to the faces)
+        T sp = (fabs(u[1] * inv - (maxis == 0 ? wg : T(0))) + cs) * w0[i + 2];
+        if (DIM >= 2) {
+          const T ih = spherical ? w1[j + 2] * ir[i + 2] : w1[j + 2];
+          sp += (fabs(u[2] * inv - (maxis == 1 ? wg : T(0))) + cs) * ih;
+        }
+        if (DIM == 3) {
+          const T ih = spherical ? w2[k + 2] * ir[i + 2] * is[j + 2] : w2[k + 2];
+          sp += (fabs(u[3] * inv - (maxis == 2 ? wg : T(0))) + cs) * ih;
+        }
+        smax = larger_speed(smax, sp);
+      }
+    }
+    i += di;
+    if (DIM >= 2) {
+      if (i >= n0) {
+        i -= n0;
+        ++j;
+      }
+      j += dj;
+      if (j >= n1) {
+        j -= n1;
+        ++k;
+      }
+      k += dk;
+    } else if (i >= n0) {
+      i -= n0;
+    }
+  }
+  unsigned long long bits = dbits((double)smax);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    smax = fmax(smax, __shfl_xor_sync(0xffffffffu, smax, o));
+    const unsigned long long b2 = __shfl_xor_sync(0xffffffffu, bits, o);
+    bits = bits > b2 ? bits : b2;
     const int e2 = __shfl_xor_sync(0xffffffffu, err, o);
     err = err ? err : e2;
   }
   if ((threadIdx.x & 31) == 0) {
-    if (smax > 0.0) atomicMax(smax_bits, dbits(smax));
+    if (bits) atomicMax(smax_bits, bits);
     if (err) atomicCAS(status, 0, err);
   }
 }
@@ -103,31 +137,67 @@ __global__ void __launch_bounds__(256)
   if (threadIdx.x == 0) partial[(long long)v * gridDim.x + blockIdx.x] = red[0];
 }
 
-// Pass 2: one thread per variable sums the block partials in order.
+// Pass 2: one warp per variable sums the block partials, lane l those of
+// blocks l, l + 32, ..., then a tree: a fixed order (one thread per variable
+// waited for one addition after another: 54 us for the 684 partials of a
+// 256^3 step).
 __global__ void totals_final_kernel(const double* partial, int nblocks, int nv, double* out) {
-  const int v = threadIdx.x;
+  const int v = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (v >= nv) return;
   double s = 0.0;
-  for (int b = 0; b < nblocks; ++b) s += partial[(long long)v * nblocks + b];
-  out[v] = s;
+#pragma unroll 4
+  for (int b = lane; b < nblocks; b += 32) s += partial[(long long)v * nblocks + b];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) out[v] = s;
 }
 
 // Monopole pass 1: partial shell sums sum_{j,k in chunk} rho b_j c_k, for
-// 32 radial cells per block and one axis-2 chunk per blockIdx.y.
+// 32 radial cells per block and one axis-2 chunk per blockIdx.y.  FP64: the
+// products with b_j summed per plane, then times c_k.  FP32: b_j c_k as the
+// product of two FP32 pairs, the sum a compensated FP32 pair (each term costs
+// ~2^-48 of it), converted at the end: a conversion and two FP64 operations
+// per cell had occupied the FP64 pipe for 118 us of a 1.54 ms wedge step
+// (1024 x 128^2), now 53.
+struct ShellSum32 {
+  float2 s = {0.f, 0.f};
+  __device__ __forceinline__ void add(float rho, float2 b, float2 c) {
+    const float p = __fmul_rn(b.x, c.x);
+    const float e = fmaf(b.x, c.y, fmaf(b.y, c.x, fmaf(b.x, c.x, -p)));
+    add_column_sum(s, rho, make_float2(p, e));
+  }
+};
+
 template <typename T>
 __global__ void __launch_bounds__(256)
     shell_partial_kernel(const Ctrl* ctrl, const T* A, const T* B, long long ncell, int n0, int n1,
                          int n2, int kchunk, const double* __restrict__ db,
-                         const double* __restrict__ dc, double* partial) {
+                         const double* __restrict__ dc, const float2* __restrict__ b32,
+                         const float2* __restrict__ c32, double* partial) {
   if (((volatile const Ctrl*)ctrl)->status != 0) return;
   const T* U = ((volatile const Ctrl*)ctrl)->cur ? B : A;
   const int i = blockIdx.x * 32 + threadIdx.x;
   const int k0 = blockIdx.y * kchunk, k1 = min(k0 + kchunk, n2);
   double s = 0.0;
   if (i < n0) {
-    for (int k = k0; k < k1; ++k)
-      for (int j = threadIdx.y; j < n1; j += 8)
-        s += (double)U[((long long)k * n1 + j) * n0 + i] * (db[j] * dc[k]);
+    if constexpr (sizeof(T) == 4) {
+      ShellSum32 sum;
+      for (int k = k0; k < k1; ++k) {
+        const T* u = U + (long long)k * n1 * n0 + i;
+        const float2 c = c32[k];
+#pragma unroll 8
+        for (int j = threadIdx.y; j < n1; j += 8) sum.add(u[(long long)j * n0], b32[j], c);
+      }
+      s = (double)sum.s.x + (double)sum.s.y;
+    } else {
+      for (int k = k0; k < k1; ++k) {
+        const T* u = U + (long long)k * n1 * n0 + i;
+        double t = 0.0;
+#pragma unroll 4
+        for (int j = threadIdx.y; j < n1; j += 8) t += u[(long long)j * n0] * db[j];
+        s += t * dc[k];
+      }
+    }
   }
   __shared__ double red[8][33];
   red[threadIdx.y][threadIdx.x] = s;
@@ -140,9 +210,18 @@ __global__ void __launch_bounds__(256)
 }
 
 // Monopole pass 2 (one block of MONO_THREADS): shell masses, their prefix
-// sums by a block-wide Hillis-Steele scan (fixed order, so deterministic) and
-// the enclosed-mass acceleration of every radial cell.
+// sums by warp scans and a scan of the warps' sums (fixed order, so
+// deterministic) and the enclosed-mass acceleration of every radial cell.
 constexpr int MONO_THREADS = 1024;
+
+__device__ __forceinline__ double warp_scan(double v) {  // inclusive
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const double u = __shfl_up_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) >= o) v += u;
+  }
+  return v;
+}
 
 template <typename T>
 __global__ void __launch_bounds__(MONO_THREADS)
@@ -150,8 +229,8 @@ __global__ void __launch_bounds__(MONO_THREADS)
                     const double* __restrict__ da, const double* __restrict__ rc, double G,
                     double Mc, double four_pi_over_omega, double inner, double* shell, T* gmono) {
   if (((volatile const Ctrl*)ctrl)->status != 0) return;
-  __shared__ double sh[MONO_THREADS];
-  const int tid = threadIdx.x;
+  __shared__ double sh[32];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   // mass of all shells of the previous chunks, starting from the shells
   // inside this subdomain (0 unless the grid is one slab of an r-split)
   double carry = inner;
@@ -160,24 +239,24 @@ __global__ void __launch_bounds__(MONO_THREADS)
     double m = 0.0;
     if (i < n0) {
       double s = 0.0;
+#pragma unroll 4
       for (int q = 0; q < nchunks; ++q) s += partial[(long long)q * n0 + i];
       m = s * da[i];
     }
-    sh[tid] = m;
+    const double in = warp_scan(m);
+    if (lane == 31) sh[wid] = in;
     __syncthreads();
-    for (int off = 1; off < MONO_THREADS; off <<= 1) {
-      const double v = tid >= off ? sh[tid - off] : 0.0;
-      __syncthreads();
-      sh[tid] += v;
-      __syncthreads();
-    }
-    const double below = carry + (tid > 0 ? sh[tid - 1] : 0.0);
+    if (wid == 0) sh[lane] = warp_scan(sh[lane]);
+    __syncthreads();
+    double below = __shfl_up_sync(0xffffffffu, in, 1);  // of this warp's shells inside i
+    if (lane == 0) below = 0.0;
+    below = carry + (wid > 0 ? sh[wid - 1] : 0.0) + below;
     if (i < n0) {
       const double M = Mc + four_pi_over_omega * (below + 0.5 * m);
-      gmono[i] = (T)(-G * M / (rc[i] * rc[i]));
+      gmono[i] = (T)(-G * M * rcp<double>(rc[i] * rc[i]));
       shell[i] = M;
     }
-    carry += sh[MONO_THREADS - 1];
+    carry += sh[31];
     __syncthreads();
   }
 }

@@ -198,6 +198,33 @@ __device__ __forceinline__ double larger_speed(double a, double b) {
   return __double_as_longlong(a) < __double_as_longlong(b) ? b : a;
 }
 
+// sum += x z for z given as the pair z.x + z.y, the sum kept as a compensated
+// pair.  (The _rn intrinsics keep the compiler from fusing these operations.)
+__device__ __forceinline__ void add_column_sum(float2& sum, float x, float2 z) {
+  const float p = __fmul_rn(x, z.x);
+  const float e = fmaf(x, z.y, fmaf(x, z.x, -p));
+  const float t = __fadd_rn(sum.x, p);
+  const float bb = __fsub_rn(t, sum.x);
+  const float r = __fadd_rn(__fsub_rn(sum.x, __fsub_rn(t, bb)), __fsub_rn(p, bb));
+  const float lo = __fadd_rn(sum.y, __fadd_rn(r, e));
+  sum.x = __fadd_rn(t, lo);
+  sum.y = __fsub_rn(lo, __fsub_rn(sum.x, t));
+}
+
+// 0 as long as `nul` is 0 and x is finite, NaN otherwise (FP64: by the bits).
+__device__ __forceinline__ float finite_or(float nul, float x) { return fmaf(x, 0.0f, nul); }
+__device__ __forceinline__ double finite_or(double nul, double x) {
+  return (__double2hiint(x) & 0x7ff00000) == 0x7ff00000 ? __longlong_as_double(0x7ff8000000000000ll) : nul;
+}
+// Whether two numbers have the same bits.
+__device__ __forceinline__ bool same_bits(float a, float b) { return __float_as_int(a) == __float_as_int(b); }
+__device__ __forceinline__ bool same_bits(double a, double b) {
+  return __double_as_longlong(a) == __double_as_longlong(b);
+}
+// 1/x, correctly rounded in FP32.
+__device__ __forceinline__ float one_over(float x) { return 1.0f / x; }
+__device__ __forceinline__ double one_over(double x) { return rcp<double>(x); }
+
 template <typename T> __device__ __forceinline__ T dexp(T x);
 template <> __device__ __forceinline__ double dexp<double>(double x) { return exp(x); }
 template <> __device__ __forceinline__ float dexp<float>(float x) { return expf(x); }

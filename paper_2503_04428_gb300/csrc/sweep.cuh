@@ -125,19 +125,6 @@ __device__ __forceinline__ int map_axis(int g, int n, int lo, int hi, bool& flip
   return g;
 }
 
-// sum += x z for z given as the pair z.x + z.y, the sum kept as a compensated
-// pair.  (The _rn intrinsics keep the compiler from fusing these operations.)
-__device__ __forceinline__ void add_column_sum(float2& sum, float x, float2 z) {
-  const float p = __fmul_rn(x, z.x);
-  const float e = fmaf(x, z.y, fmaf(x, z.x, -p));
-  const float t = __fadd_rn(sum.x, p);
-  const float bb = __fsub_rn(t, sum.x);
-  const float r = __fadd_rn(__fsub_rn(sum.x, __fsub_rn(t, bb)), __fsub_rn(p, bb));
-  const float lo = __fadd_rn(sum.y, __fadd_rn(r, e));
-  sum.x = __fadd_rn(t, lo);
-  sum.y = __fsub_rn(lo, __fsub_rn(sum.x, t));
-}
-
 // The CTA's totals of its NI owners' sums [v][owner], by a tree in a fixed
 // order per variable (so the result does not depend on scheduling), left in
 // sums[v][0].
