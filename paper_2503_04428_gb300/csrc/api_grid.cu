@@ -491,6 +491,39 @@ static int launch_step(hydro_ctx* h, double dt_host, double cfl, double t_end, C
                             : launch_step_t<float>(h, dt_host, cfl, t_end, ctrl);
 }
 
+// nsteps CFL steps of a small 1D or 2D grid of the plain ideal gas by launches
+// of many steps (sweep_steps_kernel); *taken: whether the handle takes that
+// path.  (Not with in-step totals, whose partials are those of one step, nor
+// with the monopole, whose shell sums are kernels of their own.)
+template <typename T>
+static int launch_steps_t(hydro_ctx* h, int nsteps, double cfl, double t_end, bool* taken) {
+  *taken = false;
+  if (nsteps < 2 || h->dim > 2 || h->eos_rad || h->eps_dual > 0.0 || h->xaxis >= 0 || h->maxis >= 0 || h->step_tot ||
+      h->gravity == GRAV_MONO)
+    return HYDRO_OK;
+  const SweepArgs<T> a = sweep_args<T>(h, 0.0, cfl, t_end, h->ctrl);
+  auto launch = [&](const StepsArgs& sa) {
+    return h->dim == 1 ? steps_dispatch<T, 1>(a, sa, h->nsx, h->riemann, h->stream, &h->shape, taken)
+                       : steps_dispatch<T, 2>(a, sa, h->nsx, h->riemann, h->stream, &h->shape, taken);
+  };
+  StepsArgs sa = {nullptr, 0};
+  cudaError_t e = launch(sa);
+  if (e != cudaSuccess) return cuda_fail(e, "sweep launch");
+  if (!*taken) return HYDRO_OK;
+  const size_t words = sizeof(unsigned long long) * 2 * 2 * h->num_sms;  // (at most two CTAs per SM)
+  if (!h->steps_speed) {
+    const int st = h->arena.alloc(&h->steps_speed, words);
+    if (st) return st;
+  }
+  sa.speed = (unsigned long long*)h->steps_speed;
+  for (int left = nsteps; left > 0; left -= sa.nsteps) {
+    sa.nsteps = std::min(left, 4096);  // (a launch of tens of milliseconds at most)
+    HCK(cudaMemsetAsync(sa.speed, 0, words, h->stream));
+    if ((e = launch(sa)) != cudaSuccess) return cuda_fail(e, "sweep launch");
+  }
+  return HYDRO_OK;
+}
+
 static int read_ctrl(hydro_ctx* h) {
   HCK(cudaMemcpyAsync(h->ctrl_host, h->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->stream));
   HCK(cudaStreamSynchronize(h->stream));
@@ -1048,6 +1081,15 @@ int hydro_run(hydro_t h, int nsteps, double cfl, double t_end, double* t_out) {
     return HYDRO_OK;
   }
   int st;
+  bool taken = false;
+  st = h->precision == 64 ? launch_steps_t<double>(h, nsteps, cfl, t_end, &taken)
+                          : launch_steps_t<float>(h, nsteps, cfl, t_end, &taken);
+  if (st) return st;
+  if (taken) {
+    st = check_status(h, "hydro_run");
+    if (t_out) *t_out = h->ctrl_host->t;
+    return st;
+  }
   if (!h->graph || h->graph_cfl != cfl || h->graph_tend != t_end) {
     if (h->graph) {
       cudaGraphExecDestroy(h->graph);

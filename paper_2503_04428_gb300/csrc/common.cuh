@@ -166,6 +166,14 @@ inline int plan_zchunk(long long tiles, int n2, long long slots, int per, double
 
 template <typename T, int DIM>
 cudaError_t sweep_dispatch(const SweepArgs<T>& a, int nsx, int rs, cudaStream_t s, LaunchShape* sh);
+// Several steps in one launch (sweep_steps_kernel).
+struct StepsArgs {
+  unsigned long long* speed;  // 2 x CTAs words, zeroed before the launch: by step parity, the CTAs' speed maxima
+  int nsteps;
+};
+template <typename T, int DIM>
+cudaError_t steps_dispatch(const SweepArgs<T>& a, const StepsArgs& sa, int nsx, int rs, cudaStream_t s,
+                           LaunchShape* sh, bool* taken);
 // The FP32 3D step of the plain ideal gas with HLL or HLLC (march3.cuh).
 cudaError_t march3_dispatch(const SweepArgs<float>& a, int nsx, int rs, cudaStream_t s, LaunchShape* sh);
 // The FP32 2D step of the plain ideal gas with HLL or HLLC (march2.cuh).

@@ -84,6 +84,7 @@ struct hydro_ctx {
   bool step_tot = false, step_tot_ok = false;
   double* step_tot_part = nullptr;
   hydro::LaunchShape shape;  // of the last step launched
+  void* steps_speed = nullptr;  // several steps per launch: the words the CTAs publish
   // domain decomposition (Sect. 3.3.1): exchanged sides of axis xaxis, the
   // two face coordinates beyond each (nearest first), their halo buffers
   // [nv][2][cross section] on the device, and the monopole's inner mass

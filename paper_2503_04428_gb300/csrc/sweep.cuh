@@ -146,7 +146,8 @@ enum { PRED_ALL = 0, PRED_ZHI = 1, PRED_ZLO = 2 };
 // (Sect. 2.5); bit 2: a slab of a decomposed grid or a moving grid (exchanged
 // ghosts, moving faces; ideal gas only).  Each combination is its own
 // instantiation, so the plain step carries none of the optional work.
-template <typename T, int DIM, int NSX, int RS, int MODE, bool SMALL>
+// SMALL: the small tiles; MULTI: several steps in one launch (sweep_steps_kernel).
+template <typename T, int DIM, int NSX, int RS, int MODE, bool SMALL, bool MULTI = false>
 struct Sweep {
   static constexpr int EOS = MODE & 1;
   static constexpr bool DUAL = (MODE & 2) != 0;
@@ -197,6 +198,7 @@ struct Sweep {
   T acc[NV];
   T dUo[NV];
   T fzb3 = T(0), tth = T(0), x2 = T(0), s3 = T(0);
+  T Ucell[MULTI ? NV : 1];  // several steps per launch: the owned cell's conserved state
   T aq1 = T(0), aq2 = T(0);  // dual energy: divergences of u e and of u (times dt^-1)
 
   __device__ Sweep(const SweepArgs<T>& args, T* smem) : a(args) {
@@ -290,6 +292,12 @@ struct Sweep {
     else return a.gas;
   }
 
+  // State loads: several steps per launch read other CTAs' fresh cells, from L2.
+  static __device__ __forceinline__ T load(const T* p) {
+    if constexpr (MULTI) return __ldcg(p);
+    else return __ldg(p);
+  }
+
   __device__ __forceinline__ T& W(int slot, int v, int ey, int ex) {
     return Ws[((slot * NV + v) * EY + ey) * EX + ex];
   }
@@ -317,7 +325,7 @@ struct Sweep {
         const long long c = zoff + (long long)(y0 - HY + ey) * n0 + (x0 - 2 + ex);
         T u[NV], w[NV];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) u[v] = v < nvact ? __ldg(Uin + (long long)v * a.ncell + c) : T(0);
+        for (int v = 0; v < NV; ++v) u[v] = v < nvact ? load(Uin + (long long)v * a.ncell + c) : T(0);
         if constexpr (EOS == 1) {
           T c2, t;
           int k = 0;
@@ -350,7 +358,7 @@ struct Sweep {
       if (layer < 0) {
         const long long c = ((long long)sz * n1 + sj) * n0 + si;
 #pragma unroll
-        for (int v = 0; v < NV; ++v) u[v] = v < nvact ? __ldg(Uin + (long long)v * a.ncell + c) : T(0);
+        for (int v = 0; v < NV; ++v) u[v] = v < nvact ? load(Uin + (long long)v * a.ncell + c) : T(0);
       } else {
         // the neighbour subdomain's cell, from the halo of that side; the
         // other axes are mapped (and flipped) as for any ghost
@@ -819,7 +827,10 @@ struct Sweep {
     const long long c = ((long long)gz * n1 + gj) * n0 + gi;
     T Uo[NV], Un[NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) Uo[v] = v < nvact ? Uin[(long long)v * a.ncell + c] : T(0);
+    for (int v = 0; v < NV; ++v) {
+      if constexpr (MULTI) Uo[v] = Ucell[v];
+      else Uo[v] = v < nvact ? Uin[(long long)v * a.ncell + c] : T(0);
+    }
 #pragma unroll
     for (int v = 0; v < NV; ++v) Un[v] = Uo[v] + dt * acc[v];
 
@@ -961,8 +972,10 @@ struct Sweep {
     }
     smax = larger_speed(smax, sp);
 #pragma unroll
-    for (int v = 0; v < NV; ++v)
+    for (int v = 0; v < NV; ++v) {
       if (v < nvact) Uout[(long long)v * a.ncell + c] = Un[v];
+      if constexpr (MULTI) Ucell[v] = Un[v];
+    }
   }
 
   // The owner's work after the face solves of plane gz: in 3D, close the
@@ -1177,6 +1190,167 @@ __global__ void __launch_bounds__(SweepShape<T, DIM, NSX, SMALL>::NT,
                      (MODE & 1) ? (unsigned long long)sw.t_iters : sw.n_iters, s_dt);
 }
 
+// Several steps of a small 1D or 2D grid in one cooperative launch.  A step of
+// such a grid is a chain of latencies (launch, control block, loads, atomics
+// of the commit: ~9 of the 14.5 us of a 1000-cell FP64 step), so here the CTAs
+// stay, the owners keep their cells in registers, and one word per CTA and
+// step replaces the commit: a CTA publishes its speed maximum (release, after
+// its stores), waits (bounded) for every CTA's and takes their maximum itself.
+// A word's sign bit says which use of it is meant: the words of even and odd
+// steps are apart, zeroed before the launch, and each use flips the sign, so
+// none is overwritten before all have read it (9.6 us per step; 9.8 with a
+// counter beside the words).  A step that fails in a CTA
+// publishes NaN: every CTA ends with the state before it.  The buffers
+// alternate as between launches.
+constexpr int ST_STEP_TIMEOUT = -6;  // HYDRO_ERR_TIMEOUT
+
+template <typename T, int DIM, int NSX, int RS>
+__global__ void __launch_bounds__(SweepShape<T, DIM, NSX, true>::NT, 1)
+    sweep_steps_kernel(const SweepArgs<T> args, const StepsArgs sa) {
+  using S = SweepShape<T, DIM, NSX, true>;
+  constexpr int NT = S::NT;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ double s_dt;
+  __shared__ T s_hfac;
+  __shared__ unsigned long long s_speed[NT / 32];
+  __shared__ int s_err[NT / 32], s_go;
+  Ctrl* const ctrl = args.ctrl;
+  const volatile Ctrl* vc = ctrl;
+  const int cur0 = vc->cur;
+  const long long step0 = vc->step;
+  const unsigned int ctas = gridDim.x * gridDim.y, cta = blockIdx.x + gridDim.x * blockIdx.y;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+
+  Sweep<T, DIM, NSX, RS, 0, true, true> sw(args, reinterpret_cast<T*>(smem_raw));
+  sw.x0 = blockIdx.x * S::TX;
+  sw.y0 = blockIdx.y * S::TY;
+  sw.stage_geometry();  // (read after the first barrier below)
+  sw.n2 = sw.z1 = 1;
+  {
+    const T* U = cur0 ? args.B : args.A;
+    const int t = threadIdx.x, gi = sw.x0 + t % S::TX, gj = DIM >= 2 ? sw.y0 + t / S::TX : 0;
+    const bool own = t < S::NI && gi < args.n[0] && (DIM < 2 || gj < args.n[1]);
+    const int nvact = NSX < 3 ? S::NV : 2 + DIM + args.ns;
+#pragma unroll
+    for (int v = 0; v < S::NV; ++v)
+      sw.Ucell[v] = own && v < nvact ? __ldcg(U + (long long)v * args.ncell + (long long)gj * args.n[0] + gi) : T(0);
+  }
+  // thread 0: the state's speed, its time, and the steps done
+  double smax = vc->smax_cur, t = vc->t, last_dt = vc->last_dt;
+  constexpr unsigned long long FAILED = 0x7ff8000000000000ull;
+  const bool idle = vc->status != 0;  // (an earlier failure; constant until a step of this launch fails)
+  int done = 0;
+  for (;;) {
+    if (threadIdx.x == 0) {
+      double dt = 0.0;
+      if (!idle && done < sa.nsteps) {
+        dt = args.cfl / smax;
+        if (args.t_end > 0.0) dt = fmin(dt, args.t_end - t);
+      }
+      s_dt = dt;
+      if (args.heating == HEAT_NI56)
+        s_hfac = (T)(args.ni_lambda * (args.ni_a * exp(-t / args.ni_tni) + args.ni_qco * exp(-t / args.ni_tco)));
+    }
+    const bool odd = ((cur0 ^ done) & 1) != 0;
+    sw.Uin = odd ? args.B : args.A;
+    sw.Uout = odd ? args.Aw : args.B;
+    sw.load_plane(0);
+    __syncthreads();
+    const double dtd = s_dt;
+    if (!(dtd > 0.0)) break;
+    sw.dt = (T)dtd;
+    sw.half_dt = T(0.5) * sw.dt;
+    sw.hfac = args.heating == HEAT_NI56 ? s_hfac : T(0);
+    sw.smax = T(0);
+    sw.template predictor<PRED_ALL>(0);
+    __syncthreads();
+    sw.template faces<true, false>(0);
+    __syncthreads();
+    sw.owner_step(0, false, true);
+    unsigned long long bits = dbits((double)sw.smax);
+    int err = sw.err;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long b2 = __shfl_xor_sync(0xffffffffu, bits, o);
+      bits = bits > b2 ? bits : b2;
+    }
+    if (__any_sync(0xffffffffu, err != 0)) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const int e2 = __shfl_xor_sync(0xffffffffu, err, o);
+        err = err ? err : e2;
+      }
+    }
+    if (lane == 0) {
+      s_speed[wid] = bits;
+      s_err[wid] = err;
+    }
+    __syncthreads();  // (also: every thread's stores of the step come before the release below)
+    unsigned long long* const speed = sa.speed + (size_t)(done & 1) * ctas;
+    const unsigned long long use = (done >> 1) & 1 ? 0ull : 1ull << 63;
+    if (wid == 0) {
+      if (lane == 0) {
+        for (int w = 1; w < NT / 32; ++w) {
+          bits = bits > s_speed[w] ? bits : s_speed[w];
+          err = err ? err : s_err[w];
+        }
+        if (err) {
+          bits = FAILED;
+          if (atomicCAS(&ctrl->status, 0, err) == 0) ctrl->err_step = step0 + done;
+        }
+        asm volatile("st.release.gpu.global.u64 [%0], %1;\n" ::"l"(speed + cta), "l"(bits | use) : "memory");
+      }
+      unsigned long long m = 0ull;
+      for (unsigned int c = lane; c < ctas; c += 32) {
+        unsigned long long b = 0ull;
+        int poll = 0;
+        do {
+          asm volatile("ld.acquire.gpu.global.u64 %0, [%1];\n" : "=l"(b) : "l"(speed + c) : "memory");
+        } while (((b ^ use) >> 63) != 0ull && ++poll < (1 << 22));
+        if (((b ^ use) >> 63) != 0ull) {  // the bounded wait expired
+          b = FAILED;
+          if (atomicCAS(&ctrl->status, 0, ST_STEP_TIMEOUT) == 0) ctrl->err_step = step0 + done;
+        }
+        b &= ~(1ull << 63);
+        m = m > b ? m : b;
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long b2 = __shfl_xor_sync(0xffffffffu, m, o);
+        m = m > b2 ? m : b2;
+      }
+      if (m < FAILED) smax = __longlong_as_double((long long)m);
+      if (lane == 0) s_go = m < FAILED;
+    }
+    __syncthreads();
+    if (!s_go) break;  // this step failed: the state before it stays
+    t += dtd;
+    last_dt = dtd;
+    ++done;
+  }
+  // counters, and the commit of the steps done
+  unsigned long long fb = sw.n_fallback, it = sw.n_iters;
+  if (__any_sync(0xffffffffu, fb != 0 || it != 0)) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      fb += __shfl_xor_sync(0xffffffffu, fb, o);
+      it += __shfl_xor_sync(0xffffffffu, it, o);
+    }
+    if (lane == 0) {
+      if (fb) atomicAdd(&ctrl->fallbacks, fb);
+      if (it) atomicAdd(&ctrl->iters, it);
+    }
+  }
+  if (cta == 0 && threadIdx.x == 0 && done > 0) {
+    volatile Ctrl* w = ctrl;
+    w->smax_cur = smax;
+    w->t = t;
+    w->last_dt = last_dt;
+    w->step = step0 + done;
+    w->cur = cur0 ^ (done & 1);
+  }
+}
+
 // Launch one instantiation and report the launch's shape.
 template <typename T, int DIM, int NSX, int RS, int MODE, bool SMALL>
 cudaError_t launch_tiled(const SweepArgs<T>& args, cudaStream_t s, LaunchShape* sh) {
@@ -1220,6 +1394,35 @@ bool small_tile(const int* n, int sms) {
   return busiest(M::TX, M::TY, M::NT) < busiest(L::TX, L::TY, L::NT);
 }
 
+// nsteps steps in one launch (sa set but for its step count): whether the
+// grid takes this path (small tiles, at most two CTAs per SM, all resident),
+// reported in *taken; with nsteps 0 nothing is launched.
+template <typename T, int DIM, int NSX, int RS>
+cudaError_t launch_steps(const SweepArgs<T>& args, const StepsArgs& sa, cudaStream_t s, LaunchShape* sh, bool* taken) {
+  using S = SweepShape<T, DIM, NSX, true>;
+  *taken = false;
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  dim3 grid((args.n[0] + S::TX - 1) / S::TX, DIM >= 2 ? (args.n[1] + S::TY - 1) / S::TY : 1);
+  const long long ctas = (long long)grid.x * grid.y;
+  if (!small_tile<T, DIM, NSX>(args.n, sms) || ctas > 2 * sms) return cudaSuccess;
+  const void* fn = (const void*)sweep_steps_kernel<T, DIM, NSX, RS>;
+  const size_t smem = S::smem_bytes_for(0);
+  if ((e = smem_attr_once(fn, (int)smem)) != cudaSuccess) return e;
+  long long slots;
+  if ((e = kernel_slots(fn, S::NT, smem, &slots)) != cudaSuccess) return e;
+  if (ctas > slots) return cudaSuccess;
+  *taken = true;
+  if (sa.nsteps < 1) return cudaSuccess;
+  *sh = LaunchShape{S::TX, S::TY, 1, S::NT, ctas};
+  SweepArgs<T> a = args;
+  StepsArgs b = sa;
+  void* params[] = {&a, &b};
+  return cudaLaunchCooperativeKernel(fn, grid, dim3(S::NT), params, smem, s);
+}
+
 template <typename T, int DIM, int NSX, int RS, int MODE = 0>
 cudaError_t launch_sweep(const SweepArgs<T>& a, cudaStream_t s, LaunchShape* sh) {
   if constexpr (DIM < 3 && MODE == 0) {
@@ -1251,6 +1454,30 @@ cudaError_t launch_sweep(const SweepArgs<T>& a, cudaStream_t s, LaunchShape* sh)
       default: return cudaErrorInvalidValue;                                                  \
     }                                                                                         \
   }
+// Several steps in one launch: all solvers, or the exact one alone (FP32 2D).
+#define HYDRO_STEPS_CASES(T, DIM, NSX, HYDRO_RS_CASES)                                        \
+  switch (rs) {                                                                               \
+    HYDRO_RS_CASES(T, DIM, NSX)                                                               \
+    default: return cudaSuccess;                                                              \
+  }
+#define HYDRO_RS_ALL(T, DIM, NSX)                                                             \
+  case RS_HLL: return launch_steps<T, DIM, NSX, RS_HLL>(a, sa, s, sh, taken);                 \
+  case RS_HLLC: return launch_steps<T, DIM, NSX, RS_HLLC>(a, sa, s, sh, taken);               \
+  case RS_EXACT: return launch_steps<T, DIM, NSX, RS_EXACT>(a, sa, s, sh, taken);
+#define HYDRO_RS_EXACT_ONLY(T, DIM, NSX)                                                      \
+  case RS_EXACT: return launch_steps<T, DIM, NSX, RS_EXACT>(a, sa, s, sh, taken);
+#define HYDRO_STEPS_DISPATCH(T, DIM, HYDRO_RS_CASES)                                          \
+  template <>                                                                                 \
+  cudaError_t steps_dispatch<T, DIM>(const SweepArgs<T>& a, const StepsArgs& sa, int nsx,     \
+                                     int rs, cudaStream_t s, LaunchShape* sh, bool* taken) {  \
+    *taken = false;                                                                           \
+    switch (nsx) {                                                                            \
+      case 0: HYDRO_STEPS_CASES(T, DIM, 0, HYDRO_RS_CASES)                                    \
+      case 1: HYDRO_STEPS_CASES(T, DIM, 1, HYDRO_RS_CASES)                                    \
+      default: HYDRO_STEPS_CASES(T, DIM, 3, HYDRO_RS_CASES)                                   \
+    }                                                                                         \
+  }
+
 // The exact solver alone (the FP32 2D and 3D forms, whose HLL and HLLC steps march).
 #define HYDRO_SWEEP_DISPATCH_EXACT(T, DIM)                                                    \
   template <>                                                                                 \

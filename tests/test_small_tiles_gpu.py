@@ -39,3 +39,56 @@ def test_sizes(hydro_lib, n, precision):
         tot = g.totals()
         assert np.allclose(g.step_totals(), tot, rtol=0, atol=1e-6 * np.abs(tot).max())
         g.close()
+
+
+@pytest.mark.parametrize("precision", [64, 32])
+@pytest.mark.parametrize("n", [[2], [29], [300], [4000], [3, 5], [40, 33], [120, 100]])
+def test_run_equals_single_steps(hydro_lib, n, precision):
+    """hydro_run (many steps in one launch on these grids) against the same
+    steps one by one with hydro_cfl_dt, to the rounding of the steps: 12 steps
+    of at most ~100 roundings, eps = 1.1e-16 / 6e-8, allowing a factor of 30
+    for the flow's growth; and the time clipped to t_end, a run past it doing
+    nothing more."""
+    for k, riemann in enumerate((O.HLL, O.HLLC, O.EXACT)):
+        case = wl.smooth_random(len(n), n, k + 1, seed=90 + k, bc=[(T, R), (P, P)][:len(n)], riemann=riemann)
+        a, b = [hydro_lib.Grid.from_case(case, precision) for _ in range(2)]
+        for _ in range(12):
+            b.step(b.cfl_dt(0.4))
+        t = a.run(12, 0.4)
+        sb = b.stats()
+        assert a.stats()["steps"] == sb["steps"] == 12
+        tol = 3e-13 if precision == 64 else 2e-4
+        assert abs(t - sb["t"]) <= tol * sb["t"]
+        A, B = a.get_state().astype(np.float64), b.get_state().astype(np.float64)
+        assert np.abs(A - B).max() <= tol * np.abs(B).max()
+        t_end = t + 1.5 * a.stats()["last_dt"]
+        assert a.run(100, 0.4, t_end) == pytest.approx(t_end, rel=1e-14)
+        done = a.stats()["steps"]
+        assert 13 <= done <= 15
+        a.run(7, 0.4, t_end)
+        assert a.stats()["steps"] == done
+        a.close()
+        b.close()
+
+
+@pytest.mark.parametrize("n", [[200], [40, 24]])
+def test_failed_run_keeps_the_last_good_state(hydro_lib, n):
+    """A run at a hopeless CFL number fails after some steps: status, step
+    count and state are those of the last good step, and the handle goes on."""
+    case = wl.smooth_random(len(n), n, 0, seed=5, amp=0.5, riemann=O.HLLC)
+    a, b = [hydro_lib.Grid.from_case(case, 64) for _ in range(2)]
+    good = 0
+    with pytest.raises(hydro_lib.HydroError) as e1:
+        for _ in range(60):
+            b.step(b.cfl_dt(6.0))
+            good += 1
+    with pytest.raises(hydro_lib.HydroError) as e2:
+        a.run(60, 6.0)
+    assert e1.value.status == e2.value.status
+    assert a.stats()["steps"] == good and a.stats()["t"] == pytest.approx(b.stats()["t"], rel=1e-9)
+    A, B = a.get_state(), b.get_state()
+    assert np.abs(A - B).max() <= 1e-6 * np.abs(B).max()
+    a.run(3, 0.2)
+    assert a.stats()["steps"] == good + 3
+    a.close()
+    b.close()
