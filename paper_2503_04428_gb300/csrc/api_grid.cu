@@ -350,7 +350,8 @@ Gas<T> make_gas(double gm) {
   g.Bq = (T)((gm - 1.0) / (gm + 1.0));
   g.two_gm1 = (T)(2.0 / (gm - 1.0));
   g.ig = (T)(1.0 / gm);
-  g.pow_c = (T)(2.0 * gm / (gm - 1.0));
+  const double iz = 2.0 * gm / (gm - 1.0), n = std::round(iz);
+  g.root = std::fabs(iz - n) < 1e-9 && n >= 4.0 && n <= 8.0 ? (int)n : 0;
   return g;
 }
 template Gas<float> make_gas<float>(double);

@@ -509,9 +509,9 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 5)
         const T r0 = slot[i0], r1 = slot[BVSTR + i0], r2 = slot[2 * BVSTR + i0];
         bool eq = true;
         for (int i = i0 + lane; i < i1; i += 32)
-          eq = eq & (slot[i] == r0) & (slot[BVSTR + i] == r1) & (slot[2 * BVSTR + i] == r2);
+          eq = eq & equal_values(slot[i], r0) & equal_values(slot[BVSTR + i], r1) & equal_values(slot[2 * BVSTR + i], r2);
         if (__all_sync(0xffffffffu, eq)) {
-          if (!(have_u & (r0 == ur[0]) & (r1 == ur[1]) & (r2 == ur[2]))) {
+          if (!(have_u & equal_values(r0, ur[0]) & equal_values(r1, ur[1]) & equal_values(r2, ur[2]))) {
             have_u = true;
             ur[0] = r0;
             ur[1] = r1;
@@ -520,7 +520,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 5)
             u_spd = us.s;
             if (err == 0) err = us.st;
           }
-          smax = fmax(smax, u_spd * fn);
+          smax = larger_speed(smax, u_spd * fn);
           const int a0 = s_beg + k * BSPAN * BSEG, a1 = min(a0 + BSPAN * BSEG, s_end);
           const T o0 = ur[0] + T(0), o1 = ur[1] + T(0), o2 = ur[2] + T(0);
           for (int c = a0 + lane; c < a1; c += 32) {
@@ -551,12 +551,13 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 5)
         // undisturbed stretch of a tube: no shuffles), then against lane 0.
         // (every vote and shuffle runs on every lane: a collective inside a
         // short-circuit condition would leave lanes out of it)
-        bool uniform = __all_sync(0xffffffffu, have_u & (Ua[0] == ur[0]) & (Ua[1] == ur[1]) & (Ua[2] == ur[2]));
+        bool uniform = __all_sync(0xffffffffu, have_u & equal_values(Ua[0], ur[0]) & equal_values(Ua[1], ur[1]) &
+                                                  equal_values(Ua[2], ur[2]));
         if (!uniform) {
           const T r0 = __shfl_sync(0xffffffffu, Ua[0], 0);
           const T r1 = __shfl_sync(0xffffffffu, Ua[1], 0);
           const T r2 = __shfl_sync(0xffffffffu, Ua[2], 0);
-          uniform = __all_sync(0xffffffffu, (Ua[0] == r0) & (Ua[1] == r1) & (Ua[2] == r2));
+          uniform = __all_sync(0xffffffffu, equal_values(Ua[0], r0) & equal_values(Ua[1], r1) & equal_values(Ua[2], r2));
           if (uniform) {
             // a new uniform state: its validity and |u| + c, kept for the
             // windows that repeat it
@@ -572,7 +573,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 5)
         if (uniform) {
           // (equal values compare equal but for the sign of zero, which
           // U + 0 erases: the cached state's U + 0 is the window's)
-          smax = fmax(smax, u_spd * fn);
+          smax = larger_speed(smax, u_spd * fn);
           if (lane < ncell) {
             T* o = out + c0 + lane;
             o[0] = ur[0] + T(0);
@@ -611,12 +612,12 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 5)
           to_prim<T, 1, 0>(uh, Whi, gas);
           // a non-physical prediction falls back to the cell average
           const bool own = lane >= 1 && lane <= ncell;  // cells of this segment
-          if (!(Wlo[0] > T(0)) || !(Wlo[2] > T(0))) {
+          if (!is_pos(Wlo[0]) || !is_pos(Wlo[2])) {
 #pragma unroll
             for (int v = 0; v < 3; ++v) Wlo[v] = Wc[v];
             if (own) ++n_fb;
           }
-          if (!(Whi[0] > T(0)) || !(Whi[2] > T(0))) {
+          if (!is_pos(Whi[0]) || !is_pos(Whi[2])) {
 #pragma unroll
             for (int v = 0; v < 3; ++v) Whi[v] = Wc[v];
             if (own) ++n_fb;
@@ -632,7 +633,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 5)
         }
         const bool face = lane <= ncell;
         const bool owned = face && (lane < ncell || c0 + lane == nb);
-        const bool same = WL[0] == WR[0] && WL[1] == WR[1] && WL[2] == WR[2];
+        const bool same = equal_values(WL[0], WR[0]) && equal_values(WL[1], WR[1]) && equal_values(WL[2], WR[2]);
         T pg = T(0);
         int kind = 0;
         bool by_mlp = false;  // pg came from the network
@@ -713,8 +714,8 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 5)
           }
           to_prim<T, 1, 0>(u, w, gas);
           if (!finite) err = err ? err : ST_NONFINITE;
-          else if (!(w[0] > T(0)) || !(w[2] > T(0))) err = err ? err : ST_NEG;
-          smax = fmax(smax, (fabs(w[1]) + dsqrt(qdiv(gas.g * w[2], w[0]))) * fn);
+          else if (!is_pos(w[0]) || !is_pos(w[2])) err = err ? err : ST_NEG;
+          smax = larger_speed(smax, (fabs(w[1]) + dsqrt(qdiv(gas.g * w[2], w[0]))) * fn);
 #pragma unroll
           for (int v = 0; v < 3; ++v) Uout[v * a.stride + c] = u[v];
         }

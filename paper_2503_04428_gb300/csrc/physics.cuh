@@ -35,7 +35,7 @@ struct Gas {
   T Bq;       // (gamma - 1)/(gamma + 1)
   T two_gm1;  // 2/(gamma - 1)
   T ig;       // 1/gamma
-  T pow_c;    // 2 gamma/(gamma - 1)
+  int root;   // 1/z if that is one of 4, ..., 8 (gamma = 2, 5/3, 3/2, 7/5, 4/3), else 0
 };
 
 // FP64 on this part: one warp instruction occupies an SM's FP64 pipe for 19
@@ -215,6 +215,11 @@ __device__ __forceinline__ void add_column_sum(float2& sum, float x, float2 z) {
 __device__ __forceinline__ float finite_or(float nul, float x) { return fmaf(x, 0.0f, nul); }
 __device__ __forceinline__ double finite_or(double nul, double x) {
   return (__double2hiint(x) & 0x7ff00000) == 0x7ff00000 ? __longlong_as_double(0x7ff8000000000000ll) : nul;
+}
+// Whether two numbers are equal (FP64: have the same bits, so 0 and -0 differ).
+__device__ __forceinline__ bool equal_values(float a, float b) { return a == b; }
+__device__ __forceinline__ bool equal_values(double a, double b) {
+  return __double_as_longlong(a) == __double_as_longlong(b);
 }
 // Whether two numbers have the same bits.
 __device__ __forceinline__ bool same_bits(float a, float b) { return __float_as_int(a) == __float_as_int(b); }
@@ -524,22 +529,87 @@ __device__ __forceinline__ void riemann_hllc(const T* WL, const T* WR, T* F, con
 // ---------------------------------------------------------------------------
 // Exact Riemann solver (Toro 2009 ch. 4).
 // ---------------------------------------------------------------------------
-// One side's pressure function f_K(p) and its derivative: shock branch
-// (p > p_K) with A = 2/((g+1) rho_K), B = (g-1)/(g+1) p_K; rarefaction
-// branch (p <= p_K) from the isentrope.
+// y^n, n in 4 .. 8 (the same n in all threads).
 template <typename T>
-__device__ __forceinline__ void press_fn(T p, T rK, T pK, T cK, const Gas<T>& gas, T& f, T& df) {
-  if (p > pK) {
-    const T A = qdiv(gas.A2, rK), B = gas.Bq * pK;
-    const T q = dsqrt(qdiv(A, B + p));
-    f = (p - pK) * q;
-    df = q * (T(1) - T(0.5) * qdiv(p - pK, B + p));
+__device__ __forceinline__ T power_n(T y, int n) {
+  const T y2 = y * y, y4 = y2 * y2;
+  if (n == 8) return y4 * y4;
+  T w = y4;
+  if (n & 2) w *= y2;
+  if (n & 1) w *= y;
+  return w;
+}
+// One third-order (Halley) step for y^n = x from y with relative error e:
+// y + 2 y (x - y^n)/((n + 1) y^n + (n - 1) x), error ~ n^2/12 e^3.  The
+// quotient is a correction of relative size e, so it needs only its leading
+// digits: its divisor's reciprocal is refined once (FP64).
+__device__ __forceinline__ float root_step(float y, float x, int n) {
+  const float w = power_n(y, n);
+  return fmaf(y * (x - w), __fdividef(1.0f, 0.5f * (n + 1) * w + 0.5f * (n - 1) * x), y);
+}
+__device__ __forceinline__ double root_step(double y, double x, int n) {
+  const double w = power_n(y, n), den = fma(0.5 * (n + 1), w, 0.5 * (n - 1) * x);
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(den));
+  r = fma(r, fma(-den, r, 1.0), r);
+  return fma(y * (x - w), r, y);
+}
+// x^z, z = (gamma - 1)/(2 gamma), x > 0 a ratio of pressures.  For the usual
+// gammas 1/z is a small integer and x^z a root: a hardware estimate (relative
+// error ~1e-6) and one root_step, correct to about 1 ulp -- 10 FP64
+// operations, against the ~43 of exp2(z log2 x), whose FP32 form is also
+// twice as long and less exact.
+__device__ __forceinline__ float pow_z(float x, const Gas<float>& gas) {
+  if (gas.root == 0) return dpow<float>(x, gas.z);
+  float t;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(__log2f(x) * gas.z));
+  return root_step(t, x, gas.root);
+}
+__device__ __forceinline__ double pow_z(double x, const Gas<double>& gas) {
+  if (gas.root == 0) return dpow<double>(x, gas.z);
+  // log2 x from its exponent and leading 23 bits; 2^t scaled back by the exponent
+  const int hx = __double2hiint(x), lx = __double2loint(x);
+  const float m = __int_as_float(0x3f800000 | ((hx & 0xfffff) << 3) | (int)((unsigned)lx >> 29));
+  const float t = ((float)((hx >> 20) - 1023) + __log2f(m)) * (float)gas.z, ti = rintf(t);
+  float f;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(t - ti));
+  double y = (double)f;
+  y = __hiloint2double(__double2hiint(y) + ((int)ti << 20), __double2loint(y));
+  return root_step(y, x, gas.root);
+}
+// x^(1/z)
+template <typename T>
+__device__ __forceinline__ T pow_iz(T x, const Gas<T>& gas) {
+  return gas.root ? power_n(x, gas.root) : dpow<T>(x, gas.iz);
+}
+
+// What the pressure function of one side needs at every iterate.
+template <typename T>
+struct PressSide {
+  T p, ip;   // p_K and its reciprocal
+  T A, B;    // 2/((g+1) rho_K), (g-1)/(g+1) p_K
+  T f0, irc;  // 2 c_K/(g-1), 1/(rho_K c_K) = c_K/(g p_K)
+  __device__ __forceinline__ PressSide(T rK, T pK, T cK, const Gas<T>& gas)
+      : p(pK), ip(rcp<T>(pK)), A(qdiv(gas.A2, rK)), B(gas.Bq * pK), f0(gas.two_gm1 * cK) {
+    irc = cK * ip * gas.ig;
+  }
+};
+
+// One side's pressure function f_K(p) and its derivative: shock branch
+// (p > p_K) with A and B; rarefaction branch (p <= p_K) from the isentrope.
+// (rp = 1/p)
+template <typename T>
+__device__ __forceinline__ void press_fn(T p, T rp, const PressSide<T>& k, const Gas<T>& gas, T& f, T& df) {
+  if (p > k.p) {
+    const T d = p - k.p, r = rcp<T>(p + k.B);
+    const T q = dsqrt(k.A * r);
+    f = d * q;
+    df = q * (T(1) - T(0.5) * (d * r));
   } else {
-    const T pr = qdiv(p, pK);
-    const T pz = dpow(pr, gas.z);  // (p/pK)^((g-1)/(2g))
-    f = gas.two_gm1 * cK * (pz - T(1));
+    const T pz = pow_z(p * k.ip, gas);  // (p/pK)^((g-1)/(2g))
+    f = k.f0 * (pz - T(1));
     // (p/pK)^(-(g+1)/(2g)) = (p/pK)^z / (p/pK)
-    df = qdiv(pz, pr * rK * cK);
+    df = pz * (k.p * rp) * k.irc;
   }
 }
 
@@ -550,17 +620,18 @@ template <typename T>
 __device__ __forceinline__ T toro_guess(T rL, T uL, T pL, T cL, T rR, T uR, T pR, T cR,
                                         const Gas<T>& gas, int& kind) {
   T ppv = T(0.5) * (pL + pR) - T(0.125) * (uR - uL) * (rL + rR) * (cL + cR);
-  ppv = fmax(ppv, T(0));
-  const T pmin = fmin(pL, pR), pmax = fmax(pL, pR);
-  if (qdiv(pmax, pmin) <= T(2) && ppv >= pmin && ppv <= pmax) {
+  ppv = is_pos(ppv) ? ppv : T(0);
+  const T pmin = min_of(pL, pR), pmax = max_of(pL, pR);
+  if (pmax <= T(2) * pmin && ppv >= pmin && ppv <= pmax) {
     kind = 0;
     return ppv;
   }
   if (ppv < pmin) {
     kind = 1;
+    // p_L (num/(c_L + c_R (p_L/p_R)^z))^(1/z)
     const T num = cL + cR - T(0.5) * gas.gm1 * (uR - uL);
-    const T den = qdiv(cL, dpow(pL, gas.z)) + qdiv(cR, dpow(pR, gas.z));
-    return dpow(qdiv(num, den), gas.iz);
+    const T den = cL + cR * pow_z(qdiv(pL, pR), gas);
+    return pL * pow_iz(qdiv(num, den), gas);
   }
   kind = 2;
   const T gL = dsqrt(qdiv(qdiv(gas.A2, rL), ppv + gas.Bq * pL));
@@ -579,44 +650,40 @@ __device__ __forceinline__ T toro_guess(T rL, T uL, T pL, T cL, T rR, T uR, T pR
 // rounding of f_L + f_R + du then decides the step, and no later iterate is
 // better determined (near vacuum, where the two rarefaction terms nearly
 // cancel du, the 1e-6 change is never reached).
+// The last step's change dp is below that tolerance (or within the residual's
+// rounding), so f at its iterate is f + f' dp to O(dp^2), below the rounding of
+// f: the star velocity takes that instead of a further evaluation.
 template <typename T>
 __device__ __forceinline__ int newton_star(T p, T rL, T uL, T pL, T cL, T rR, T uR, T pR, T cR,
                                            const Gas<T>& gas, T tol, T& ps, T& us, int& iters) {
   const T du = uR - uL;
   const T pfloor = T(1e-14) * T(0.5) * (pL + pR);
   if (!(p > pfloor)) p = pfloor;
-  // One evaluation site for the pressure functions (the iterates and the
-  // final p): the solver's code stays short.
-  bool conv = false, fin = false;
-  int it = 0;
-  T fL, dfL, fR, dfR;
-  for (;;) {
-    press_fn(p, rL, pL, cL, gas, fL, dfL);
-    press_fn(p, rR, pR, cR, gas, fR, dfR);
-    if (fin || it >= 100) break;  // f at the final p (or the iteration limit)
+  const PressSide<T> L(rL, pL, cL, gas), R(rR, pR, cR, gas);
+  bool conv = false;
+  for (int it = 1; it <= 100; ++it) {
+    T fL, dfL, fR, dfR;
+    const T rp = rcp<T>(p);
+    press_fn(p, rp, L, gas, fL, dfL);
+    press_fn(p, rp, R, gas, fR, dfR);
     const T res = fL + fR + du;
     T pn = p - qdiv(res, dfL + dfR);
     if (pn < T(0)) pn = pfloor;
-    ++it;
-    const T ch = qdiv(T(2) * fabs(pn - p), pn + p);
+    const T dp = pn - p;
+    const bool small = T(2) * fabs(dp) < tol * (pn + p);
     p = pn;
-    if (conv) {
-      fin = true;  // the extra step after convergence is done
-      continue;
+    // FP64 takes one more step after convergence, FP32 after the residual's rule only
+    if (conv || (sizeof(T) == 4 && small)) {
+      iters = it;
+      ps = p;
+      us = T(0.5) * (uL + uR) + T(0.5) * ((fR + dfR * dp) - (fL + dfL * dp));
+      return ST_OK;
     }
-    if (ch < tol) {
-      conv = true;
-      if constexpr (sizeof(T) == 4) fin = true;  // FP32: this step was the last
-    }
-    if constexpr (sizeof(T) == 4) {
-      if (fabs(res) <= T(8 * 1.1920929e-7) * (fabs(fL) + fabs(fR) + fabs(du))) conv = true;
-    }
+    conv = small;
+    if constexpr (sizeof(T) == 4) conv = fabs(res) <= T(8 * 1.1920929e-7) * (fabs(fL) + fabs(fR) + fabs(du));
   }
-  iters = it;
-  if (!conv) return ST_NEWTON;
-  ps = p;
-  us = T(0.5) * (uL + uR) + T(0.5) * (fR - fL);
-  return ST_OK;
+  iters = 100;
+  return ST_NEWTON;
 }
 
 // A primitive 1D state returned by value (a local whose address an
@@ -626,81 +693,57 @@ struct Prim3 {
   T rho, u, p;
 };
 
-// The state inside a rarefaction fan at x/t = S (Toro ch. 4.5): sign = +1
-// for the left fan (c = 2/(g+1) (cK + (g-1)/2 (uK - S)), u = c + S), -1 for
-// the right one (c = 2/(g+1) (cK - (g-1)/2 (uK - S)), u = S - c); rho and P
-// from the isentrope through (rK, pK).  Out of line: x/t = S lies inside a
-// fan only near sonic points, and the hot solver code stays shorter.
+// The state inside a left rarefaction fan at x/t = S (Toro ch. 4.5): c =
+// 2/(g+1) (cK + (g-1)/2 (uK - S)), u = S + c; rho and P from the isentrope
+// through (rK, pK).  Out of line: x/t = S lies inside a fan only near sonic
+// points, and the hot solver code stays shorter.
 template <typename T>
-static __device__ __noinline__ Prim3<T> fan_state(T S, T sign, T rK, T uK, T pK, T cK, Gas<T> gas) {
-  const T c = gas.A2 * (cK + sign * T(0.5) * gas.gm1 * (uK - S));
+static __device__ __noinline__ Prim3<T> fan_state(T S, T rK, T uK, T pK, T cK, Gas<T> gas) {
+  const T c = gas.A2 * (cK + T(0.5) * gas.gm1 * (uK - S));
+  const T x = qdiv(c, cK), t = dpow(x, gas.two_gm1);
   Prim3<T> w;
-  w.u = S + sign * c;
-  w.rho = rK * dpow(qdiv(c, cK), gas.two_gm1);
-  w.p = pK * dpow(qdiv(c, cK), gas.pow_c);
+  w.u = S + c;
+  w.rho = rK * t;
+  w.p = pK * (t * x * x);  // 2g/(g-1) = 2/(g-1) + 2
   return w;
 }
 
 // Sample the exact solution at x/t = S given the star state (Toro ch. 4.5);
 // returns the (rho, u, P) there and whether it lies left of the contact
-// (ties left).
+// (ties left).  A point right of the contact is sampled as the mirror image,
+// so that both sides run the same code.
 template <typename T>
 __device__ __forceinline__ bool sample_xi(T S, T rL, T uL, T pL, T cL, T rR, T uR, T pR, T cR, T ps,
                                           T us, const Gas<T>& gas, T& rho, T& u, T& p) {
-  if (S <= us) {
-    if (ps > pL) {
-      const T SL = uL - cL * dsqrt(gas.zp * qdiv(ps, pL) + gas.z);
-      if (S <= SL) { rho = rL; u = uL; p = pL; }
-      else {
-        const T q = qdiv(ps, pL);
-        rho = qdiv(rL * (q + gas.Bq), gas.Bq * q + T(1));
-        u = us; p = ps;
-      }
-    } else {
-      const T SHL = uL - cL;
-      const T cs = cL * dpow(qdiv(ps, pL), gas.z);
-      const T STL = us - cs;
-      if (S <= SHL) { rho = rL; u = uL; p = pL; }
-      else if (S >= STL) {
-        rho = rL * dpow(qdiv(ps, pL), gas.ig);
-        u = us; p = ps;
-      } else {
-        {
-          const Prim3<T> f = fan_state<T>(S, T(1), rL, uL, pL, cL, gas);
-          rho = f.rho;
-          u = f.u;
-          p = f.p;
-        }  // inside the left fan
-      }
+  const bool left = S <= us;
+  const T rK = left ? rL : rR, uK = left ? uL : -uR, pK = left ? pL : pR, cK = left ? cL : cR;
+  const T x = left ? S : -S, um = left ? us : -us;
+  const T q = qdiv(ps, pK);
+  rho = rK;
+  u = uK;
+  p = pK;
+  if (ps > pK) {
+    const T SK = uK - cK * dsqrt(gas.zp * q + gas.z);
+    if (x > SK) {
+      rho = qdiv(rK * (q + gas.Bq), gas.Bq * q + T(1));
+      u = um;
+      p = ps;
     }
-    return true;
-  }
-  if (ps > pR) {
-    const T SR = uR + cR * dsqrt(gas.zp * qdiv(ps, pR) + gas.z);
-    if (S >= SR) { rho = rR; u = uR; p = pR; }
-    else {
-      const T q = qdiv(ps, pR);
-      rho = qdiv(rR * (q + gas.Bq), gas.Bq * q + T(1));
-      u = us; p = ps;
-    }
-  } else {
-    const T SHR = uR + cR;
-    const T cs = cR * dpow(qdiv(ps, pR), gas.z);
-    const T STR = us + cs;
-    if (S >= SHR) { rho = rR; u = uR; p = pR; }
-    else if (S <= STR) {
-      rho = rR * dpow(qdiv(ps, pR), gas.ig);
-      u = us; p = ps;
+  } else if (x > uK - cK) {
+    const T pz = pow_z(q, gas);  // c*/c_K
+    if (x >= um - cK * pz) {
+      rho = qdiv(rK * q, pz * pz);  // q^(1/g) = q^(1 - 2z)
+      u = um;
+      p = ps;
     } else {
-      {
-          const Prim3<T> f = fan_state<T>(S, T(-1), rR, uR, pR, cR, gas);
-          rho = f.rho;
-          u = f.u;
-          p = f.p;
-        }  // inside the right fan
+      const Prim3<T> f = fan_state<T>(x, rK, uK, pK, cK, gas);
+      rho = f.rho;
+      u = f.u;
+      p = f.p;
     }
   }
-  return false;
+  if (!left) u = -u;
+  return left;
 }
 
 // The same at x/t = 0, the value the Godunov flux needs.
@@ -723,7 +766,7 @@ __device__ __forceinline__ Gas<double> gas_double(const Gas<float>& g) {
   d.g = gg; d.gm1 = gg - 1.0; d.igm1 = 1.0 / (gg - 1.0); d.z = (gg - 1.0) / (2.0 * gg);
   d.iz = 1.0 / d.z; d.zp = (gg + 1.0) / (2.0 * gg); d.A2 = 2.0 / (gg + 1.0);
   d.Bq = (gg - 1.0) / (gg + 1.0); d.two_gm1 = 2.0 / (gg - 1.0); d.ig = 1.0 / gg;
-  d.pow_c = 2.0 * gg / (gg - 1.0);
+  d.root = 0;  // (of the FP32 gamma, 1/z is no integer)
   return d;
 }
 
@@ -756,7 +799,7 @@ static __device__ __noinline__ Star32 newton_star_fp64(float p0, float rL, float
 // the cancellation of the two rarefaction terms against du.
 template <typename T>
 __device__ __forceinline__ bool hard_face(T pL, T pR, T du, T vac) {
-  return qdiv(fmax(pL, pR), fmin(pL, pR)) > T(1e6) || vac - du < T(0.2) * vac;
+  return max_of(pL, pR) > T(1e6) * min_of(pL, pR) || vac - du < T(0.2) * vac;
 }
 
 // Star state from a given initial guess p0 and the sound speeds cL, cR of
@@ -799,7 +842,7 @@ __device__ __forceinline__ int riemann_exact(const T* WL, const T* WR, T* F, con
   // the sample is the state) -- take it directly.
   bool same = true;
 #pragma unroll
-  for (int v = 0; v < NV; ++v) same = same && WL[v] == WR[v];
+  for (int v = 0; v < NV; ++v) same = same && equal_values(WL[v], WR[v]);
   if (same) {
     iters = 0;
     kind = 0;
@@ -858,7 +901,7 @@ __device__ __forceinline__ int riemann_exact_from(const T* WL, const T* WR, T cL
 constexpr double MLP_GATE_RATIO = 4.0;
 template <typename T>
 __device__ __forceinline__ bool mlp_gate(int kind, T pL, T pR) {
-  return kind == 2 && fmax(pL, pR) > T(MLP_GATE_RATIO) * fmin(pL, pR);
+  return kind == 2 && max_of(pL, pR) > T(MLP_GATE_RATIO) * min_of(pL, pR);
 }
 
 constexpr int MLP_IN = 6, MLP_H = 64;
