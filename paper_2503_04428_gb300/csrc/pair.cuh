@@ -42,18 +42,8 @@ __device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
   return r;
 }
-// Reciprocal and square root by the hardware approximations (1-2 ulp).
-__device__ __forceinline__ float rcp_fast(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-__device__ __forceinline__ float rsqrt_fast(float x) {
-  float r;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-__device__ __forceinline__ f2 rcp2(f2 a) { return make_f2(rcp_fast(lo(a)), rcp_fast(hi(a))); }
+// Reciprocal and reciprocal square root by the hardware approximations (1-2 ulp).
+__device__ __forceinline__ f2 rcp2(f2 a) { return make_f2(rcp<float>(lo(a)), rcp<float>(hi(a))); }
 __device__ __forceinline__ f2 rsqrt2(f2 a) { return make_f2(rsqrt_fast(lo(a)), rsqrt_fast(hi(a))); }
 __device__ __forceinline__ f2 minmod2(f2 a, f2 b) { return make_f2(minmod(lo(a), lo(b)), minmod(hi(a), hi(b))); }
 __device__ __forceinline__ f2 limit2(int kind, f2 a, f2 b) {

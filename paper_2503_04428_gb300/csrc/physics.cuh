@@ -48,9 +48,18 @@ struct Gas {
 // relative error is below 2^-18: 3 and 5 FP64 operations against 4.5 and 7.5
 // of the correctly rounded ones, with errors of about 1 ulp.
 
-// 1/x (FP32: the fast 2-ulp form; FP64: x normal, |x| < 2^1021).
+// FP32 takes the hardware approximations (1-2 ulp; the FP32 bulk's rounding
+// error is ~1e-7 per operation either way) in their .ftz forms: the others
+// guard subnormal arguments with four more instructions each, a fifth of the
+// exact solver's stream.
+
+// 1/x (x normal; FP32: |x| < 2^126, FP64: |x| < 2^1021).
 template <typename T> __device__ __forceinline__ T rcp(T x);
-template <> __device__ __forceinline__ float rcp<float>(float x) { return __fdividef(1.0f, x); }
+template <> __device__ __forceinline__ float rcp<float>(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
 template <> __device__ __forceinline__ double rcp<double>(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
@@ -61,9 +70,15 @@ template <> __device__ __forceinline__ double rcp<double>(double x) {
 
 // Square roots of positive x.  The FP32 bulk takes x rsqrt(x) (about 3 ulp):
 // the correctly rounded sqrtf sequence cost 2-3 % of the FP32 step's
-// instructions.
+// instructions.  rsqrt_fast: 1/sqrt(x), of the smallest normal number if x is
+// less, so that every x >= 0 has a finite root x rsqrt_fast(x).
+__device__ __forceinline__ float rsqrt_fast(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fmaxf(x, 1.17549435e-38f)));
+  return r;
+}
 template <typename T> __device__ __forceinline__ T dsqrt(T x);
-template <> __device__ __forceinline__ float dsqrt<float>(float x) { return x * rsqrtf(x); }
+template <> __device__ __forceinline__ float dsqrt<float>(float x) { return x * rsqrt_fast(x); }
 template <> __device__ __forceinline__ double dsqrt<double>(double x) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
@@ -100,15 +115,42 @@ template <> __device__ __forceinline__ float dpow<float>(float x, float y) { ret
 
 // Quotient of the state conversions, wave speeds and the exact solver
 // (pressure functions, guess, Newton step, sampling): a times the reciprocal
-// above (FP32: the fast 2-ulp division; the FP32 bulk's rounding error is
-// ~1e-7 per operation either way, and Newton corrects its own iterates).
-// FP64: b normal, |b| < 2^1021; 4 FP64 operations against 7.5.
+// above (Newton corrects its own iterates).  FP64: 4 operations against 7.5.
 template <typename T> __device__ __forceinline__ T qdiv(T a, T b) { return a * rcp<T>(b); }
-template <> __device__ __forceinline__ float qdiv<float>(float a, float b) { return __fdividef(a, b); }
 
 template <typename T> __device__ __forceinline__ T temp_tol();
 template <> __device__ __forceinline__ double temp_tol<double>() { return 1e-13; }
 template <> __device__ __forceinline__ float temp_tol<float>() { return 1e-6f; }
+
+// A temperature and the Newton iterations it took.
+template <typename T>
+struct TempIts {
+  T t;
+  int its;
+};
+// The solve of GasRad::temperature.  Out of line: a step has 15 sites of it,
+// and inlined they overflowed the instruction cache (1.8 stalls per issue).
+template <typename T>
+static __device__ __noinline__ TempIts<T> newton_temperature(T c1, T c4, T y, T t0) {
+  T t = qdiv(y, c1);
+  if (!is_pos(y)) return {t, 0};
+  if (t0 > T(0)) t = t0;
+  else if (c4 > T(0)) t = min_of(t, dsqrt(dsqrt(qdiv(y, c4))));
+  bool conv = false;
+  int it = 0;
+  for (; it < 60; ++it) {
+    const T t3 = t * t * t;
+    const T tn = t - qdiv(c1 * t + c4 * t3 * t - y, c1 + T(4) * c4 * t3);
+    const T ch = fabs(tn - t);
+    t = tn;
+    if (conv) break;
+    if (ch < temp_tol<T>() * tn) {
+      if constexpr (sizeof(T) == 4) break;  // FP32: this step was the last
+      conv = true;
+    }
+  }
+  return {t, it < 60 ? it + 1 : 60};
+}
 
 // Ideal gas in equilibrium with radiation, Eq. 6-7: e = rho R T/(gamma-1) +
 // a T^4, P = rho R T + a T^4/3 with R = k_b/(mu m_u), and the sound speed of
@@ -134,25 +176,9 @@ struct GasRad : Gas<T> {
   // y/c1 <= 0, which the positivity checks reject.
   // (its, if given, accumulates the Newton iterations taken.)
   __device__ __forceinline__ T temperature(T c1, T c4, T y, T t0 = T(0), int* its = nullptr) const {
-    T t = qdiv(y, c1);
-    if (!(y > T(0))) return t;
-    if (t0 > T(0)) t = t0;
-    else if (c4 > T(0)) t = fmin(t, dsqrt(dsqrt(qdiv(y, c4))));
-    bool conv = false;
-    int it = 0;
-    for (; it < 60; ++it) {
-      const T t3 = t * t * t;
-      const T tn = t - qdiv(c1 * t + c4 * t3 * t - y, c1 + T(4) * c4 * t3);
-      const T ch = qdiv(fabs(tn - t), tn);
-      t = tn;
-      if (conv) break;
-      if (ch < temp_tol<T>()) {
-        if constexpr (sizeof(T) == 4) break;  // FP32: this step was the last
-        conv = true;
-      }
-    }
-    if (its) *its += it < 60 ? it + 1 : 60;
-    return t;
+    const TempIts<T> r = newton_temperature<T>(c1, c4, y, t0);
+    if (its) *its += r.its;
+    return r.t;
   }
   // Eq. 7 from the gas and radiation pressures
   __device__ __forceinline__ T sound2(T rho, T pg, T pr) const {
@@ -375,20 +401,31 @@ __device__ __forceinline__ double minmod(double dm, double dp) {
   const double m = bm < bp ? dm : dp;
   return (__double2hiint(dm) ^ __double2hiint(dp)) < 0 ? 0.0 : m;
 }
-// The product of two slopes is taken as positive from here on (FP64: the
-// quotients below need a normal divisor; slopes of less than ~1e-145 do not
-// matter).
-__device__ __forceinline__ bool slopes_agree(float pr) { return pr > 0.0f; }
-__device__ __forceinline__ bool slopes_agree(double pr) { return __double2hiint(pr) > 0x01d00000; }  // > 2^-994
+// van Leer's 2ab/(a+b) and van Albada's ab(a+b)/(a^2+b^2) where the signs
+// agree.  FP32: through the ratio s of the smaller to the larger magnitude,
+// so that no product of two small slopes underflows (densities of 1e-24 have
+// slopes of that size); magnitudes below 2^-125 give 0.
+__device__ __forceinline__ float smooth_limit(bool vanleer, float dm, float dp) {
+  const float m = fmaxf(fabsf(dm), fabsf(dp)), n = fminf(fabsf(dm), fabsf(dp));
+  if ((__float_as_int(dm) ^ __float_as_int(dp)) < 0 || !(m > 2.4e-38f)) return 0.0f;
+  const float s = n * rcp<float>(m);
+  const float r = vanleer ? (n + n) * rcp<float>(1.0f + s) : n * (1.0f + s) * rcp<float>(1.0f + s * s);
+  return __int_as_float(__float_as_int(r) | (__float_as_int(dm) & 0x80000000));
+}
+// (FP64: the product as the sign test; the quotients need a normal divisor,
+// and slopes of less than ~1e-149 do not matter.)
+__device__ __forceinline__ double smooth_limit(bool vanleer, double dm, double dp) {
+  const double pr = dm * dp;
+  if (__double2hiint(pr) <= 0x01d00000) return 0.0;  // 2^-994
+  return vanleer ? qdiv(2.0 * pr, dm + dp) : qdiv(pr * (dm + dp), dm * dm + dp * dp);
+}
 
 // Homogeneous of degree 1: limit(k, s a, s b) = s limit(k, a, b) for s > 0.
 template <typename T>
 __device__ __forceinline__ T limit(int kind, T dm, T dp) {
   if (kind == LIM_MINMOD) return minmod(dm, dp);
-  const T pr = dm * dp;
-  if (kind == LIM_FIRST || !slopes_agree(pr)) return T(0);
-  if (kind == LIM_VANLEER) return qdiv(T(2) * pr, dm + dp);
-  return qdiv(pr * (dm + dp), dm * dm + dp * dp);
+  if (kind == LIM_FIRST) return T(0);
+  return smooth_limit(kind == LIM_VANLEER, dm, dp);
 }
 
 // ---------------------------------------------------------------------------
@@ -545,7 +582,7 @@ __device__ __forceinline__ T power_n(T y, int n) {
 // digits: its divisor's reciprocal is refined once (FP64).
 __device__ __forceinline__ float root_step(float y, float x, int n) {
   const float w = power_n(y, n);
-  return fmaf(y * (x - w), __fdividef(1.0f, 0.5f * (n + 1) * w + 0.5f * (n - 1) * x), y);
+  return fmaf(y * (x - w), rcp<float>(0.5f * (n + 1) * w + 0.5f * (n - 1) * x), y);
 }
 __device__ __forceinline__ double root_step(double y, double x, int n) {
   const double w = power_n(y, n), den = fma(0.5 * (n + 1), w, 0.5 * (n - 1) * x);
