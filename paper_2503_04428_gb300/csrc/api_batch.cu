@@ -39,6 +39,7 @@ struct BatchState {
   unsigned int* tcnt = nullptr;
   double* t_tube = nullptr;
   double* t_prev = nullptr;
+  void* kept = nullptr;  // 5 x ntubes words: the bookkeeping a state being set would replace
   BatchCtrl* bctrl = nullptr;
   BatchCtrl* bctrl_host = nullptr;
   // launch shape: warps per CTA, cells per item, CTAs
@@ -385,8 +386,7 @@ static int autotune_batch(hydro_ctx* h, double cfl) {
 template <typename T>
 static int batch_init(hydro_ctx* h, int slot, int* status) {
   BatchState* bs = h->bs;
-  int* d_status = nullptr;
-  HCK(cudaMalloc(&d_status, sizeof(int)));
+  int* const d_status = (int*)h->word;
   HCK(cudaMemsetAsync(d_status, 0, sizeof(int), h->stream));
   batch_init_kernel<T><<<bs->ntubes, 256, 0, h->stream>>>((const T*)h->buf[slot], bs->stride, bs->off_d, 0,
                                                            bs->ntubes, make_gas<T>(h->gamma), &bs->bctrl->c,
@@ -394,9 +394,9 @@ static int batch_init(hydro_ctx* h, int slot, int* status) {
                                                            reinterpret_cast<int*>(bs->tcnt + bs->ntubes),
                                                            bs->t_tube, bs->t_prev, d_status);
   HCK(cudaGetLastError());
-  HCK(cudaMemcpyAsync(status, d_status, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  HCK(cudaMemcpyAsync(h->word_host, d_status, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   HCK(cudaStreamSynchronize(h->stream));
-  cudaFree(d_status);
+  std::memcpy(status, h->word_host, sizeof(int));
   return HYDRO_OK;
 }
 
@@ -493,26 +493,21 @@ int hydro_batch_set_state_impl(hydro_ctx* h, const void* U, int where) {
   HCK(cudaMemcpy2DAsync(h->buf[slot], (size_t)bs->stride * h->esize, U, (size_t)bs->total * h->esize,
                         (size_t)bs->total * h->esize, 3,
                         where == HYDRO_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->stream));
-  // the speeds of the new state go to the slots of the current step count
-  // (the rest of the bookkeeping is written only if the state is valid)
-  std::vector<unsigned long long> keep_smax(3 * (size_t)bs->ntubes);
-  std::vector<double> keep_t(2 * (size_t)bs->ntubes);
-  HCK(cudaMemcpyAsync(keep_smax.data(), bs->smax, sizeof(unsigned long long) * 3 * bs->ntubes,
-                      cudaMemcpyDeviceToHost, h->stream));
-  HCK(cudaMemcpyAsync(keep_t.data(), bs->t_tube, sizeof(double) * bs->ntubes, cudaMemcpyDeviceToHost, h->stream));
-  HCK(cudaMemcpyAsync(keep_t.data() + bs->ntubes, bs->t_prev, sizeof(double) * bs->ntubes, cudaMemcpyDeviceToHost,
-                      h->stream));
+  // the bookkeeping of the new state replaces the current one, which is kept
+  // (speeds, then times, on the device) until the state has proved valid
+  const size_t n = (size_t)bs->ntubes, word = sizeof(double);
+  unsigned char* const kept = (unsigned char*)bs->kept;
+  HCK(cudaMemcpyAsync(kept, bs->smax, 3 * n * word, cudaMemcpyDeviceToDevice, h->stream));
+  HCK(cudaMemcpyAsync(kept + 3 * n * word, bs->t_tube, n * word, cudaMemcpyDeviceToDevice, h->stream));
+  HCK(cudaMemcpyAsync(kept + 4 * n * word, bs->t_prev, n * word, cudaMemcpyDeviceToDevice, h->stream));
   int status = 0;
   st = h->precision == 64 ? batch_init<double>(h, slot, &status) : batch_init<float>(h, slot, &status);
   if (st) return st;
   if (status) {
     // the previous state and its bookkeeping stay
-    HCK(cudaMemcpyAsync(bs->smax, keep_smax.data(), sizeof(unsigned long long) * 3 * bs->ntubes,
-                        cudaMemcpyHostToDevice, h->stream));
-    HCK(cudaMemcpyAsync(bs->t_tube, keep_t.data(), sizeof(double) * bs->ntubes, cudaMemcpyHostToDevice,
-                        h->stream));
-    HCK(cudaMemcpyAsync(bs->t_prev, keep_t.data() + bs->ntubes, sizeof(double) * bs->ntubes,
-                        cudaMemcpyHostToDevice, h->stream));
+    HCK(cudaMemcpyAsync(bs->smax, kept, 3 * n * word, cudaMemcpyDeviceToDevice, h->stream));
+    HCK(cudaMemcpyAsync(bs->t_tube, kept + 3 * n * word, n * word, cudaMemcpyDeviceToDevice, h->stream));
+    HCK(cudaMemcpyAsync(bs->t_prev, kept + 4 * n * word, n * word, cudaMemcpyDeviceToDevice, h->stream));
     HCK(cudaStreamSynchronize(h->stream));
     set_error(status == HYDRO_ERR_NONFINITE ? "hydro_set_state: non-finite value in the state"
                                             : "hydro_set_state: density or pressure not positive");
@@ -575,6 +570,7 @@ void hydro_batch_free_impl(hydro_ctx* h) {
   cudaFree(bs->tcnt);
   cudaFree(bs->t_tube);
   cudaFree(bs->t_prev);
+  cudaFree(bs->kept);
   cudaFree(bs->bctrl);
   cudaFreeHost(bs->bctrl_host);
   cudaFree(bs->items);
@@ -844,6 +840,7 @@ int hydro_batch_create(const int* lengths, int ntubes, const hydro_eos* eos, int
       cudaMalloc(&bs->tcnt, sizeof(unsigned int) * 2 * ntubes) != cudaSuccess ||
       cudaMalloc(&bs->t_tube, sizeof(double) * ntubes) != cudaSuccess ||
       cudaMalloc(&bs->t_prev, sizeof(double) * ntubes) != cudaSuccess ||
+      cudaMalloc(&bs->kept, sizeof(double) * 5 * ntubes) != cudaSuccess ||
       cudaMalloc(&bs->bctrl, sizeof(BatchCtrl)) != cudaSuccess ||
       cudaMallocHost(&bs->bctrl_host, sizeof(BatchCtrl)) != cudaSuccess) {
     set_error("hydro_batch_create: device allocation failed");

@@ -441,6 +441,7 @@ static cudaError_t plain_step(const SweepArgs<float>& a, int nsx, int rs, cudaSt
 
 template <typename T>
 static int launch_step_t(hydro_ctx* h, double dt_host, double cfl, double t_end, Ctrl* ctrl) {
+  h->ctrl_fresh = false;
   if (h->gravity == GRAV_MONO) {
     dim3 gb((h->n[0] + 31) / 32, h->shell_nchunks), tb(32, 8);
     shell_partial_kernel<T><<<gb, tb, 0, h->stream>>>(ctrl, (const T*)h->buf[0], (const T*)h->buf[1],
@@ -517,6 +518,7 @@ static int launch_steps_t(hydro_ctx* h, int nsteps, double cfl, double t_end, bo
     if (st) return st;
   }
   sa.speed = (unsigned long long*)h->steps_speed;
+  h->ctrl_fresh = false;
   for (int left = nsteps; left > 0; left -= sa.nsteps) {
     sa.nsteps = std::min(left, 4096);  // (a launch of tens of milliseconds at most)
     HCK(cudaMemsetAsync(sa.speed, 0, words, h->stream));
@@ -528,12 +530,25 @@ static int launch_steps_t(hydro_ctx* h, int nsteps, double cfl, double t_end, bo
 static int read_ctrl(hydro_ctx* h) {
   HCK(cudaMemcpyAsync(h->ctrl_host, h->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->stream));
   HCK(cudaStreamSynchronize(h->stream));
+  h->ctrl_fresh = true;
   return HYDRO_OK;
 }
 
+// The mirror, read only if a launch may have changed the control block since:
+// a grid's entry points that launch read it before they return, so a caller's
+// cfl_dt + step loop needs one round trip per step, not two (10 us each). A
+// stream under capture takes the read, which fails as every other entry point.
+static int sync_ctrl(hydro_ctx* h) {
+  cudaStreamCaptureStatus cap;
+  if (h->ctrl_fresh && cudaStreamIsCapturing(h->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone)
+    return HYDRO_OK;
+  return read_ctrl(h);
+}
+
+// The mirror to the device, in stream order (pinned memory: not waited for;
+// whatever changes the mirror again is written again or comes after a read).
 static int write_ctrl(hydro_ctx* h) {
   HCK(cudaMemcpyAsync(h->ctrl, h->ctrl_host, sizeof(Ctrl), cudaMemcpyHostToDevice, h->stream));
-  HCK(cudaStreamSynchronize(h->stream));
   return HYDRO_OK;
 }
 
@@ -598,11 +613,9 @@ std::string device_key() {
 
 template <typename T>
 static int validate_into(hydro_ctx* h, int slot, int* status_out, double* smax_out) {
-  int* d_status = nullptr;
-  unsigned long long* d_smax = nullptr;
-  HCK(cudaMalloc(&d_status, sizeof(int) + sizeof(unsigned long long) + 8));
-  d_smax = (unsigned long long*)(d_status + 2);
-  HCK(cudaMemsetAsync(d_status, 0, sizeof(int) + sizeof(unsigned long long) + 8, h->stream));
+  int* const d_status = (int*)h->word;
+  unsigned long long* const d_smax = h->word + 1;
+  HCK(cudaMemsetAsync(h->word, 0, 2 * sizeof(unsigned long long), h->stream));
   const int blocks = (int)std::max<long long>(1, std::min<long long>((h->ncell + 255) / 256, (long long)h->num_sms * 8));
   const Gas<T> gas = make_gas<T>(h->gamma);
   const GasRad<T> grad = make_gas_rad<T>(h->gamma, h->R_gas, h->a_rad);
@@ -629,16 +642,10 @@ static int validate_into(hydro_ctx* h, int slot, int* status_out, double* smax_o
     }
   }
   HCK(cudaGetLastError());
-  int hs[4];
-  HCK(cudaMemcpyAsync(hs, d_status, 16, cudaMemcpyDeviceToHost, h->stream));
+  HCK(cudaMemcpyAsync(h->word_host, h->word, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, h->stream));
   HCK(cudaStreamSynchronize(h->stream));
-  cudaFree(d_status);
-  *status_out = hs[0];
-  unsigned long long bits;
-  std::memcpy(&bits, &hs[2], 8);
-  double s;
-  std::memcpy(&s, &bits, 8);
-  *smax_out = s;
+  std::memcpy(status_out, &h->word_host[0], sizeof(int));
+  std::memcpy(smax_out, &h->word_host[1], sizeof(double));
   return HYDRO_OK;
 }
 
@@ -660,6 +667,8 @@ int hydro_common_init(hydro_ctx* h, int precision, void* stream) {
   }
   HCK(cudaMalloc(&h->ctrl, sizeof(Ctrl)));
   HCK(cudaMallocHost(&h->ctrl_host, sizeof(Ctrl)));
+  HCK(cudaMalloc(&h->word, 2 * sizeof(unsigned long long)));
+  HCK(cudaMallocHost(&h->word_host, 2 * sizeof(unsigned long long)));
   std::memset(h->ctrl_host, 0, sizeof(Ctrl));
   h->ctrl_host->err_step = -1;
   return write_ctrl(h);
@@ -939,7 +948,7 @@ int hydro_set_inner_mass(hydro_t h, double mass) {
 int hydro_set_state(hydro_t h, const void* U, int where) {
   if (!h || !U) return arg_error("hydro_set_state: null argument");
   if (h->batched) return hydro_batch_set_state_impl(h, U, where);
-  int st = read_ctrl(h);
+  int st = sync_ctrl(h);
   if (st) return st;
   const int slot = h->ctrl_host->cur ^ 1;
   const size_t bytes = (size_t)h->nv * h->ncell * h->esize;
@@ -968,7 +977,7 @@ int hydro_set_state(hydro_t h, const void* U, int where) {
 int hydro_get_state(hydro_t h, void* U_out, int where) {
   if (!h || !U_out) return arg_error("hydro_get_state: null argument");
   if (h->batched) return hydro_batch_get_state_impl(h, U_out, where);
-  int st = read_ctrl(h);
+  int st = sync_ctrl(h);
   if (st) return st;
   const size_t bytes = (size_t)h->nv * h->ncell * h->esize;
   HCK(cudaMemcpyAsync(U_out, h->buf[h->ctrl_host->cur], bytes,
@@ -979,7 +988,7 @@ int hydro_get_state(hydro_t h, void* U_out, int where) {
 
 int hydro_set_time(hydro_t h, double t) {
   if (!h) return arg_error("hydro_set_time: null handle");
-  int st = read_ctrl(h);
+  int st = sync_ctrl(h);
   if (st) return st;
   h->ctrl_host->t = t;
   return write_ctrl(h);
@@ -988,7 +997,7 @@ int hydro_set_time(hydro_t h, double t) {
 int hydro_cfl_dt(hydro_t h, double cfl, double* dt_out) {
   if (!h || !dt_out || !(cfl > 0)) return arg_error("hydro_cfl_dt: bad argument");
   if (h->batched) return arg_error("hydro_cfl_dt: batched handles use per-tube time steps");
-  int st = read_ctrl(h);
+  int st = sync_ctrl(h);
   if (st) return st;
   if (!(h->ctrl_host->smax_cur > 0.0)) return arg_error("hydro_cfl_dt: no signal speed (state not set?)");
   *dt_out = cfl / h->ctrl_host->smax_cur;
@@ -1070,14 +1079,14 @@ int hydro_run(hydro_t h, int nsteps, double cfl, double t_end, double* t_out) {
     // a moving grid's geometry follows each step's dt: steps driven from the host
     int st;
     for (int s = 0; s < nsteps; ++s) {
-      if ((st = read_ctrl(h))) return st;
+      if ((st = sync_ctrl(h))) return st;
       const double t0 = h->ctrl_host->t;
       if (t_end > 0.0 && t0 >= t_end) break;
       double dt = cfl / h->ctrl_host->smax_cur;
       if (t_end > 0.0 && t0 + dt > t_end) dt = t_end - t0;
       if ((st = hydro_step(h, dt))) return st;
     }
-    if ((st = read_ctrl(h))) return st;
+    if ((st = sync_ctrl(h))) return st;
     if (t_out) *t_out = h->ctrl_host->t;
     return HYDRO_OK;
   }
@@ -1110,6 +1119,7 @@ int hydro_run(hydro_t h, int nsteps, double cfl, double t_end, double* t_out) {
     h->graph_tend = t_end;
   }
   const long long step0 = h->ctrl_host->step;
+  h->ctrl_fresh = false;
   for (int s = 0; s < nsteps; ++s) HCK(cudaGraphLaunch(h->graph, h->stream));
   st = check_status(h, "hydro_run");
   if (st != HYDRO_OK) h->step_tot_ok = false;
@@ -1155,7 +1165,7 @@ int hydro_step_totals(hydro_t h, double* out_nv) {
 int hydro_totals(hydro_t h, double* out_nv) {
   if (!h || !out_nv) return arg_error("hydro_totals: null argument");
   if (h->batched) return arg_error("hydro_totals: grid handle required");
-  int st = read_ctrl(h);
+  int st = sync_ctrl(h);
   if (st) return st;
   dim3 grid(h->tot_blocks, h->nv);
   if (h->precision == 64)
@@ -1177,7 +1187,7 @@ int hydro_totals(hydro_t h, double* out_nv) {
 int hydro_stats(hydro_t h, hydro_stats_t* out) {
   if (!h || !out) return arg_error("hydro_stats: null argument");
   if (h->batched) return hydro_batch_stats_impl(h, out);
-  int st = read_ctrl(h);
+  int st = sync_ctrl(h);
   if (st) return st;
   std::memset(out, 0, sizeof(*out));
   out->steps = h->ctrl_host->step;
@@ -1202,6 +1212,8 @@ void hydro_destroy(hydro_t h) {
   h->arena.release();
   if (h->ctrl) cudaFree(h->ctrl);
   if (h->ctrl_host) cudaFreeHost(h->ctrl_host);
+  if (h->word) cudaFree(h->word);
+  if (h->word_host) cudaFreeHost(h->word_host);
   if (h->owns_stream && h->stream) cudaStreamDestroy(h->stream);
   delete h;
 }

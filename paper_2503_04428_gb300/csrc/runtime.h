@@ -63,6 +63,10 @@ struct hydro_ctx {
   void* buf[2] = {nullptr, nullptr};
   hydro::Ctrl* ctrl = nullptr;       // device control block
   hydro::Ctrl* ctrl_host = nullptr;  // pinned mirror
+  bool ctrl_fresh = false;           // the mirror holds the control block and nothing in flight changes it
+  // a validation's result: status, then the speed's bits (device and pinned)
+  unsigned long long* word = nullptr;
+  unsigned long long* word_host = nullptr;
   void* geo[32] = {nullptr};         // device geometry arrays (precision T)
   double* dvol[3] = {nullptr, nullptr, nullptr};  // FP64 volume factors a, b, c
   float* dv32[3] = {nullptr, nullptr, nullptr};   // b and c as FP32 pairs (hi, lo) to ~2^-48 (FP32 in-step totals)
