@@ -13,8 +13,11 @@
 //     flux reaches the cell below it by one shuffle down; on axis 2 the upper
 //     state of the plane below stays in registers; on
 //     axis 1 the upper state goes to the row above through shared memory,
-//     which returns the flux in the same slot: the only exchange that needs a
-//     barrier (two per plane, the second also covers the staged plane).
+//     which waits for that row alone (a barrier of two warps) and returns the
+//     flux in the same slot; the CTA meets once per plane, for the fluxes and
+//     the staged plane;
+//   - the halo rows' warps, which have the least to do, stage the cells beyond
+//     one per thread.
 // 30 of a warp's 32 lanes and R - 2 of the CTA's R rows own cells; the others
 // form the predicted states of the one-cell halo (the halo rows only those of
 // axis 1).  Face states are formed twice from the limited slopes, once for
@@ -24,9 +27,11 @@
 // Measured against the general sweep (one GB300, whole passes of state in,
 // 10 or 5 steps, state out): Sedov 256^3 HLL with totals 13.3 -> 9.75 ms,
 // wedge 1024 x 128^2 (NV = 8, HLLC, monopole) 10.9 -> 8.45 ms; thread
-// instructions per cell-update 2210 -> 990 (Sedov), 46 % of issue slots busy
-// with 16 warps per SM.  Bound now: fixed-latency dependences and barriers at
-// that occupancy (registers: 128 at NV = 5, 168 at NV = 6 and 8).
+// instructions per cell-update 2210 -> 990 (Sedov), 48 % of issue slots busy
+// with 16 warps per SM.  The two-warp barriers and the halo rows' staging then
+// gave 9.65 -> 9.34 and 7.81 -> 7.50 ms.  Bound now: fixed-latency dependences
+// at that occupancy (registers: 128 at NV = 5, 168 at NV = 6 and 8): 4 %
+// fewer instructions (the totals' sums of both halves in pairs) gave nothing.
 #pragma once
 #include <algorithm>
 
@@ -38,7 +43,8 @@ namespace hydro {
 
 // Rows of warps per CTA, one CTA per SM: as many as leave the step its
 // registers without spills (NV = 5: 16 rows of 128 registers 9.75 ms, 12 of
-// 168 10.9, 8 of 128 twice per SM with spills 14.8) and fit shared memory
+// 168 10.9; with the two-warp barriers 16 rows 9.49, 8 rows twice per SM
+// 9.73) and fit shared memory
 // with the totals (NV = 6: 12, NV = 8: 10).
 template <int NSX>
 struct March3Cfg {
@@ -52,7 +58,8 @@ struct March3Shape {
   static constexpr int TX = 30, TY = R - 2;          // owned cells
   static constexpr int EX = 34, EY = R + 2;          // a staged primitive plane
   static constexpr int NT = 32 * R, WPL = EX * EY;
-  static constexpr int NSTG = (WPL + NT - 1) / NT;   // staged cells per thread and plane
+  static constexpr int WX = WPL - NT;                // staged cells beyond one per thread
+  static_assert(WX <= 128, "two warps stage the rest, two cells a thread");
   // staged geometry: of the 32 columns and of the R rows
   enum { GX_SQ, GX_SF, GX_IW, GX_IR, GX_AF, GX_INVA, GX_GA, GX_QR, GX_GR, GX_G, GX_N };
   enum { GY_SQ, GY_SF, GY_IW, GY_IS, GY_BF, GY_INVB, GY_ZC, GY_GT, GY_QT, GY_N };
@@ -69,6 +76,11 @@ struct March3Shape {
   static constexpr size_t tot_bytes = (size_t)NV * TX * TY * sizeof(double);
 };
 
+// Barrier `id` (1 .. R-1; 0 is __syncthreads) of rows id - 1, which arrives and
+// goes on, and id, which waits for it.
+__device__ __forceinline__ void rows_arrive(int id) { asm volatile("bar.arrive %0, 64;" ::"r"(id) : "memory"); }
+__device__ __forceinline__ void rows_wait(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
+
 template <int NSX, int RS, bool SPH>
 __global__ void __launch_bounds__(March3Shape<NSX, SPH>::NT, March3Shape<NSX, SPH>::MB)
     march3_kernel(const SweepArgs<float> a) {
@@ -80,8 +92,8 @@ __global__ void __launch_bounds__(March3Shape<NSX, SPH>::NT, March3Shape<NSX, SP
   f2* const GX = Ws + S::off_gx;
   f2* const GY = Ws + S::off_gy;
   // totals: [v][owner] compensated column sums over both halves
-  float2* const tsum = a.tot_part ? reinterpret_cast<float2*>(smem_raw + S::smem_bytes) : nullptr;
   constexpr int NI = TX * TY;
+  float2* const tsum = a.tot_part ? reinterpret_cast<float2*>(smem_raw + S::smem_bytes) : nullptr;
   __shared__ double s_dt;
   __shared__ float s_hfac;
   const volatile Ctrl* vc = a.ctrl;
@@ -163,18 +175,29 @@ __global__ void __launch_bounds__(March3Shape<NSX, SPH>::NT, March3Shape<NSX, SP
   // (Byte offsets in 32 bits next to uniform 64-bit plane addresses cost no
   // integer instruction per access; planes of 2^30 cells or more index by
   // element.)
-  unsigned so[S::NSTG];
-  unsigned sflip = 0;
-#pragma unroll
-  for (int q = 0; q < S::NSTG; ++q) {
-    const int idx = tid + q * NT;
+  // A thread stages cell tid; the WPL - NT cells left over are staged by the
+  // halo rows' warps, which have no faces of axes 0 and 2 to form.
+  __shared__ unsigned s_so[S::WX];
+  __shared__ unsigned char s_flip[S::WX];
+  auto source_cell = [&](int idx, unsigned& off) {
     const int ex = idx % EX, ey = idx / EX;
     bool fx, fy;
     const int si = map_axis(min(x0 - 2 + ex, n0 + 1), n0, a.bc[0][0], a.bc[0][1], fx);
     const int sj = map_axis(min(y0 - 2 + ey, n1 + 1), n1, a.bc[1][0], a.bc[1][1], fy);
-    so[q] = (unsigned)sj * (unsigned)n0 + (unsigned)si;
-    sflip |= ((fx ? 1u : 0u) | (fy ? 2u : 0u)) << (2 * q);
-  }
+    off = (unsigned)sj * (unsigned)n0 + (unsigned)si;
+    return (fx ? 1u : 0u) | (fy ? 2u : 0u);
+  };
+  unsigned so;
+  const unsigned sflip = source_cell(tid, so);
+  const bool halo_row = row == 0 || row == R - 1;
+  const int e0 = (row == 0 ? 0 : 64) + lane;  // this thread's left-over cells: e0, e0 + 32
+  if (halo_row)
+    for (int e = e0; e < e0 + 64; e += 32)
+      if (e < S::WX) {
+        unsigned o;
+        s_flip[e] = (unsigned char)source_cell(NT + e, o);
+        s_so[e] = o;
+      }
   const bool edge = x0 < 2 || x0 + TX + 2 > n0 || y0 < 2 || y0 + TY + 2 > n1;  // x or y ghosts are staged
   // a1: plane i of both halves (may be ghosts) starts to arrive, conserved,
   // in its ring slot (asynchronous 4-byte copies, issued one phase ahead of
@@ -184,7 +207,6 @@ __global__ void __launch_bounds__(March3Shape<NSX, SPH>::NT, March3Shape<NSX, SP
   };
   auto ghosts = [&](int i) { return z0 + i < 0 || zb + i >= n2; };  // either plane is one (z0 <= zb)
   auto fetch = [&](int i, int slot) {
-    f2* const raw = Ws + slot * (NV * WPL) + tid;
     int k0 = z0 + i, k1 = zb + i;
     if (ghosts(i)) {
       bool fz;
@@ -193,27 +215,30 @@ __global__ void __launch_bounds__(March3Shape<NSX, SPH>::NT, March3Shape<NSX, SP
     }
     const float* const s0 = Uin + k0 * plane;
     const float* const s1 = Uin + k1 * plane;
+    auto copy = [&](f2* raw, unsigned off) {
+      const unsigned d = smem_addr(raw);
+      if (small) {
+        const unsigned o = off * 4u;
 #pragma unroll
-    for (int q = 0; q < S::NSTG; ++q) {
-      if ((q + 1) * NT <= WPL || q * NT + tid < WPL) {
-        const unsigned d = smem_addr(raw + q * NT);
-        if (small) {
-          const unsigned o = so[q] * 4u;
-#pragma unroll
-          for (int v = 0; v < NV; ++v)
-            if (active(v)) {
-              copy4_async(d + v * WPL * 8, at_byte(s0 + v * a.ncell, o));
-              copy4_async(d + v * WPL * 8 + 4, at_byte(s1 + v * a.ncell, o));
-            }
-        } else {
+        for (int v = 0; v < NV; ++v)
+          if (active(v)) {
+            copy4_async(d + v * WPL * 8, at_byte(s0 + v * a.ncell, o));
+            copy4_async(d + v * WPL * 8 + 4, at_byte(s1 + v * a.ncell, o));
+          }
+      } else {
 #pragma unroll 1
-          for (int v = 0; v < NV; ++v)
-            if (active(v)) {
-              copy4_async(d + v * WPL * 8, s0 + v * a.ncell + so[q]);
-              copy4_async(d + v * WPL * 8 + 4, s1 + v * a.ncell + so[q]);
-            }
-        }
+        for (int v = 0; v < NV; ++v)
+          if (active(v)) {
+            copy4_async(d + v * WPL * 8, s0 + v * a.ncell + off);
+            copy4_async(d + v * WPL * 8 + 4, s1 + v * a.ncell + off);
+          }
       }
+    };
+    copy(Ws + slot * (NV * WPL) + tid, so);
+    if (halo_row) {
+#pragma unroll 1
+      for (int e = e0; e < e0 + 64; e += 32)
+        if (e < S::WX) copy(Ws + slot * (NV * WPL) + NT + e, s_so[e]);
     }
   };
   // a2: what has arrived of plane i in ring slot `slot`, to primitives
@@ -223,22 +248,24 @@ __global__ void __launch_bounds__(March3Shape<NSX, SPH>::NT, March3Shape<NSX, SP
       source(z0 + i, fz0);
       source(zb + i, fz1);
     }
-    f2* dst = Ws + slot * (NV * WPL) + tid;
+    auto convert = [&](f2* dst, unsigned flip) {
+      f2 u[NV], w[NV];
 #pragma unroll
-    for (int q = 0; q < S::NSTG; ++q) {
-      if ((q + 1) * NT <= WPL || q * NT + tid < WPL) {
-        f2 u[NV], w[NV];
-#pragma unroll
-        for (int v = 0; v < NV; ++v) u[v] = active(v) ? dst[v * WPL + q * NT] : both(0.f);
-        if (edge) {
-          if ((sflip >> (2 * q)) & 1u) u[1] = both(0.f) - u[1];
-          if ((sflip >> (2 * q)) & 2u) u[2] = both(0.f) - u[2];
-        }
-        if (fz0 || fz1) u[3] = make_f2(fz0 ? -lo(u[3]) : lo(u[3]), fz1 ? -hi(u[3]) : hi(u[3]));
-        to_prim2<3, NSX>(u, w, gas);
-#pragma unroll
-        for (int v = 0; v < NV; ++v) dst[v * WPL + q * NT] = w[v];
+      for (int v = 0; v < NV; ++v) u[v] = active(v) ? dst[v * WPL] : both(0.f);
+      if (edge) {
+        if (flip & 1u) u[1] = both(0.f) - u[1];
+        if (flip & 2u) u[2] = both(0.f) - u[2];
       }
+      if (fz0 || fz1) u[3] = make_f2(fz0 ? -lo(u[3]) : lo(u[3]), fz1 ? -hi(u[3]) : hi(u[3]));
+      to_prim2<3, NSX>(u, w, gas);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) dst[v * WPL] = w[v];
+    };
+    convert(Ws + slot * (NV * WPL) + tid, sflip);
+    if (halo_row) {
+#pragma unroll 1
+      for (int e = e0; e < e0 + 64; e += 32)
+        if (e < S::WX) convert(Ws + slot * (NV * WPL) + NT + e, s_flip[e]);
     }
   };
   // the own cells' conserved state of plane i (an owned one), for its update
@@ -516,6 +543,7 @@ __global__ void __launch_bounds__(March3Shape<NSX, SPH>::NT, March3Shape<NSX, SP
           });
 #pragma unroll
           for (int v = 0; v < NV; ++v) Yo[v * (R * 32)] = wh[v];
+          if (gj < n1) rows_arrive(row + 1);
         }
         if (row >= 1) lower(sy, ylo, [&](int h) { return lown && (rown || gj == n1) && counts(h); });
       }
@@ -523,11 +551,11 @@ __global__ void __launch_bounds__(March3Shape<NSX, SPH>::NT, March3Shape<NSX, SP
     if (i == len) break;
     if (inner) fetch_own(i);
     copies_commit();
-    __syncthreads();
     f2 F[NV];
     if (inner && row >= 1 && ract) {
       // a5, axis 1: the face below this row, its flux into the slot the
       // row below reads back
+      rows_wait(row);
       f2 wl[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) wl[v] = Yo[v * (R * 32) - 32];

@@ -58,6 +58,18 @@ __device__ __forceinline__ f2 max2_0(f2 a, f2 b) {
   return make_f2(fmaxf(fmaxf(lo(a), lo(b)), 0.f), fmaxf(fmaxf(hi(a), hi(b)), 0.f));
 }
 
+// Minima that are NaN if an argument is.
+__device__ __forceinline__ float min_or_nan(float a, float b) {
+  float r;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float min_or_nan(float a, float b, float c) {
+  float r;
+  asm("min.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+
 // The gas constants as pairs.
 struct Gas2 {
   f2 g, gm1, igm1, half, mhalf;
@@ -123,8 +135,9 @@ __device__ __forceinline__ void face_state2(const f2* l, const f2* dU, const f2*
 #pragma unroll
   for (int s = 0; s < NSX; ++s) u[2 + D + s] = fma2(l[0], l[2 + D + s], dU[2 + D + s]);
   to_prim2<D, NSX>(u, w, gas);
-  const bool bad0 = !(lo(w[0]) > 0.f) || !(lo(w[1 + D]) > 0.f), bad1 = !(hi(w[0]) > 0.f) || !(hi(w[1 + D]) > 0.f);
-  if (__any_sync(0xffffffffu, bad0 || bad1)) {
+  // (the usual outcome costs two minima and one comparison)
+  if (__any_sync(0xffffffffu, !(min_or_nan(min_or_nan(lo(w[0]), lo(w[1 + D]), hi(w[0])), hi(w[1 + D])) > 0.f))) {
+    const bool bad0 = !(min_or_nan(lo(w[0]), lo(w[1 + D])) > 0.f), bad1 = !(min_or_nan(hi(w[0]), hi(w[1 + D])) > 0.f);
 #pragma unroll
     for (int v = 0; v < NV; ++v) w[v] = pick(bad0, bad1, Wc[v], w[v]);
     count(bad0, bad1);
