@@ -458,6 +458,32 @@ __device__ __forceinline__ void flux_cons_e(const T* W, T e, T* F, T* U) {
   }
 }
 
+// FP64: the difference of the fluxes of two limited states (ideal gas) and
+// their conserved states, every fused operation written out, so that all
+// instantiations round alike.
+template <int D, int NSX, int DIR>
+__device__ __forceinline__ void flux_diff(const double* Wl, const double* Wh, double igm1, double* dF, double* Ul,
+                                          double* Uh) {
+  auto conserved = [&](const double* W, double* U) {
+    double v2 = __dmul_rn(W[1], W[1]);
+#pragma unroll
+    for (int d = 1; d < D; ++d) v2 = fma(W[1 + d], W[1 + d], v2);
+    U[0] = W[0];
+#pragma unroll
+    for (int v = 1; v < 2 + D + NSX; ++v) U[v] = __dmul_rn(W[0], W[v]);
+    U[1 + D] = fma(__dmul_rn(0.5, W[0]), v2, __dmul_rn(W[1 + D], igm1));
+  };
+  conserved(Wl, Ul);
+  conserved(Wh, Uh);
+  const double ul = Wl[1 + DIR], uh = Wh[1 + DIR], pl = Wl[1 + D], ph = Wh[1 + D];
+  const double ml = Ul[1 + DIR], mh = Uh[1 + DIR];
+  dF[0] = __dsub_rn(ml, mh);
+#pragma unroll
+  for (int v = 1; v < 2 + D + NSX; ++v) dF[v] = fma(ml, Wl[v], -__dmul_rn(mh, Wh[v]));
+  dF[1 + DIR] = __dsub_rn(fma(ml, ul, pl), fma(mh, uh, ph));
+  dF[1 + D] = fma(ul, __dadd_rn(Ul[1 + D], pl), -__dmul_rn(uh, __dadd_rn(Uh[1 + D], ph)));
+}
+
 // HLL flux of two states with known internal energies and sound speeds,
 // Davis speeds S_L, S_R.  With S_L clamped to <= 0 and S_R to >= 0 (the
 // supersonic cases included), F = a F_L + b F_R + c (U_R - U_L) with a =

@@ -33,7 +33,7 @@ namespace hydro {
 // thread per predictor cell (the tile plus a one-cell halo without corners),
 // rounded up to whole warps.  SMALL: the 1D and 2D tiles of grids whose large
 // tiles would leave SMs idle (see small_tile): 28 cells and their halo fill
-// one warp, 8 x 8 three.
+// one warp, 8 x 8 three (FP64: twice as many, see Sweep::predictor_split).
 template <typename T, int DIM, int NSX, bool SMALL>
 struct TileCfg {
   static constexpr int TX = DIM == 1 ? (SMALL ? 28 : 254) : (SMALL ? 8 : 16);
@@ -57,7 +57,11 @@ struct SweepShape {
   static constexpr int NI = TX * TY;                        // tile cells, one owner thread each
   static constexpr int NH = 2 * TY + (DIM >= 2 ? 2 * TX : 0);  // halo predictor cells
   static constexpr int NP = NI + NH;                        // predictor cells
-  static constexpr int NT = (NP + 31) / 32 * 32;            // threads per CTA
+  static constexpr int NPT = (NP + 31) / 32 * 32;
+  // threads per CTA: one per predictor cell, for the small FP64 tiles two (see
+  // Sweep::predictor_split)
+  static constexpr bool TWO = SMALL && sizeof(T) == 8;
+  static constexpr int NT = TWO ? 2 * NPT : NPT;
   static constexpr int MB = TileCfg<T, DIM, NSX, SMALL>::MB;       // resident CTAs per SM (register budget)
   static constexpr int WPL = EX * EY;
   static constexpr int NFX = (TX + 1) * TY;
@@ -68,13 +72,19 @@ struct SweepShape {
   static constexpr size_t dual_elems = (size_t)2 * (NFX + NFY + NFZ);  // dual-energy face terms
   // radiation EoS: face-state temperatures and those of the primitive planes
   static constexpr size_t rad_elems = (size_t)2 * NFX + 2 * NFY + 3 * NFZ + (size_t)WP * WPL;
+  // FP64, ideal gas: the face states' sound speeds, in the temperatures' place
+  static constexpr size_t snd_elems = (size_t)2 * NFX + 2 * NFY + 3 * NFZ;
+  __host__ __device__ static constexpr size_t face_elems(int mode) {
+    return (mode & 1) ? rad_elems : sizeof(T) == 8 ? snd_elems : 0;
+  }
   // the x and y geometry factors of the CTA's cells, staged once per CTA
   // (GX_N arrays over the TX + 2 predictor columns, GY_N over the TY + 2 rows)
   enum { GX_SQ, GX_SF, GX_IW, GX_IR, GX_AF, GX_INVA, GX_GA, GX_QR, GX_GR, GX_G, GX_N };
   enum { GY_SQ, GY_SF, GY_IW, GY_IS, GY_BF, GY_INVB, GY_ZC, GY_GT, GY_QT, GY_N };
   static constexpr size_t geo_elems = (size_t)GX_N * (TX + 2) + (DIM >= 2 ? (size_t)GY_N * (TY + 2) : 0);
+  static constexpr size_t split_elems = TWO && DIM == 2 ? (size_t)2 * NV * NPT : 0;  // what the two exchange
   __host__ __device__ static constexpr size_t smem_bytes_for(int mode) {
-    return (smem_elems + ((mode & 2) ? dual_elems : 0) + ((mode & 1) ? rad_elems : 0) + geo_elems) * sizeof(T);
+    return (smem_elems + ((mode & 2) ? dual_elems : 0) + face_elems(mode) + geo_elems + split_elems) * sizeof(T);
   }
   // conserved totals accumulated in the step: one FP64 sum per owner and
   // variable, after the rest (16-byte aligned)
@@ -159,6 +169,10 @@ template <typename T, int DIM, int NSX, int RS, int MODE, bool SMALL, bool MULTI
 struct Sweep {
   static constexpr int EOS = MODE & 1;
   static constexpr bool DUAL = (MODE & 2) != 0;
+  // A face state's sound speed is formed with the state, whose 1/rho is at
+  // hand (FP64: three operations of its pipe per state; FP32 reciprocals are
+  // cheaper than the exchange).
+  static constexpr bool SND = EOS == 0 && sizeof(T) == 8 && RS != RS_EXACT;
   static constexpr bool XM = (MODE & 4) != 0;
   // in-step totals as compensated FP32 column sums (FP32, 3D) instead of FP64 sums per cell
   static constexpr bool COLSUM = sizeof(T) == 4 && DIM == 3;
@@ -231,7 +245,7 @@ struct Sweep {
     ZTL = YTR + NFY;
     ZTR = ZTL + 2 * NFZ;
     WT = ZTR + NFZ;
-    GXs = Ws + S::smem_elems + (DUAL ? S::dual_elems : 0) + (EOS == 1 ? S::rad_elems : 0);
+    GXs = Ws + S::smem_elems + (DUAL ? S::dual_elems : 0) + S::face_elems(MODE);
     GYs = GXs + S::GX_N * (TX + 2);
   }
 
@@ -523,7 +537,8 @@ struct Sweep {
   // Turn the limited state parked at p (stride `st`) into the predicted face
   // state: W -> U, + dU, U -> W; a non-physical result falls back to Wc.
   // The radiation EoS parks the conserved state (the flux evaluation already
-  // solved for its energy) and records the temperature of the result at tp.
+  // solved for its energy) and records the temperature of the result at tp;
+  // SND: its sound speed.
   __device__ __forceinline__ void finish_state(T* p, int st, const T* Wc, const T* dU, bool owned,
                                                T* tp = nullptr) {
     T w[NV], u[NV];
@@ -556,11 +571,15 @@ struct Sweep {
 #pragma unroll
       for (int v = 0; v < NV; ++v) u[v] = p[v * st] + dU[v];
       to_prim<T, DIM, NSX>(u, w, gas());
+      T e, c = T(0);
+      if constexpr (SND) face_e_c<T>(a.gas, w[0], w[1 + DIM], T(0), e, c);
       if (!is_pos(w[0]) || !is_pos(w[1 + DIM])) {
 #pragma unroll
         for (int v = 0; v < NV; ++v) w[v] = Wc[v];
+        if constexpr (SND) face_e_c<T>(a.gas, w[0], w[1 + DIM], T(0), e, c);
         if (owned) ++n_fallback;
       }
+      if constexpr (SND) *tp = c;
     }
 #pragma unroll
     for (int v = 0; v < NV; ++v) p[v * st] = w[v];
@@ -604,12 +623,39 @@ struct Sweep {
     }
   }
 
+  // The difference of the physical fluxes of the two limited states along
+  // DIR (see limited_fluxes).
+  template <int DIR>
+  __device__ __forceinline__ void limited_diff(const T* Wl, const T* Wh, T* dF, T* Pl, T* Ph, T tc, T* tl, T* th) {
+    if constexpr (EOS == 0 && sizeof(T) == 8) {
+      flux_diff<DIM, NSX, DIR>(Wl, Wh, a.gas.igm1, dF, Pl, Ph);
+      if constexpr (XM) {
+        if (a.maxis == DIR) {
+#pragma unroll
+          for (int v = 0; v < NV; ++v) dF[v] -= a.wg * (Pl[v] - Ph[v]);
+        }
+      }
+    } else {
+      T Fl[NV], Fh[NV];
+      limited_fluxes<DIR>(Wl, Wh, Fl, Fh, Pl, Ph, tc, tl, th);
+      if constexpr (XM) {
+        if (a.maxis == DIR) moving_fluxes(Pl, Ph, Fl, Fh);
+      }
+#pragma unroll
+      for (int v = 0; v < NV; ++v) dF[v] = Fl[v] - Fh[v];
+    }
+  }
+
   // a3 + a4 for plane gz: the predictor increment dU = sum_d
   // (F_d(W_lo) - F_d(W_hi)) dt/(2 h_d) of every needed cell, and its predicted face
   // states.  PRED_ALL: tile plus halo, every face state of the plane;
   // PRED_ZHI / PRED_ZLO: tile cells only, the upper / lower z state.
   template <int PM>
   __device__ void predictor(int gz) {
+    if constexpr (S::TWO && EOS == 0 && !XM) {
+      predictor_split();
+      return;
+    }
     const int t = threadIdx.x;
     if (t >= (PM == PRED_ALL ? NP : NI)) return;
     const int n0 = a.n[0], n1 = a.n[1];
@@ -646,7 +692,7 @@ struct Sweep {
     }
     const T tcell = EOS == 1 ? WT[(slot * EY + ey) * EX + ex] : T(0);
     {
-      T Wm[NV], Wp[NV], Wl[NV], Wh[NV], Fl[NV], Fh[NV];
+      T Wm[NV], Wp[NV], Wl[NV], Wh[NV], dF[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         Wm[v] = W(slot, v, ey, ex - 1);
@@ -654,10 +700,7 @@ struct Sweep {
       }
       faces_of<0>(Wm, Wc, Wp, px, Wl, Wh);
       T Pl[NV], Ph[NV], tl = T(0), th = T(0);
-      limited_fluxes<0>(Wl, Wh, Fl, Fh, Pl, Ph, tcell, &tl, &th);
-      if constexpr (XM) {
-        if (a.maxis == 0) moving_fluxes(Pl, Ph, Fl, Fh);
-      }
+      limited_diff<0>(Wl, Wh, dF, Pl, Ph, tcell, &tl, &th);
       if constexpr (EOS == 1) {
         if (xlo) XTR[ixlo] = tl;
         if (xhi) XTL[ixhi] = th;
@@ -665,13 +708,13 @@ struct Sweep {
       const T ih = inv_h(0, px, py, gz) * half_dt;
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        dU[v] += (Fl[v] - Fh[v]) * ih;
+        dU[v] += dF[v] * ih;
         if (xlo) XR[v * NFX + ixlo] = Pl[v];
         if (xhi) XL[v * NFX + ixhi] = Ph[v];
       }
     }
     if constexpr (DIM >= 2) {
-      T Wm[NV], Wp[NV], Wl[NV], Wh[NV], Fl[NV], Fh[NV];
+      T Wm[NV], Wp[NV], Wl[NV], Wh[NV], dF[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         Wm[v] = W(slot, v, ey - 1, ex);
@@ -679,10 +722,7 @@ struct Sweep {
       }
       faces_of<1>(Wm, Wc, Wp, py, Wl, Wh);
       T Pl[NV], Ph[NV], tl = T(0), th = T(0);
-      limited_fluxes<1>(Wl, Wh, Fl, Fh, Pl, Ph, tcell, &tl, &th);
-      if constexpr (XM) {
-        if (a.maxis == 1) moving_fluxes(Pl, Ph, Fl, Fh);
-      }
+      limited_diff<1>(Wl, Wh, dF, Pl, Ph, tcell, &tl, &th);
       if constexpr (EOS == 1) {
         if (ylo) YTR[iylo] = tl;
         if (yhi) YTL[iyhi] = th;
@@ -690,13 +730,13 @@ struct Sweep {
       const T ih = inv_h(1, px, py, gz) * half_dt;
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        dU[v] += (Fl[v] - Fh[v]) * ih;
+        dU[v] += dF[v] * ih;
         if (ylo) YR[v * NFY + iylo] = Pl[v];
         if (yhi) YL[v * NFY + iyhi] = Ph[v];
       }
     }
     if constexpr (DIM == 3) {
-      T Wm[NV], Wp[NV], Wl[NV], Wh[NV], Fl[NV], Fh[NV];
+      T Wm[NV], Wp[NV], Wl[NV], Wh[NV], dF[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         Wm[v] = W(wslot(gz - 1), v, ey, ex);
@@ -704,10 +744,7 @@ struct Sweep {
       }
       faces_of<2>(Wm, Wc, Wp, gz, Wl, Wh);
       T Pl[NV], Ph[NV], tl = T(0), th = T(0);
-      limited_fluxes<2>(Wl, Wh, Fl, Fh, Pl, Ph, tcell, &tl, &th);
-      if constexpr (XM) {
-        if (a.maxis == 2) moving_fluxes(Pl, Ph, Fl, Fh);
-      }
+      limited_diff<2>(Wl, Wh, dF, Pl, Ph, tcell, &tl, &th);
       if constexpr (EOS == 1) {
         if (zlo) ZTR[iz] = tl;
         if (zhi) ZTL[(gz & 1) * NFZ + iz] = th;
@@ -715,7 +752,7 @@ struct Sweep {
       const T ih = inv_h(2, px, py, gz) * half_dt;
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        dU[v] += (Fl[v] - Fh[v]) * ih;
+        dU[v] += dF[v] * ih;
         if (zlo) ZR[v * NFZ + iz] = Pl[v];
         if (zhi) zhp[v * NFZ + iz] = Ph[v];
       }
@@ -739,6 +776,96 @@ struct Sweep {
     if constexpr (DIM == 3) {
       if (zlo) finish_state(ZR + iz, NFZ, Wc, dU, gz < z1 || gz == n2, ZTR + iz);
       if (zhi) finish_state(zhp + iz, NFZ, Wc, dU, gz + 1 < z1 || gz + 1 == n2, ztl + iz);
+    }
+  }
+
+  // predictor for the small FP64 tiles, of two threads per cell: in 2D one
+  // takes axis 0 and the other axis 1, and they exchange the flux differences;
+  // in 1D both evaluate these, and one finishes the lower and the other the
+  // upper state.  A warp's FP64 operation occupies its scheduler for 64 cycles
+  // whatever its active lanes and however few other warps there are, so the
+  // longest chain of one warp is what counts: Sod 1000 FP64 9.6 -> 8.8 us per
+  // step, 64 x 128 FP64 HLLC 42.7 -> 41.7 per cfl_dt + step.
+  __device__ void predictor_split() {
+    const int part = threadIdx.x / S::NPT, t = threadIdx.x % S::NPT;  // (part: the same in a warp)
+    const int n0 = a.n[0], n1 = a.n[1];
+    T* const mine = GXs + S::geo_elems + part * (NV * S::NPT) + t;
+    const T* const parts = GXs + S::geo_elems + t;
+    int px = 0, py = 0;
+    if (t < NP) item_cell(t, px, py);
+    const int gi = x0 - 1 + px, gj = DIM >= 2 ? y0 - 1 + py : 0;
+    const bool cell = t < NP && gi <= n0 && (DIM < 2 || gj <= n1);
+    const int ex = px + 1, ey = py + (HY - QY), row = py - QY, col = px - 1;
+    const bool rreal = DIM < 2 || gj < n1, creal = gi < n0;
+    const bool trow = DIM < 2 || (py >= 1 && py <= TY), tcol = px >= 1 && px <= TX;
+    T Wc[NV], Wl[NV], Wh[NV], dF[NV], Pl[NV], Ph[NV];
+    if (cell) {
+#pragma unroll
+      for (int v = 0; v < NV; ++v) Wc[v] = W(0, v, ey, ex);
+      T Wm[NV], Wp[NV];
+      if constexpr (DIM == 1) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          Wm[v] = W(0, v, ey, ex - 1);
+          Wp[v] = W(0, v, ey, ex + 1);
+        }
+        faces_of<0>(Wm, Wc, Wp, px, Wl, Wh);
+        flux_diff<DIM, NSX, 0>(Wl, Wh, a.gas.igm1, dF, Pl, Ph);
+      } else {
+        const int dx = part == 0 ? 1 : 0, dy = 1 - dx;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          Wm[v] = W(0, v, ey - dy, ex - dx);
+          Wp[v] = W(0, v, ey + dy, ex + dx);
+        }
+        if (part == 0) {
+          faces_of<0>(Wm, Wc, Wp, px, Wl, Wh);
+          flux_diff<DIM, NSX, 0>(Wl, Wh, a.gas.igm1, dF, Pl, Ph);
+        } else {
+          faces_of<1>(Wm, Wc, Wp, py, Wl, Wh);
+          flux_diff<DIM, NSX, (DIM >= 2 ? 1 : 0)>(Wl, Wh, a.gas.igm1, dF, Pl, Ph);
+        }
+#pragma unroll
+        for (int v = 0; v < NV; ++v) mine[v * S::NPT] = dF[v];
+      }
+    }
+    if constexpr (DIM >= 2) __syncthreads();
+    if (!cell) return;
+    T dU[NV];
+    const T ix = inv_h(0, px, py, 0) * half_dt;
+    if constexpr (DIM == 1) {
+#pragma unroll
+      for (int v = 0; v < NV; ++v) dU[v] = dF[v] * ix;
+    } else {
+      const T iy = inv_h(1, px, py, 0) * half_dt;
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        dU[v] = fma(parts[(NV + v) * S::NPT], iy, __dmul_rn(parts[v * S::NPT], ix));
+      }
+    }
+    if (threadIdx.x < NI) {
+#pragma unroll
+      for (int v = 0; v < NV; ++v) dUo[v] = dU[v];
+    }
+    auto finish = [&](bool needed, T* p, int st, const T* P, bool owned, T* tp) {
+      if (!needed) return;
+#pragma unroll
+      for (int v = 0; v < NV; ++v) p[v * st] = P[v];
+      finish_state(p, st, Wc, dU, owned, tp);
+    };
+    // (faces as in predictor: needed, slot, counted by this CTA)
+    const int ixlo = row * (TX + 1) + px - 1, iylo = (py - 1) * TX + col, iyhi = iylo + TX;
+    const bool xlo = px >= 1 && trow && rreal, xhi = px <= TX && trow && rreal && creal;
+    const bool lo_owned = px - 1 < TX || gi == n0, hi_owned = px < TX || gi + 1 == n0;
+    if constexpr (DIM == 1) {
+      if (part == 0) finish(xlo, XR + ixlo, NFX, Pl, lo_owned, XTR + ixlo);
+      else finish(xhi, XL + ixlo + 1, NFX, Ph, hi_owned, XTL + ixlo + 1);
+    } else if (part == 0) {
+      finish(xlo, XR + ixlo, NFX, Pl, lo_owned, XTR + ixlo);
+      finish(xhi, XL + ixlo + 1, NFX, Ph, hi_owned, XTL + ixlo + 1);
+    } else {
+      finish(py >= 1 && tcol && creal, YR + iylo, NFY, Pl, py - 1 < TY || gj == n1, YTR + iylo);
+      finish(py <= TY && tcol && creal && rreal, YL + iyhi, NFY, Ph, py < TY || gj + 1 == n1, YTL + iyhi);
     }
   }
 
@@ -777,7 +904,11 @@ struct Sweep {
   template <int DIR>
   __device__ __forceinline__ void riemann_fixed(const T* WL, const T* WR, T* F, bool owned, T TL = T(0),
                                                 T TR = T(0)) {
-    if constexpr (RS == RS_HLL) {
+    if constexpr (SND) {
+      const T eL = WL[1 + DIM] * a.gas.igm1, eR = WR[1 + DIM] * a.gas.igm1;
+      if constexpr (RS == RS_HLL) hll_flux<T, DIM, NSX, DIR>(WL, WR, eL, eR, TL, TR, F);
+      else hllc_flux<T, DIM, NSX, DIR>(WL, WR, eL, eR, TL, TR, F);
+    } else if constexpr (RS == RS_HLL) {
       riemann_hll<T, DIM, NSX, DIR>(WL, WR, F, gas(), TL, TR);
     } else if constexpr (RS == RS_HLLC) {
       riemann_hllc<T, DIM, NSX, DIR>(WL, WR, F, gas(), TL, TR);
@@ -797,7 +928,7 @@ struct Sweep {
     constexpr int NXY = XY ? NFX + NFY : 0;
     constexpr int NALL = NXY + (Z ? NFZ : 0);
     const T* zlp = ZL + ((gz - 1) & 1) * NV * NFZ;
-    constexpr bool dual = DUAL;
+    constexpr bool dual = DUAL, FT = EOS == 1 || SND;
     for (int idx = threadIdx.x; idx < NALL; idx += NT) {
       T WL[NV], WR[NV], F[NV];
       if (XY && idx < NFX) {
@@ -808,7 +939,7 @@ struct Sweep {
           WL[v] = XL[v * NFX + idx];
           WR[v] = XR[v * NFX + idx];
         }
-        riemann<0>(WL, WR, F, f < TX || x0 + f == n0, EOS ? XTL[idx] : T(0), EOS ? XTR[idx] : T(0));
+        riemann<0>(WL, WR, F, f < TX || x0 + f == n0, FT ? XTL[idx] : T(0), FT ? XTR[idx] : T(0));
         if constexpr (dual) dual_terms(WL, WR, F, XQ, NFX, idx);
 #pragma unroll
         for (int v = 0; v < NV; ++v) XL[v * NFX + idx] = F[v];
@@ -821,8 +952,8 @@ struct Sweep {
           WL[v] = YL[v * NFY + k];
           WR[v] = YR[v * NFY + k];
         }
-        riemann<(DIM >= 2 ? 1 : 0)>(WL, WR, F, fy < TY || y0 + fy == n1, EOS ? YTL[k] : T(0),
-                                    EOS ? YTR[k] : T(0));
+        riemann<(DIM >= 2 ? 1 : 0)>(WL, WR, F, fy < TY || y0 + fy == n1, FT ? YTL[k] : T(0),
+                                    FT ? YTR[k] : T(0));
         if constexpr (dual) dual_terms(WL, WR, F, YQ, NFY, k);
 #pragma unroll
         for (int v = 0; v < NV; ++v) YL[v * NFY + k] = F[v];
@@ -836,7 +967,7 @@ struct Sweep {
           WR[v] = ZR[v * NFZ + k];
         }
         riemann<(DIM == 3 ? 2 : 0)>(WL, WR, F, gz < z1 || gz == n2,
-                                    EOS ? ZTL[((gz - 1) & 1) * NFZ + k] : T(0), EOS ? ZTR[k] : T(0));
+                                    FT ? ZTL[((gz - 1) & 1) * NFZ + k] : T(0), FT ? ZTR[k] : T(0));
         if constexpr (dual) dual_terms(WL, WR, F, ZQ, NFZ, k);
 #pragma unroll
         for (int v = 0; v < NV; ++v) ZR[v * NFZ + k] = F[v];
@@ -851,8 +982,12 @@ struct Sweep {
     const int fx = j * (TX + 1) + i;
     const T Afl = gx(S::GX_AF, i + 1), Afh = gx(S::GX_AF, i + 2), ia = gx(S::GX_INVA, i + 1);
     constexpr bool dual = DUAL;
+    const bool sph = a.spherical;  // (Cartesian area factors are 1)
 #pragma unroll
-    for (int v = 0; v < NV; ++v) acc[v] = (XL[v * NFX + fx] * Afl - XL[v * NFX + fx + 1] * Afh) * ia;
+    for (int v = 0; v < NV; ++v) {
+      const T fl = XL[v * NFX + fx], fh = XL[v * NFX + fx + 1];
+      acc[v] = (sph ? fl * Afl - fh * Afh : fl - fh) * ia;
+    }
     if constexpr (dual) {
       aq1 = (XQ[fx] * Afl - XQ[fx + 1] * Afh) * ia;
       aq2 = (XQ[NFX + fx] * Afl - XQ[NFX + fx + 1] * Afh) * ia;
@@ -862,7 +997,10 @@ struct Sweep {
       const T cy = gx(S::GX_GA, i + 1) * gy(S::GY_INVB, j + 1);
       const int fy = j * TX + i;
 #pragma unroll
-      for (int v = 0; v < NV; ++v) acc[v] += (YL[v * NFY + fy] * Bfl - YL[v * NFY + fy + TX] * Bfh) * cy;
+      for (int v = 0; v < NV; ++v) {
+        const T fl = YL[v * NFY + fy], fh = YL[v * NFY + fy + TX];
+        acc[v] += (sph ? fl * Bfl - fh * Bfh : fl - fh) * cy;
+      }
       if constexpr (dual) {
         aq1 += (YQ[fy] * Bfl - YQ[fy + TX] * Bfh) * cy;
         aq2 += (YQ[NFY + fy] * Bfl - YQ[NFY + fy + TX] * Bfh) * cy;
@@ -1276,8 +1414,8 @@ __global__ void __launch_bounds__(SweepShape<T, DIM, NSX, SMALL>::NT,
 // its stores), waits (bounded) for every CTA's and takes their maximum itself.
 // A word's sign bit says which use of it is meant: the words of even and odd
 // steps are apart, zeroed before the launch, and each use flips the sign, so
-// none is overwritten before all have read it (9.6 us per step; 9.8 with a
-// counter beside the words).  A step that fails in a CTA
+// none is overwritten before all have read it (8.8 us per step; a counter
+// beside the words cost 0.2 more).  A step that fails in a CTA
 // publishes NaN: every CTA ends with the state before it.  The buffers
 // alternate as between launches.
 constexpr int ST_STEP_TIMEOUT = -6;  // HYDRO_ERR_TIMEOUT
@@ -1469,7 +1607,7 @@ bool small_tile(const int* n, int sms) {
   };
   using L = SweepShape<T, DIM, NSX, false>;
   using M = SweepShape<T, DIM, NSX, true>;
-  return busiest(M::TX, M::TY, M::NT) < busiest(L::TX, L::TY, L::NT);
+  return busiest(M::TX, M::TY, M::NPT) < busiest(L::TX, L::TY, L::NPT);
 }
 
 // nsteps steps in one launch (sa set but for its step count): whether the
