@@ -29,9 +29,11 @@
 // wedge 1024 x 128^2 (NV = 8, HLLC, monopole) 10.9 -> 8.45 ms; thread
 // instructions per cell-update 2210 -> 990 (Sedov), 48 % of issue slots busy
 // with 16 warps per SM.  The two-warp barriers and the halo rows' staging then
-// gave 9.65 -> 9.34 and 7.81 -> 7.50 ms.  Bound now: fixed-latency dependences
-// at that occupancy (registers: 128 at NV = 5, 168 at NV = 6 and 8): 4 %
-// fewer instructions (the totals' sums of both halves in pairs) gave nothing.
+// gave 9.65 -> 9.34 and 7.81 -> 7.50 ms, the totals' widths staged with the
+// other axis-2 factors 9.33 -> 9.25.  Bound now: fixed-latency dependences at
+// that occupancy (registers: 128 at NV = 5, 168 at NV = 6 and 8): 4 % fewer
+// instructions (the totals' sums of both halves in pairs) gave nothing, and
+// sums by FP64 instructions cost 11.95 ms.
 #pragma once
 #include <algorithm>
 
@@ -63,7 +65,7 @@ struct March3Shape {
   // staged geometry: of the 32 columns and of the R rows
   enum { GX_SQ, GX_SF, GX_IW, GX_IR, GX_AF, GX_INVA, GX_GA, GX_QR, GX_GR, GX_G, GX_N };
   enum { GY_SQ, GY_SF, GY_IW, GY_IS, GY_BF, GY_INVB, GY_ZC, GY_GT, GY_QT, GY_N };
-  enum { GZ_SQ, GZ_SF, GZ_IW, GZ_IC, GZ_N };              // axis-2 factors of planes -1 .. len
+  enum { GZ_SQ, GZ_SF, GZ_IW, GZ_IC, GZ_VH, GZ_VL, GZ_N };  // axis-2 factors of planes -1 .. len
   static constexpr int MAXLEN = 128;                      // planes of a half at most
   static constexpr int off_y = 4 * NV * WPL;              // [v][row][lane]: upper state, then the flux
   static constexpr int off_uo = off_y + NV * R * 32;      // [v][thread] the own cell's conserved state
@@ -163,6 +165,11 @@ __global__ void __launch_bounds__(March3Shape<NSX, SPH>::NT, March3Shape<NSX, SP
     GZ[S::GZ_SQ * st + p] = make_f2(a.geo.sq[2][e0 + 2], a.geo.sq[2][e1 + 2]);
     GZ[S::GZ_SF * st + p] = make_f2(a.geo.sf[2][e0 + 2], a.geo.sf[2][e1 + 2]);
     GZ[S::GZ_IW * st + p] = make_f2(a.geo.inv_w[2][e0 + 2], a.geo.inv_w[2][e1 + 2]);
+    if (tsum) {
+      const float2 v0 = a.dv32[2][min(max(e0, 0), n2 - 1)], v1 = a.dv32[2][min(max(e1, 0), n2 - 1)];
+      GZ[S::GZ_VH * st + p] = make_f2(v0.x, v1.x);
+      GZ[S::GZ_VL * st + p] = make_f2(v0.y, v1.y);
+    }
     GZ[S::GZ_IC * st + p] = make_f2(a.geo.invc[min(max(e0, 0), n2 - 1)], a.geo.invc[min(max(e1, 0), n2 - 1)]);
   }
   if (tsum)
@@ -464,7 +471,8 @@ __global__ void __launch_bounds__(March3Shape<NSX, SPH>::NT, March3Shape<NSX, SP
               new_state2<3, NSX>(a, dt, gx[S::GX_G * 33], s_hfac, Uo, acc, Un);
               if (tsum) {
                 float2* ts = tsum + (row - 1) * TX + lane - 1;
-                const float2 t0 = a.dv32[2][z0 + i - 1], t1 = a.dv32[2][w1 ? zb + i - 1 : z0 + i - 1];
+                const f2 vh = gz(S::GZ_VH, i - 1), vl = gz(S::GZ_VL, i - 1);
+                const float2 t0 = make_float2(lo(vh), lo(vl)), t1 = make_float2(hi(vh), hi(vl));
 #pragma unroll
                 for (int v = 0; v < NV; ++v)
                   if (active(v)) {
