@@ -216,8 +216,10 @@ int hydro_step(hydro_t h, double dt);
 
 /* nsteps time steps with the time step computed on the device from the CFL
  * condition (dt = cfl/smax, clipped so that t does not pass t_end when
- * t_end > 0), without host round trips (captured as one CUDA graph after
- * the first call).  On error the state rolls back to the last good step.
+ * t_end > 0), without host round trips: one CUDA graph launch per step, or
+ * many steps in one cooperative launch on small 1D and 2D grids (ideal gas,
+ * no in-step totals, no monopole).  On error the state rolls back to the last
+ * good step.
  * *t_out (may be NULL) receives the time reached. */
 int hydro_run(hydro_t h, int nsteps, double cfl, double t_end, double* t_out);
 
@@ -227,16 +229,16 @@ int hydro_totals(hydro_t h, double* out_nv);
 /* Conserved totals accumulated inside the step (the FP32 form keeps its
  * bulk arithmetic in FP32 and its conservation sums in FP64).  With on != 0
  * every later step (hydro_step, hydro_run) also sums U dV of the cells it
- * updates: each CTA of the fused sweep in a fixed order over its cells,
- * into its own FP64 partial (the FP32 3D form sums each column of cells as
- * a compensated FP32 pair of exact products and converts the column's sum
- * to FP64; its totals equal the FP64 sums of the FP32 state to ~1e-14
- * relative);
+ * updates: each CTA in a fixed order over its cells, into its own FP64
+ * partial (the FP32 3D form, and in 2D its HLL and HLLC form, sums each
+ * column of cells as a compensated FP32 pair of exact products and converts
+ * the column's sum to FP64; its totals equal the FP64 sums of the FP32 state
+ * to ~1e-14 relative);
  * hydro_step_totals then sums the partials in a fixed order, so the
  * totals of the new state cost no second pass over it and are deterministic.
  * The partials take nv x (the most CTAs of any launch shape) doubles, and a
- * step with totals uses 8 nv bytes more shared memory per updated cell of a
- * CTA.  Rejected on a moving grid (HYDRO_ERR_UNSUPPORTED). */
+ * step with totals uses 8 nv bytes more shared memory per cell (3D: column
+ * of cells) of a CTA.  Rejected on a moving grid (HYDRO_ERR_UNSUPPORTED). */
 int hydro_set_step_totals(hydro_t h, int on);
 /* The totals (nv doubles, host) of the current state from the last step's
  * partials; HYDRO_ERR_ARG if the totals are off, or no step has completed

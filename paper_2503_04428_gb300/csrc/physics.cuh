@@ -306,22 +306,6 @@ __device__ __forceinline__ void to_prim_ct(const T* U, T* W, T& c2, T& t, const 
   for (int s = 0; s < NSX; ++s) W[2 + D + s] = U[2 + D + s] * ir;
 }
 
-template <typename T, int D, int NSX, typename G>
-__device__ __forceinline__ void to_prim_c2(const T* U, T* W, T& c2, const G& gas) {
-  const T rho = U[0];
-  const T ir = rcp<T>(rho);
-  T ke = T(0);
-#pragma unroll
-  for (int d = 0; d < D; ++d) {
-    W[1 + d] = U[1 + d] * ir;
-    ke += U[1 + d] * W[1 + d];
-  }
-  W[0] = rho;
-  gas.from_e(rho, U[1 + D] - T(0.5) * ke, W[1 + D], c2);
-#pragma unroll
-  for (int s = 0; s < NSX; ++s) W[2 + D + s] = U[2 + D + s] * ir;
-}
-
 // Internal energy per volume of the primitive state (rho, p) (Eq. 5 or 6).
 template <typename T, typename G>
 __device__ __forceinline__ T eint_of(const G& gas, T rho, T p) {
@@ -331,18 +315,6 @@ __device__ __forceinline__ T eint_of(const G& gas, T rho, T p) {
     return e;
   } else {
     return p * gas.igm1;
-  }
-}
-
-// Square of the sound speed at (rho, p): gamma p/rho (Eq. 5) or Eq. 7.
-template <typename T, typename G>
-__device__ __forceinline__ T sound2_of(const G& gas, T rho, T p) {
-  if constexpr (G::RAD) {
-    T e, c2;
-    gas.from_p(rho, p, e, c2);
-    return c2;
-  } else {
-    return qdiv(gas.g * p, rho);
   }
 }
 
