@@ -411,6 +411,7 @@ static SweepArgs<T> sweep_args(hydro_ctx* h, double dt_host, double cfl, double 
   a.t_end = t_end;
   a.zchunk = 1;  // (planned at the launch)
   a.ctrl = ctrl;
+  a.mirror = dt_host > 0.0 ? h->ctrl_back : nullptr;
   a.geo = geom_of<T>(h);
   a.xaxis = h->xaxis;
   a.halo[0] = (const T*)h->halo_d[0];
@@ -555,7 +556,7 @@ static int write_ctrl(hydro_ctx* h) {
 // After a launch sequence: read the status; on failure clear it (the state
 // is already the last good one) and report.
 static int check_status(hydro_ctx* h, const char* what) {
-  int st = read_ctrl(h);
+  int st = sync_ctrl(h);
   if (st) return st;
   const int code = h->ctrl_host->status;
   if (code == 0) return HYDRO_OK;
@@ -667,6 +668,7 @@ int hydro_common_init(hydro_ctx* h, int precision, void* stream) {
   }
   HCK(cudaMalloc(&h->ctrl, sizeof(Ctrl)));
   HCK(cudaMallocHost(&h->ctrl_host, sizeof(Ctrl)));
+  HCK(cudaMallocHost(&h->ctrl_back, sizeof(Ctrl)));
   HCK(cudaMalloc(&h->word, 2 * sizeof(unsigned long long)));
   HCK(cudaMallocHost(&h->word_host, 2 * sizeof(unsigned long long)));
   std::memset(h->ctrl_host, 0, sizeof(Ctrl));
@@ -1020,8 +1022,16 @@ int hydro_step(hydro_t h, double dt) {
     st = h->precision == 64 ? moving_geometry<double>(h, dt) : moving_geometry<float>(h, dt);
     if (st) return st;
   }
+  // the launch leaves the control block in ctrl_back (not if it found an
+  // earlier failure: then its ticket count stays as set here)
+  h->ctrl_back->done = ~0u;
   st = launch_step(h, dt, 0.0, 0.0, h->ctrl);
   if (st) return st;
+  HCK(cudaStreamSynchronize(h->stream));
+  if (h->ctrl_back->done == 0u) {
+    *h->ctrl_host = *h->ctrl_back;
+    h->ctrl_fresh = true;
+  }
   st = check_status(h, "hydro_step");
   h->step_tot_ok = h->step_tot && st == HYDRO_OK;
   if (moving) {
@@ -1212,6 +1222,7 @@ void hydro_destroy(hydro_t h) {
   h->arena.release();
   if (h->ctrl) cudaFree(h->ctrl);
   if (h->ctrl_host) cudaFreeHost(h->ctrl_host);
+  if (h->ctrl_back) cudaFreeHost(h->ctrl_back);
   if (h->word) cudaFree(h->word);
   if (h->word_host) cudaFreeHost(h->word_host);
   if (h->owns_stream && h->stream) cudaStreamDestroy(h->stream);

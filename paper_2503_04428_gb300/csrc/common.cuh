@@ -70,6 +70,7 @@ struct SweepArgs {
   const T* A;             // state buffer 0
   T* B;                   // state buffer 1 (in/out chosen by ctrl->cur)
   T* Aw;                  // writable alias of A
+  Ctrl* mirror;           // host memory that receives the control block at the end of the launch, or null
   int n[3];
   long long ncell;
   int bc[3][2];

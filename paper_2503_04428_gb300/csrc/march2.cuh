@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(March2Shape<NSX, SPH>::NT, March2Shape<NSX, SP
     reduce_totals<NV, NT, NT>(td);
     if (tid < NV) a.tot_part[(long long)tid * gridDim.x + blockIdx.x] = td[tid * NT];
   }
-  finish_step<NT>(a.ctrl, (double)smax, err, (unsigned long long)n_fb, 0ull, dtd);
+  finish_step<NT>(a.ctrl, (double)smax, err, (unsigned long long)n_fb, 0ull, dtd, a.mirror);
 }
 
 template <int NSX, int RS, bool SPH>

@@ -610,7 +610,7 @@ __global__ void __launch_bounds__(March3Shape<NSX, SPH>::NT, March3Shape<NSX, SP
     const long long cta = blockIdx.x + gridDim.x * ((long long)blockIdx.y + (long long)gridDim.y * blockIdx.z);
     if (tid < NV) a.tot_part[tid * ncta + cta] = td[tid * NI];
   }
-  finish_step<NT>(a.ctrl, (double)smax, err, (unsigned long long)n_fb, 0ull, s_dt);
+  finish_step<NT>(a.ctrl, (double)smax, err, (unsigned long long)n_fb, 0ull, s_dt, a.mirror);
 }
 
 template <int NSX, int RS, bool SPH>

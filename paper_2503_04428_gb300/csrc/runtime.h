@@ -63,6 +63,7 @@ struct hydro_ctx {
   void* buf[2] = {nullptr, nullptr};
   hydro::Ctrl* ctrl = nullptr;       // device control block
   hydro::Ctrl* ctrl_host = nullptr;  // pinned mirror
+  hydro::Ctrl* ctrl_back = nullptr;  // pinned: where a single step leaves the control block
   bool ctrl_fresh = false;           // the mirror holds the control block and nothing in flight changes it
   // a validation's result: status, then the speed's bits (device and pinned)
   unsigned long long* word = nullptr;

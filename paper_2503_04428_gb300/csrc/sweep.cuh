@@ -1217,12 +1217,13 @@ struct Sweep {
   }
 };
 
-// Block-wide reductions into the control block, then the last-CTA commit.
+// Block-wide reductions into the control block, then the last-CTA commit and,
+// where the host waits for this launch alone, the control block to the host.
 // (The maximum of the non-negative speeds is taken on their bit patterns:
 // integer compares, where an FP64 compare would occupy the FP64 pipe.)
 template <int NT>
 __device__ void finish_step(Ctrl* ctrl, double speed, int err, unsigned long long fb,
-                            unsigned long long it, double dt) {
+                            unsigned long long it, double dt, Ctrl* mirror) {
   __shared__ unsigned long long red_s[NT / 32];
   __shared__ int red_e[NT / 32];
   __shared__ unsigned long long red_f[NT / 32], red_i[NT / 32];
@@ -1278,6 +1279,13 @@ __device__ void finish_step(Ctrl* ctrl, double speed, int err, unsigned long lon
         vc->cur = vc->cur ^ 1;
       }
       vc->done = 0;
+      if (mirror) {
+        // (a copy by the copy engine after the kernel takes 4 us longer)
+        const volatile unsigned long long* const from = reinterpret_cast<const volatile unsigned long long*>(ctrl);
+        volatile unsigned long long* const to = reinterpret_cast<volatile unsigned long long*>(mirror);
+#pragma unroll
+        for (int i = 0; i < (int)(sizeof(Ctrl) / 8); ++i) to[i] = from[i];
+      }
       __threadfence();
     }
   }
@@ -1403,7 +1411,7 @@ __global__ void __launch_bounds__(SweepShape<T, DIM, NSX, SMALL>::NT,
     if (threadIdx.x < S::NV) args.tot_part[threadIdx.x * ncta + cta] = sw.tsum[threadIdx.x * S::NI];
   }
   finish_step<S::NT>(args.ctrl, (double)sw.smax, sw.err, sw.n_fallback,
-                     (MODE & 1) ? (unsigned long long)sw.t_iters : sw.n_iters, s_dt);
+                     (MODE & 1) ? (unsigned long long)sw.t_iters : sw.n_iters, s_dt, args.mirror);
 }
 
 // Several steps of a small 1D or 2D grid in one cooperative launch.  A step of
