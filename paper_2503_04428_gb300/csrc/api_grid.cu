@@ -350,8 +350,12 @@ Gas<T> make_gas(double gm) {
   g.Bq = (T)((gm - 1.0) / (gm + 1.0));
   g.two_gm1 = (T)(2.0 / (gm - 1.0));
   g.ig = (T)(1.0 / gm);
+  // A root only where 1/z is the integer to the rounding of gamma and of this
+  // quotient (a few 1e-16 of it): x^(1/n) next to the constants of a gamma
+  // 3e-11 away moved p* by 4e-10 in FP64.  FP32 rounds gamma to 6e-8 anyway.
   const double iz = 2.0 * gm / (gm - 1.0), n = std::round(iz);
-  g.root = std::fabs(iz - n) < 1e-9 && n >= 4.0 && n <= 8.0 ? (int)n : 0;
+  const double tol = sizeof(T) == 8 ? 1e-15 * n : 1e-9;
+  g.root = std::fabs(iz - n) <= tol && n >= 4.0 && n <= 8.0 ? (int)n : 0;
   return g;
 }
 template Gas<float> make_gas<float>(double);

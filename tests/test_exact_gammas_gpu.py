@@ -36,3 +36,21 @@ def test_star_states(hydro_lib, gamma, precision):
         p, u = O.exact_star(g, WL[k], WR[k])[:2]
         assert abs(ps[k] - p) <= tol * p, (k, ps[k], p)
         assert abs(us[k] - u) <= tol * max(abs(u), cmax[k]), (k, us[k], u)
+
+
+@pytest.mark.parametrize("gamma", [1.3333333333, 1.3333333334, 1.6666666667, 1.6666666666, 1.40000000003, 1.5 + 1e-11,
+                                   2.0 - 1e-10, 1.4 + 2e-14])
+def test_gammas_next_to_a_root(hydro_lib, gamma):
+    """FP64 star states at gammas whose 1/z is nearly, but not, an integer:
+    the powers have to be those of the gamma given, to the same 1e-11."""
+    states = [((1.0, 0.0, 1.0), (0.125, 0.0, 0.1)), ((1.0, -2.0, 0.4), (1.0, 2.0, 0.4)),
+              ((1.0, -1.0, 1e3), (2.0, 1.0, 1e-2)), ((3.0, 0.5, 2.0), (1.0, 0.9, 1.9))]
+    W = [np.array([s[k] for s in states]) for k in range(2)]
+    c = [np.sqrt(gamma * w[:, 2] / w[:, 0]) for w in W]
+    keep = W[1][:, 1] - W[0][:, 1] < 0.95 * 2 / (gamma - 1) * (c[0] + c[1])  # (the second is a vacuum at gamma = 2)
+    W = [w[keep] for w in W]
+    ps, us, _ = hydro_lib.hydro_exact_solve(W[0], W[1], gamma)
+    for k in range(len(ps)):
+        p, u = O.exact_star(gamma, W[0][k], W[1][k])[:2]
+        assert abs(ps[k] - p) <= 1e-11 * p, (k, ps[k], p)
+        assert abs(us[k] - u) <= 1e-11 * max(abs(u), np.sqrt(gamma * W[0][k, 2] / W[0][k, 0])), (k, us[k], u)
