@@ -222,6 +222,7 @@ struct Sweep {
   T fzb3 = T(0), tth = T(0), x2 = T(0), s3 = T(0);
   T Ucell[MULTI ? NV : 1];  // several steps per launch: the owned cell's conserved state
   T aq1 = T(0), aq2 = T(0);  // dual energy: divergences of u e and of u (times dt^-1)
+  T topen = T(0);            // radiation EoS: the open cell's temperature (its plane's slot is refilled before it closes)
 
   __device__ Sweep(const SweepArgs<T>& args, T* smem) : a(args) {
     Ws = smem;
@@ -983,6 +984,7 @@ struct Sweep {
     const T Afl = gx(S::GX_AF, i + 1), Afh = gx(S::GX_AF, i + 2), ia = gx(S::GX_INVA, i + 1);
     constexpr bool dual = DUAL;
     const bool sph = a.spherical;  // (Cartesian area factors are 1)
+    if constexpr (EOS == 1) topen = WT[(wslot(gz) * EY + j + HY) * EX + i + 2];
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       const T fl = XL[v * NFX + fx], fh = XL[v * NFX + fx + 1];
@@ -1155,7 +1157,7 @@ struct Sweep {
     if constexpr (EOS == 1) {
       T tn;
       int k = 0;
-      to_prim_ct<T, DIM, NSX>(Un, Wn, c2n, tn, a.grad, WT[(wslot(gz) * EY + j + HY) * EX + i + 2], &k);
+      to_prim_ct<T, DIM, NSX>(Un, Wn, c2n, tn, a.grad, topen, &k);
       t_iters += k;
     } else {
       to_prim<T, DIM, NSX>(Un, Wn, a.gas);
