@@ -128,6 +128,24 @@ struct TempIts {
   T t;
   int its;
 };
+// GasRad::temperature from the upper bound, for a start so far below the root
+// that 60 steps do not reach it: the first then lands far above (in FP32 it
+// may overflow), where each further one takes off a quarter at most.  (Of its
+// own: the bound tested at each step cost the radiation wedge 2-6 %, a second
+// pass of the usual loop 3 %, this 0.6 %.)
+template <typename T>
+static __device__ __noinline__ TempIts<T> far_temperature(T c1, T c4, T y) {
+  T t = qdiv(y, c1);
+  if (c4 > T(0)) t = min_of(t, dsqrt(dsqrt(qdiv(y, c4))));
+  int it = 0;
+  for (; it < 60; ++it) {
+    const T t3 = t * t * t;
+    const T tn = t - qdiv(c1 * t + c4 * t3 * t - y, c1 + T(4) * c4 * t3);
+    if (!(tn < t)) break;
+    t = tn;
+  }
+  return {t, 60 + it};
+}
 // The solve of GasRad::temperature.  Out of line: a step has 15 sites of it,
 // and inlined they overflowed the instruction cache (1.8 stalls per issue).
 template <typename T>
@@ -149,6 +167,7 @@ static __device__ __noinline__ TempIts<T> newton_temperature(T c1, T c4, T y, T 
       conv = true;
     }
   }
+  if (it == 60 && t0 > T(0)) return far_temperature<T>(c1, c4, y);
   return {t, it < 60 ? it + 1 : 60};
 }
 
@@ -169,7 +188,8 @@ struct GasRad : Gas<T> {
   // is increasing and convex in t > 0, so Newton from the upper bound
   // min(y/c1, (y/c4)^(1/4)) descends monotonically to the root; from any
   // other positive start t0 (a nearby temperature the caller knows) the first
-  // step lands above the root and the descent follows.  It stops when the
+  // step lands above the root and the descent follows (from that bound again
+  // if 60 steps do not end it: a start below a few hundredths of the root).  It stops when the
   // relative step is below temp_tol and takes one more step; in FP32 the step
   // below temp_tol (1e-6) is the last (quadratic convergence leaves that
   // iterate ~1e-12 from the root, below FP32 resolution).  y <= 0 gives

@@ -12,6 +12,7 @@ import pytest
 import oracle as O
 from paper_2503_04428_gb300 import workloads as wl
 
+from parity import check
 from test_parity_grid import step_compare
 
 pytestmark = pytest.mark.gpu
@@ -109,3 +110,22 @@ def test_rad_temperature_layers(hydro_lib, precision, riemann):
         its.append(g.stats()["newton_iters"])
         g.close()
     assert max(its) <= 1.2 * min(its), its
+
+
+@pytest.mark.parametrize("precision", [64, 32])
+@pytest.mark.parametrize("riemann", [O.HLL, O.HLLC])
+def test_rad_cold_cells_heated_in_one_step(hydro_lib, precision, riemann):
+    """Cold layers beside layers a thousand times hotter: one CFL step heats their edge cells by a factor of hundreds,
+    and the temperature iteration, which starts at the cold value, has to arrive: the state and the next signal speed
+    are the oracle's."""
+    case = _layers(2, 1000.0, riemann, n=18)
+    if precision == 32:
+        case["U"] = case["U"].astype(np.float32).astype(np.float64)
+    s = O.solver_from_case(case)
+    g = hydro_lib.Grid.from_case(case, precision)
+    dt = s.cfl_dt(0.4)
+    s.step(dt)
+    g.step(dt)
+    check(s.get_state(), g.get_state(), 3, case["gamma"], precision)
+    assert g.cfl_dt(0.4) == pytest.approx(s.cfl_dt(0.4), rel=1e-11 if precision == 64 else 1e-5)
+    g.close()
