@@ -1464,7 +1464,7 @@ __global__ void __launch_bounds__(SweepShape<T, DIM, NSX, true>::NT, 1)
   // thread 0: the state's speed, its time, and the steps done
   double smax = vc->smax_cur, t = vc->t, last_dt = vc->last_dt;
   constexpr unsigned long long FAILED = 0x7ff8000000000000ull;
-  const bool idle = vc->status != 0;  // (an earlier failure; constant until a step of this launch fails)
+  const bool idle = vc->status != 0;  // (an earlier failure: written by this launch only after all have read it)
   int done = 0;
   for (;;) {
     if (threadIdx.x == 0) {
@@ -1520,13 +1520,11 @@ __global__ void __launch_bounds__(SweepShape<T, DIM, NSX, true>::NT, 1)
           bits = bits > s_speed[w] ? bits : s_speed[w];
           err = err ? err : s_err[w];
         }
-        if (err) {
-          bits = FAILED;
-          if (atomicCAS(&ctrl->status, 0, err) == 0) ctrl->err_step = step0 + done;
-        }
+        if (err) bits = FAILED;
         asm volatile("st.release.gpu.global.u64 [%0], %1;\n" ::"l"(speed + cta), "l"(bits | use) : "memory");
       }
       unsigned long long m = 0ull;
+      bool late = false;
       for (unsigned int c = lane; c < ctas; c += 32) {
         unsigned long long b = 0ull;
         int poll = 0;
@@ -1535,7 +1533,7 @@ __global__ void __launch_bounds__(SweepShape<T, DIM, NSX, true>::NT, 1)
         } while (((b ^ use) >> 63) != 0ull && ++poll < (1 << 22));
         if (((b ^ use) >> 63) != 0ull) {  // the bounded wait expired
           b = FAILED;
-          if (atomicCAS(&ctrl->status, 0, ST_STEP_TIMEOUT) == 0) ctrl->err_step = step0 + done;
+          late = true;
         }
         b &= ~(1ull << 63);
         m = m > b ? m : b;
@@ -1544,6 +1542,13 @@ __global__ void __launch_bounds__(SweepShape<T, DIM, NSX, true>::NT, 1)
       for (int o = 16; o > 0; o >>= 1) {
         const unsigned long long b2 = __shfl_xor_sync(0xffffffffu, m, o);
         m = m > b2 ? m : b2;
+      }
+      // The status only now that every CTA has published: each has read it for
+      // `idle` before that, and one that took this failure for an earlier one
+      // would end without its word and leave the others to their whole wait.
+      late = __any_sync(0xffffffffu, late);
+      if (lane == 0 && (err != 0 || late)) {
+        if (atomicCAS(&ctrl->status, 0, err ? err : ST_STEP_TIMEOUT) == 0) ctrl->err_step = step0 + done;
       }
       if (m < FAILED) smax = __longlong_as_double((long long)m);
       if (lane == 0) s_go = m < FAILED;

@@ -5,6 +5,8 @@ of fewer tiles than the GPU has SMs, at and around multiples of the tiles (28
 cells in 1D, 8 x 8 in 2D), with every solver, precision and scalar count, and
 a grid on either side of the rule that picks the tile.
 """
+import time
+
 import numpy as np
 import pytest
 
@@ -92,3 +94,23 @@ def test_failed_run_keeps_the_last_good_state(hydro_lib, n):
     assert a.stats()["steps"] == good + 3
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("n", [[4000], [100, 90]])
+def test_failure_in_the_first_step_ends_the_run_at_once(hydro_lib, n):
+    """A first step that fails in one corner of the grid ends a many-step run without any CTA waiting out its bound (4
+    million polls, seconds), however late the others start: a hundred runs, each of milliseconds (a tenth of a second
+    allowed), each leaving the state as it was."""
+    case = wl.smooth_random(len(n), n, 0, seed=5, amp=0.01, riemann=O.HLLC, bc=[(T, T)] * len(n))
+    case["U"][1, ..., :2] = -30.0 * case["U"][0, ..., :2]  # two columns torn off
+    case["U"][-1, ..., :2] += 0.5 * 900.0 * case["U"][0, ..., :2]
+    g = hydro_lib.Grid.from_case(case, 64)
+    U = g.get_state()
+    for _ in range(100):
+        t = time.perf_counter()
+        with pytest.raises(hydro_lib.HydroError) as e:
+            g.run(50, 5.0)
+        assert time.perf_counter() - t < 0.1
+        assert e.value.status in (hydro_lib.HYDRO_ERR_NEGATIVE_STATE, hydro_lib.HYDRO_ERR_NONFINITE)
+        assert g.stats()["steps"] == 0 and np.array_equal(g.get_state(), U)
+    g.close()
