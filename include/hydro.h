@@ -47,7 +47,9 @@ typedef enum {
   HYDRO_ERR_NEGATIVE_STATE = -3,  /* a cell reached rho <= 0 or P <= 0 */
   HYDRO_ERR_NONFINITE = -4,       /* NaN or Inf in the state */
   HYDRO_ERR_NEWTON = -5,          /* exact-solver Newton did not converge in 100 iterations */
-  HYDRO_ERR_TIMEOUT = -6,         /* a bounded device wait expired (batched: a window copy never landed) */
+  HYDRO_ERR_TIMEOUT = -6,         /* a bounded device wait expired (batched: a window copy never landed;
+                                   * grids: another CTA of a many-step launch never reported, or the
+                                   * state was lost that way and none has been set since) */
   HYDRO_ERR_OOM = -7,             /* device allocation failed */
   HYDRO_ERR_VACUUM = -8,          /* exact solver: the data generate vacuum */
   HYDRO_ERR_UNSUPPORTED = -9      /* combination not built (see message) */
@@ -219,9 +221,18 @@ int hydro_step(hydro_t h, double dt);
  * t_end > 0), without host round trips: one CUDA graph launch per step, or
  * many steps in one cooperative launch on small 1D and 2D grids (ideal gas,
  * no in-step totals, no monopole).  On error the state rolls back to the last
- * good step.
+ * good step; after HYDRO_ERR_TIMEOUT alone (a bounded wait between the CTAs of
+ * such a launch expired, which a working GPU does not do) there is no good
+ * state any more, and every call that needs one returns HYDRO_ERR_TIMEOUT
+ * until hydro_set_state.
  * *t_out (may be NULL) receives the time reached. */
 int hydro_run(hydro_t h, int nsteps, double cfl, double t_end, double* t_out);
+
+/* Bound of the waits between the CTAs of a many-step launch of hydro_run, in
+ * polls of device memory (about 1 us each; at the start 2^22).  With 0 every
+ * such wait expires at once.  The paper has no counterpart: this serves tests
+ * of the failure path. */
+int hydro_set_step_wait(hydro_t h, int polls);
 
 /* Conserved totals sum_cells U dV, FP64, deterministic order; out has nv entries. */
 int hydro_totals(hydro_t h, double* out_nv);

@@ -513,7 +513,7 @@ static int launch_steps_t(hydro_ctx* h, int nsteps, double cfl, double t_end, bo
     return h->dim == 1 ? steps_dispatch<T, 1>(a, sa, h->nsx, h->riemann, h->stream, &h->shape, taken)
                        : steps_dispatch<T, 2>(a, sa, h->nsx, h->riemann, h->stream, &h->shape, taken);
   };
-  StepsArgs sa = {nullptr, 0};
+  StepsArgs sa = {nullptr, 0, h->step_polls};
   cudaError_t e = launch(sa);
   if (e != cudaSuccess) return cuda_fail(e, "sweep launch");
   if (!*taken) return HYDRO_OK;
@@ -557,8 +557,15 @@ static int write_ctrl(hydro_ctx* h) {
   return HYDRO_OK;
 }
 
+// Whether the handle's state was lost to an expired wait (check_status).
+static int refuse_lost(const hydro_ctx* h, const char* what) {
+  if (!h->lost) return HYDRO_OK;
+  set_error(std::string(what) + ": the state was lost when a device wait expired (set it again)");
+  return HYDRO_ERR_TIMEOUT;
+}
+
 // After a launch sequence: read the status; on failure clear it (the state
-// is already the last good one) and report.
+// is already the last good one, but for an expired wait) and report.
 static int check_status(hydro_ctx* h, const char* what) {
   int st = sync_ctrl(h);
   if (st) return st;
@@ -570,7 +577,9 @@ static int check_status(hydro_ctx* h, const char* what) {
         : code == HYDRO_ERR_NONFINITE    ? " (non-finite state)"
         : code == HYDRO_ERR_NEWTON       ? " (Newton did not converge)"
         : code == HYDRO_ERR_VACUUM       ? " (vacuum generated)"
+        : code == HYDRO_ERR_TIMEOUT      ? " (a bounded device wait expired: the state is lost)"
                                          : "");
+  if (code == HYDRO_ERR_TIMEOUT) h->lost = true;
   h->ctrl_host->status = 0;
   h->ctrl_host->done = 0;
   h->ctrl_host->err_step = -1;
@@ -894,7 +903,8 @@ int hydro_set_halo(hydro_t h, int axis, int side, const void* halo, int where) {
 int hydro_get_boundary(hydro_t h, int axis, int side, void* out, int where) {
   if (!h || h->batched || !out) return arg_error("hydro_get_boundary: grid handle and output required");
   if (axis < 0 || axis >= h->dim || side < 0 || side > 1) return arg_error("hydro_get_boundary: bad axis or side");
-  int st;
+  int st = refuse_lost(h, "hydro_get_boundary");
+  if (st) return st;
   if (!h->pack_d && (st = h->arena.alloc(&h->pack_d, (size_t)halo_bytes(h, axis)))) return st;
   if (h->xaxis >= 0 && axis != h->xaxis) return arg_error("hydro_get_boundary: not the exchanged axis");
   void* dst = where == HYDRO_DEVICE ? out : h->pack_d;
@@ -920,6 +930,7 @@ int hydro_shell_masses(hydro_t h, double* m_out) {
   if (!h || h->batched || !m_out) return arg_error("hydro_shell_masses: grid handle and output required");
   if (h->gravity != HYDRO_GRAV_POINT_MONOPOLE)
     return arg_error("hydro_shell_masses: the handle has no monopole gravity");
+  if (const int st = refuse_lost(h, "hydro_shell_masses")) return st;
   dim3 gb((h->n[0] + 31) / 32, h->shell_nchunks), tb(32, 8);
   if (h->precision == 64)
     shell_partial_kernel<double><<<gb, tb, 0, h->stream>>>(h->ctrl, (const double*)h->buf[0],
@@ -976,6 +987,7 @@ int hydro_set_state(hydro_t h, const void* U, int where) {
   h->ctrl_host->status = 0;
   h->ctrl_host->done = 0;
   h->ctrl_host->err_step = -1;
+  h->lost = false;
   h->step_tot_ok = false;  // the step totals describe an earlier state
   return write_ctrl(h);
 }
@@ -983,7 +995,8 @@ int hydro_set_state(hydro_t h, const void* U, int where) {
 int hydro_get_state(hydro_t h, void* U_out, int where) {
   if (!h || !U_out) return arg_error("hydro_get_state: null argument");
   if (h->batched) return hydro_batch_get_state_impl(h, U_out, where);
-  int st = sync_ctrl(h);
+  int st = refuse_lost(h, "hydro_get_state");
+  if (st || (st = sync_ctrl(h))) return st;
   if (st) return st;
   const size_t bytes = (size_t)h->nv * h->ncell * h->esize;
   HCK(cudaMemcpyAsync(U_out, h->buf[h->ctrl_host->cur], bytes,
@@ -1003,7 +1016,8 @@ int hydro_set_time(hydro_t h, double t) {
 int hydro_cfl_dt(hydro_t h, double cfl, double* dt_out) {
   if (!h || !dt_out || !(cfl > 0)) return arg_error("hydro_cfl_dt: bad argument");
   if (h->batched) return arg_error("hydro_cfl_dt: batched handles use per-tube time steps");
-  int st = sync_ctrl(h);
+  int st = refuse_lost(h, "hydro_cfl_dt");
+  if (st || (st = sync_ctrl(h))) return st;
   if (st) return st;
   if (!(h->ctrl_host->smax_cur > 0.0)) return arg_error("hydro_cfl_dt: no signal speed (state not set?)");
   *dt_out = cfl / h->ctrl_host->smax_cur;
@@ -1020,7 +1034,8 @@ static int move_faces(hydro_ctx* h, double dt) {
 int hydro_step(hydro_t h, double dt) {
   if (!h || h->batched) return arg_error("hydro_step: grid handle required");
   if (!(dt > 0.0) || !std::isfinite(dt)) return arg_error("hydro_step: dt must be positive and finite");
-  int st;
+  int st = refuse_lost(h, "hydro_step");
+  if (st) return st;
   const bool moving = h->maxis >= 0 && h->wgrid != 0.0;
   if (moving && h->coords == HYDRO_SPHERICAL) {
     st = h->precision == 64 ? moving_geometry<double>(h, dt) : moving_geometry<float>(h, dt);
@@ -1089,9 +1104,10 @@ int hydro_run(hydro_t h, int nsteps, double cfl, double t_end, double* t_out) {
               "use hydro_step");
     return HYDRO_ERR_UNSUPPORTED;
   }
+  int st = refuse_lost(h, "hydro_run");
+  if (st) return st;
   if (h->maxis >= 0 && h->wgrid != 0.0) {
     // a moving grid's geometry follows each step's dt: steps driven from the host
-    int st;
     for (int s = 0; s < nsteps; ++s) {
       if ((st = sync_ctrl(h))) return st;
       const double t0 = h->ctrl_host->t;
@@ -1104,7 +1120,6 @@ int hydro_run(hydro_t h, int nsteps, double cfl, double t_end, double* t_out) {
     if (t_out) *t_out = h->ctrl_host->t;
     return HYDRO_OK;
   }
-  int st;
   bool taken = false;
   st = h->precision == 64 ? launch_steps_t<double>(h, nsteps, cfl, t_end, &taken)
                           : launch_steps_t<float>(h, nsteps, cfl, t_end, &taken);
@@ -1140,6 +1155,12 @@ int hydro_run(hydro_t h, int nsteps, double cfl, double t_end, double* t_out) {
   else if (h->ctrl_host->step > step0) h->step_tot_ok = h->step_tot;
   if (t_out) *t_out = h->ctrl_host->t;
   return st;
+}
+
+int hydro_set_step_wait(hydro_t h, int polls) {
+  if (!h || h->batched || polls < 0) return arg_error("hydro_set_step_wait: grid handle and polls >= 0 required");
+  h->step_polls = polls;
+  return HYDRO_OK;
 }
 
 int hydro_set_step_totals(hydro_t h, int on) {
@@ -1179,7 +1200,8 @@ int hydro_step_totals(hydro_t h, double* out_nv) {
 int hydro_totals(hydro_t h, double* out_nv) {
   if (!h || !out_nv) return arg_error("hydro_totals: null argument");
   if (h->batched) return arg_error("hydro_totals: grid handle required");
-  int st = sync_ctrl(h);
+  int st = refuse_lost(h, "hydro_totals");
+  if (st || (st = sync_ctrl(h))) return st;
   if (st) return st;
   dim3 grid(h->tot_blocks, h->nv);
   if (h->precision == 64)

@@ -171,6 +171,7 @@ cudaError_t sweep_dispatch(const SweepArgs<T>& a, int nsx, int rs, cudaStream_t 
 struct StepsArgs {
   unsigned long long* speed;  // 2 x CTAs words, zeroed before the launch: by step parity, the CTAs' speed maxima
   int nsteps;
+  int polls;  // bound of the wait for another CTA's word
 };
 template <typename T, int DIM>
 cudaError_t steps_dispatch(const SweepArgs<T>& a, const StepsArgs& sa, int nsx, int rs, cudaStream_t s,

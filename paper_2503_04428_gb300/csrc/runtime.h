@@ -90,6 +90,8 @@ struct hydro_ctx {
   double* step_tot_part = nullptr;
   hydro::LaunchShape shape;  // of the last step launched
   void* steps_speed = nullptr;  // several steps per launch: the words the CTAs publish
+  int step_polls = 1 << 22;     // and the bound of their waits for them
+  bool lost = false;            // such a wait expired: there is no state until one is set
   // domain decomposition (Sect. 3.3.1): exchanged sides of axis xaxis, the
   // two face coordinates beyond each (nearest first), their halo buffers
   // [nv][2][cross section] on the device, and the monopole's inner mass

@@ -1426,7 +1426,9 @@ __global__ void __launch_bounds__(SweepShape<T, DIM, NSX, SMALL>::NT,
 // steps are apart, zeroed before the launch, and each use flips the sign, so
 // none is overwritten before all have read it (8.8 us per step; a counter
 // beside the words cost 0.2 more).  A step that fails in a CTA
-// publishes NaN: every CTA ends with the state before it.  The buffers
+// publishes NaN: every CTA ends with the state before it.  (A wait that
+// expires ends its CTA alone, and the others may be a step further by the
+// time they miss its word: the host takes the state for lost.)  The buffers
 // alternate as between launches.
 constexpr int ST_STEP_TIMEOUT = -6;  // HYDRO_ERR_TIMEOUT
 
@@ -1526,11 +1528,9 @@ __global__ void __launch_bounds__(SweepShape<T, DIM, NSX, true>::NT, 1)
       unsigned long long m = 0ull;
       bool late = false;
       for (unsigned int c = lane; c < ctas; c += 32) {
-        unsigned long long b = 0ull;
-        int poll = 0;
-        do {
+        unsigned long long b = ~use;
+        for (int poll = 0; poll < sa.polls && ((b ^ use) >> 63) != 0ull; ++poll)
           asm volatile("ld.acquire.gpu.global.u64 %0, [%1];\n" : "=l"(b) : "l"(speed + c) : "memory");
-        } while (((b ^ use) >> 63) != 0ull && ++poll < (1 << 22));
         if (((b ^ use) >> 63) != 0ull) {  // the bounded wait expired
           b = FAILED;
           late = true;

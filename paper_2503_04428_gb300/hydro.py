@@ -93,6 +93,7 @@ _SIGS = {
     "hydro_exact_sample": [_D, _D, C.c_long, C.c_double, C.POINTER(C.c_longlong), _D, C.c_long, _D],
     "hydro_batch_times": [_VP, _D],
     "hydro_set_step_totals": [_VP, C.c_int],
+    "hydro_set_step_wait": [_VP, C.c_int],
     "hydro_step_totals": [_VP, _D],
     "hydro_batch_set_launch": [_VP, C.c_int, C.c_int, C.c_int],
     "hydro_set_exchange": [_VP, C.c_int, C.c_int, _D],
@@ -435,6 +436,10 @@ class Grid:
     def set_step_totals(self, on=True):
         """Accumulate the conserved totals inside every later step (hydro_set_step_totals)."""
         _call("hydro_set_step_totals", self.h, 1 if on else 0)
+
+    def set_step_wait(self, polls):
+        """Bound of the waits inside a many-step launch of run (hydro_set_step_wait)."""
+        _call("hydro_set_step_wait", self.h, int(polls))
 
     def step_totals(self):
         """Totals of the current state from the last step's in-step partials (hydro_step_totals)."""

@@ -114,3 +114,30 @@ def test_failure_in_the_first_step_ends_the_run_at_once(hydro_lib, n):
         assert e.value.status in (hydro_lib.HYDRO_ERR_NEGATIVE_STATE, hydro_lib.HYDRO_ERR_NONFINITE)
         assert g.stats()["steps"] == 0 and np.array_equal(g.get_state(), U)
     g.close()
+
+
+@pytest.mark.parametrize("n", [[20], [500], [40, 24]])
+def test_an_expired_wait_loses_the_state(hydro_lib, n):
+    """A many-step run whose waits expire (bound 0: no word is ever seen) reports HYDRO_ERR_TIMEOUT, and since its CTAs
+    may have ended at different steps, every call that needs the state refuses until one is set; then the handle works."""
+    H = hydro_lib
+    case = wl.smooth_random(len(n), n, 0, seed=5, riemann=O.HLLC)
+    g = H.Grid.from_case(case, 64)
+    g.set_step_wait(0)
+    with pytest.raises(H.HydroError) as e:
+        g.run(10, 0.4)
+    assert e.value.status == H.HYDRO_ERR_TIMEOUT and "wait" in str(e.value)
+    for call in (lambda: g.run(1, 0.4), lambda: g.step(1e-6), g.get_state, lambda: g.cfl_dt(0.4), g.totals,
+                 lambda: g.get_boundary(0, 0)):
+        with pytest.raises(H.HydroError) as e:
+            call()
+        assert e.value.status == H.HYDRO_ERR_TIMEOUT
+    g.set_step_wait(1 << 22)
+    g.set_state(case["U"])
+    steps = g.stats()["steps"]
+    assert np.array_equal(g.get_state(), case["U"].reshape(g.shape))
+    g.run(10, 0.4)
+    assert g.stats()["steps"] == steps + 10
+    with pytest.raises(H.HydroError):
+        g.set_step_wait(-1)
+    g.close()
