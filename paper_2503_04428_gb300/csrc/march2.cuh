@@ -353,10 +353,10 @@ __global__ void __launch_bounds__(March2Shape<NSX, SPH>::NT, March2Shape<NSX, SP
   }
   __syncthreads();
   if (tsum) {
-    // the columns' sums times dvol[0] in FP64, in place, then a tree in a
-    // fixed order per variable
+    // the columns' sums times dvol[0] (and the absent axis's dvol[2]) in FP64,
+    // in place, then a tree in a fixed order per variable
     double* const td = reinterpret_cast<double*>(tsum);
-    const double w = lown ? a.dvol[0][gi] : 0.0;
+    const double w = lown ? a.dvol[0][gi] * a.dvol[2][0] : 0.0;
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       const float2 c = tsum[v * NT + tid];

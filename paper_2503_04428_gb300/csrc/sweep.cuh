@@ -1143,9 +1143,8 @@ struct Sweep {
           if (v < nvact) add_column_sum(ts[v * NI + o], (float)Un[v], z);
       } else {
         // FP64 sums of U dV
-        double dV = a.dvol[0][gi];
-        if constexpr (DIM >= 2) dV *= a.dvol[1][gj];
-        if constexpr (DIM == 3) dV *= a.dvol[2][gz];
+        // (an absent axis has one factor: 1, or the angle it spans)
+        const double dV = a.dvol[0][gi] * a.dvol[1][DIM >= 2 ? gj : 0] * a.dvol[2][DIM == 3 ? gz : 0];
 #pragma unroll
         for (int v = 0; v < NV; ++v)
           if (v < nvact) tsum[v * NI + o] += (double)Un[v] * dV;

@@ -144,3 +144,23 @@ def test_fp32_step_totals_are_exact_sums_of_the_fp32_state(hydro_lib, k):
     err = np.abs(tg - exact) / scale
     print(name, "worst |step total - FP64 sum| / sum |U| dV: %.2e" % err.max())
     assert err.max() <= 1e-12, (name, err)
+
+
+@pytest.mark.parametrize("precision", [64, 32])
+@pytest.mark.parametrize("riemann", [O.HLL, O.HLLC, O.EXACT])
+@pytest.mark.parametrize("n", [(40,), (300,), (33, 12), (200, 150)])
+def test_totals_span_the_absent_angles(hydro_lib, n, riemann, precision):
+    """A spherical grid without an angular axis spans that angle: its in-step totals are those of the separate pass and
+    of the oracle (1D: all of 4 pi; 2D: 2 pi in azimuth), for every form of the step."""
+    case = wl.sphere_state(*n, n_scalars=1, dim=len(n), riemann=riemann)
+    case["U"] = case["U"].astype(np.float32).astype(np.float64)
+    s = O.solver_from_case(case)
+    g = hydro_lib.Grid.from_case(case, precision)
+    g.set_step_totals(True)
+    dt = s.cfl_dt(0.4)
+    s.step(dt)
+    g.step(dt)
+    tol = 1e-12 if precision == 64 else 1e-5
+    assert _rel(g.step_totals(), s.totals()) <= tol
+    assert _rel(g.step_totals(), g.totals()) <= (1e-13 if precision == 64 else 1e-6)
+    g.close()
