@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(March2Shape<NSX, SPH>::NT, March2Shape<NSX, SP
   constexpr unsigned FULL = 0xffffffffu;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   f2* const Ws = reinterpret_cast<f2*>(smem_raw);
-  float2* const tsum = a.tot_part ? reinterpret_cast<float2*>(smem_raw + S::smem_bytes) : nullptr;
+  double* const tsum = a.tot_part ? reinterpret_cast<double*>(smem_raw + S::smem_bytes) : nullptr;  // [v][thread]
   __shared__ double s_dt;
   __shared__ float s_hfac;
   const volatile Ctrl* vc = a.ctrl;
@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(March2Shape<NSX, SPH>::NT, March2Shape<NSX, SP
   f2* const ring = Ws + tid;  // own slots: row i at ((i + 2) & 3) * NV * NT, variable v at v * NT
   if (tsum)
 #pragma unroll
-    for (int v = 0; v < NV; ++v) tsum[v * NT + tid] = make_float2(0.f, 0.f);
+    for (int v = 0; v < NV; ++v) tsum[v * NT + tid] = 0.0;
   if (!active(NV - 1))
 #pragma unroll
     for (int r = 0; r < 4; ++r) ring[(r * NV + NV - 1) * NT] = both(0.f);
@@ -275,12 +275,16 @@ __global__ void __launch_bounds__(March2Shape<NSX, SPH>::NT, March2Shape<NSX, SP
             for (int v = 0; v < NV; ++v) Uo[v] = ring[(((i + 1) & 3) * NV + v) * NT];
             new_state2<2, NSX>(a, dt, gx[S::GX_G * 33], s_hfac, Uo, acc, Un);
             if (tsum) {
-              const float2 t0 = a.dv32[1][z0 + i - 1], t1 = a.dv32[1][w1 ? zb + i - 1 : z0 + i - 1];
+              // the thread's sums of U dvol[1], in FP64 (512 x 1536: 42.5 us per
+              // step; compensated FP32 pairs took 36.7 and lost their low
+              // words at densities below ~1e-31)
+              const double t0 = a.dvol[1][z0 + i - 1], t1 = w1 ? a.dvol[1][zb + i - 1] : 0.0;
 #pragma unroll
               for (int v = 0; v < NV; ++v)
                 if (active(v)) {
-                  add_column_sum(tsum[v * NT + tid], lo(Un[v]), t0);
-                  if (w1) add_column_sum(tsum[v * NT + tid], hi(Un[v]), t1);
+                  double t = fma((double)lo(Un[v]), t0, tsum[v * NT + tid]);
+                  if (w1) t = fma((double)hi(Un[v]), t1, t);
+                  tsum[v * NT + tid] = t;
                 }
             }
             f2 ih[2] = {gx[S::GX_IW * 33], gy(S::GY_IW, i - 1)};
@@ -353,18 +357,14 @@ __global__ void __launch_bounds__(March2Shape<NSX, SPH>::NT, March2Shape<NSX, SP
   }
   __syncthreads();
   if (tsum) {
-    // the columns' sums times dvol[0] (and the absent axis's dvol[2]) in FP64,
-    // in place, then a tree in a fixed order per variable
-    double* const td = reinterpret_cast<double*>(tsum);
+    // the threads' sums times dvol[0] (and the absent axis's dvol[2]), then a
+    // tree in a fixed order per variable
     const double w = lown ? a.dvol[0][gi] * a.dvol[2][0] : 0.0;
 #pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      const float2 c = tsum[v * NT + tid];
-      td[v * NT + tid] = ((double)c.x + (double)c.y) * w;
-    }
+    for (int v = 0; v < NV; ++v) tsum[v * NT + tid] *= w;
     __syncthreads();
-    reduce_totals<NV, NT, NT>(td);
-    if (tid < NV) a.tot_part[(long long)tid * gridDim.x + blockIdx.x] = td[tid * NT];
+    reduce_totals<NV, NT, NT>(tsum);
+    if (tid < NV) a.tot_part[(long long)tid * gridDim.x + blockIdx.x] = tsum[tid * NT];
   }
   finish_step<NT>(a.ctrl, (double)smax, err, (unsigned long long)n_fb, 0ull, dtd, a.mirror);
 }

@@ -10,6 +10,8 @@ the Kahan-compensated FP32 partials of that pass against FP64 sums, 1e-6),
 conservation on a periodic box (mass, momenta and energy unchanged to
 roundoff), and determinism (two runs, the same bits).
 """
+import math
+
 import numpy as np
 import pytest
 
@@ -164,3 +166,23 @@ def test_totals_span_the_absent_angles(hydro_lib, n, riemann, precision):
     assert _rel(g.step_totals(), s.totals()) <= tol
     assert _rel(g.step_totals(), g.totals()) <= (1e-13 if precision == 64 else 1e-6)
     g.close()
+
+
+@pytest.mark.parametrize("riemann,scale", [(O.HLL, 1.0), (O.HLL, 1e-33), (O.HLL, 1e15), (O.HLLC, 1.0), (O.HLLC, 1e-33),
+                                           (O.HLLC, 1e15), (O.EXACT, 1.0)])
+@pytest.mark.parametrize("n", [(84, 1000), (200, 37)])
+def test_fp32_2d_step_totals_are_fp64_sums(hydro_lib, n, riemann, scale):
+    """The FP32 2D step sums U dV in FP64, whatever the units: within the rounding of a few hundred FP64 additions and
+    products (2^-53 each, on sum |U| dV) of the correctly rounded sums of the state it wrote."""
+    case = wl.smooth_random(2, list(n), 1, seed=31, riemann=riemann, bc=[(O.PERIODIC, O.PERIODIC), (O.REFLECTIVE, O.TRANSMISSIVE)])
+    g = hydro_lib.Grid.from_case(dict(case, U=(scale * case["U"]).astype(np.float32)), 32)
+    g.set_step_totals(True)
+    g.run(3, 0.4)
+    tot = g.step_totals()
+    U = g.get_state().astype(np.float64)[:, 0]
+    g.close()
+    dV = np.diff(case["faces"][1])[:, None] * np.diff(case["faces"][0])[None, :]
+    for v in range(len(U)):
+        terms = (U[v] * dV).ravel()
+        size = math.fsum(np.abs(terms))
+        assert abs(tot[v] - math.fsum(terms)) <= 400 * 2.0 ** -53 * size, (v, tot[v], math.fsum(terms))
