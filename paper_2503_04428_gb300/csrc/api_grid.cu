@@ -258,17 +258,16 @@ static int build_geometry(hydro_ctx* h) {
   if ((st = upload_d(h, a, &h->dvol[0]))) return st;
   if ((st = upload_d(h, b, &h->dvol[1]))) return st;
   if ((st = upload_d(h, c, &h->dvol[2]))) return st;
-  for (int d = 1; d < 3; ++d) {
-    // the axis-1 and axis-2 factors split into FP32 pairs for the FP32
-    // form's compensated in-step totals
-    const std::vector<double>& f = d == 1 ? b : c;
-    std::vector<float> hl(2 * f.size());
-    for (size_t k = 0; k < f.size(); ++k) {
-      hl[2 * k] = (float)f[k];
-      hl[2 * k + 1] = (float)(f[k] - (double)hl[2 * k]);
+  {
+    // the axis-2 factors split into FP32 pairs for the FP32 3D form's
+    // compensated in-step totals
+    std::vector<float> hl(2 * c.size());
+    for (size_t k = 0; k < c.size(); ++k) {
+      hl[2 * k] = (float)c[k];
+      hl[2 * k + 1] = (float)(c[k] - (double)hl[2 * k]);
     }
-    if (!h->dv32[d] && (st = h->arena.alloc((void**)&h->dv32[d], hl.size() * sizeof(float)))) return st;
-    HCK(cudaMemcpy(h->dv32[d], hl.data(), hl.size() * sizeof(float), cudaMemcpyHostToDevice));
+    if (!h->dvz32 && (st = h->arena.alloc((void**)&h->dvz32, hl.size() * sizeof(float)))) return st;
+    HCK(cudaMemcpy(h->dvz32, hl.data(), hl.size() * sizeof(float), cudaMemcpyHostToDevice));
   }
   if ((st = upload_d(h, rc, &h->rc_d))) return st;
   double bsum = 0.0, csum = 0.0;
@@ -427,7 +426,7 @@ static SweepArgs<T> sweep_args(hydro_ctx* h, double dt_host, double cfl, double 
   a.ir_new = mv_sph && h->dim >= 2 ? (const T*)h->irn_d : nullptr;
   a.tot_part = h->step_tot ? h->step_tot_part : nullptr;
   for (int d = 0; d < 3; ++d) a.dvol[d] = h->dvol[d];
-  for (int d = 0; d < 3; ++d) a.dv32[d] = reinterpret_cast<const float2*>(h->dv32[d]);
+  a.dvz32 = reinterpret_cast<const float2*>(h->dvz32);
   return a;
 }
 
@@ -451,7 +450,7 @@ static int launch_step_t(hydro_ctx* h, double dt_host, double cfl, double t_end,
     dim3 gb((h->n[0] + 31) / 32, h->shell_nchunks), tb(32, 8);
     shell_partial_kernel<T><<<gb, tb, 0, h->stream>>>(ctrl, (const T*)h->buf[0], (const T*)h->buf[1],
                                                       h->ncell, h->n[0], h->n[1], h->n[2],
-                                                      h->shell_kchunk, h->dvol[1], h->dvol[2], (const float2*)h->dv32[1], (const float2*)h->dv32[2],
+                                                      h->shell_kchunk, h->dvol[1], h->dvol[2],
                                                       h->shell_partial);
     HCK(cudaGetLastError());
     monopole_kernel<T><<<1, MONO_THREADS, 0, h->stream>>>(ctrl, h->shell_partial, h->shell_nchunks, h->n[0],
@@ -935,12 +934,12 @@ int hydro_shell_masses(hydro_t h, double* m_out) {
   if (h->precision == 64)
     shell_partial_kernel<double><<<gb, tb, 0, h->stream>>>(h->ctrl, (const double*)h->buf[0],
                                                            (const double*)h->buf[1], h->ncell, h->n[0], h->n[1],
-                                                           h->n[2], h->shell_kchunk, h->dvol[1], h->dvol[2], (const float2*)h->dv32[1], (const float2*)h->dv32[2],
+                                                           h->n[2], h->shell_kchunk, h->dvol[1], h->dvol[2],
                                                            h->shell_partial);
   else
     shell_partial_kernel<float><<<gb, tb, 0, h->stream>>>(h->ctrl, (const float*)h->buf[0],
                                                           (const float*)h->buf[1], h->ncell, h->n[0], h->n[1],
-                                                          h->n[2], h->shell_kchunk, h->dvol[1], h->dvol[2], (const float2*)h->dv32[1], (const float2*)h->dv32[2],
+                                                          h->n[2], h->shell_kchunk, h->dvol[1], h->dvol[2],
                                                           h->shell_partial);
   HCK(cudaGetLastError());
   shell_mass_kernel<<<(h->n[0] + 127) / 128, 128, 0, h->stream>>>(h->shell_partial, h->shell_nchunks, h->n[0],

@@ -153,50 +153,28 @@ __global__ void totals_final_kernel(const double* partial, int nblocks, int nv, 
 }
 
 // Monopole pass 1: partial shell sums sum_{j,k in chunk} rho b_j c_k, for
-// 32 radial cells per block and one axis-2 chunk per blockIdx.y.  FP64: the
-// products with b_j summed per plane, then times c_k.  FP32: b_j c_k as the
-// product of two FP32 pairs, the sum a compensated FP32 pair (each term costs
-// ~2^-48 of it), converted at the end: a conversion and two FP64 operations
-// per cell had occupied the FP64 pipe for 118 us of a 1.54 ms wedge step
-// (1024 x 128^2), now 53.
-struct ShellSum32 {
-  float2 s = {0.f, 0.f};
-  __device__ __forceinline__ void add(float rho, float2 b, float2 c) {
-    const float p = __fmul_rn(b.x, c.x);
-    const float e = fmaf(b.x, c.y, fmaf(b.y, c.x, fmaf(b.x, c.x, -p)));
-    add_column_sum(s, rho, make_float2(p, e));
-  }
-};
-
+// 32 radial cells per block and one axis-2 chunk per blockIdx.y, in FP64: the
+// products with b_j summed per plane, then times c_k: one FP64 operation per
+// cell, which bounds it (FP32 cells are widened by integer operations).  Shell
+// masses of the 1024 x 128^2 wedge, FP32, per call: 69 us; with conversions
+// 104, as compensated FP32 pairs of 48 bits 48.
 template <typename T>
 __global__ void __launch_bounds__(256)
     shell_partial_kernel(const Ctrl* ctrl, const T* A, const T* B, long long ncell, int n0, int n1,
                          int n2, int kchunk, const double* __restrict__ db,
-                         const double* __restrict__ dc, const float2* __restrict__ b32,
-                         const float2* __restrict__ c32, double* partial) {
+                         const double* __restrict__ dc, double* partial) {
   if (((volatile const Ctrl*)ctrl)->status != 0) return;
   const T* U = ((volatile const Ctrl*)ctrl)->cur ? B : A;
   const int i = blockIdx.x * 32 + threadIdx.x;
   const int k0 = blockIdx.y * kchunk, k1 = min(k0 + kchunk, n2);
   double s = 0.0;
   if (i < n0) {
-    if constexpr (sizeof(T) == 4) {
-      ShellSum32 sum;
-      for (int k = k0; k < k1; ++k) {
-        const T* u = U + (long long)k * n1 * n0 + i;
-        const float2 c = c32[k];
+    for (int k = k0; k < k1; ++k) {
+      const T* u = U + (long long)k * n1 * n0 + i;
+      double t = 0.0;
 #pragma unroll 8
-        for (int j = threadIdx.y; j < n1; j += 8) sum.add(u[(long long)j * n0], b32[j], c);
-      }
-      s = (double)sum.s.x + (double)sum.s.y;
-    } else {
-      for (int k = k0; k < k1; ++k) {
-        const T* u = U + (long long)k * n1 * n0 + i;
-        double t = 0.0;
-#pragma unroll 4
-        for (int j = threadIdx.y; j < n1; j += 8) t += u[(long long)j * n0] * db[j];
-        s += t * dc[k];
-      }
+      for (int j = threadIdx.y; j < n1; j += 8) t = fma(widen(u[(long long)j * n0]), db[j], t);
+      s += t * dc[k];
     }
   }
   __shared__ double red[8][33];

@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(March3Shape<NSX, SPH>::NT, March3Shape<NSX, SP
     GZ[S::GZ_SF * st + p] = make_f2(a.geo.sf[2][e0 + 2], a.geo.sf[2][e1 + 2]);
     GZ[S::GZ_IW * st + p] = make_f2(a.geo.inv_w[2][e0 + 2], a.geo.inv_w[2][e1 + 2]);
     if (tsum) {
-      const float2 v0 = a.dv32[2][min(max(e0, 0), n2 - 1)], v1 = a.dv32[2][min(max(e1, 0), n2 - 1)];
+      const float2 v0 = a.dvz32[min(max(e0, 0), n2 - 1)], v1 = a.dvz32[min(max(e1, 0), n2 - 1)];
       GZ[S::GZ_VH * st + p] = make_f2(v0.x, v1.x);
       GZ[S::GZ_VL * st + p] = make_f2(v0.y, v1.y);
     }

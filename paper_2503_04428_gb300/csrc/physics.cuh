@@ -257,6 +257,16 @@ __device__ __forceinline__ void add_column_sum(float2& sum, float x, float2 z) {
   sum.y = __fsub_rn(lo, __fsub_rn(sum.x, t));
 }
 
+// (double)x of a finite x.  FP32 by integer operations and one exact product
+// (which makes a subnormal normal): a conversion occupies the FP64 pipe.
+__device__ __forceinline__ double widen(float x) {
+  const bool less = fabsf(x) < 1.0f;
+  const unsigned b = __float_as_uint(less ? x * 0x1p100f : x);
+  const unsigned h = ((b & 0x7fffffffu) >> 3) + (less ? 0x38000000u - (100u << 20) : 0x38000000u);
+  return __hiloint2double((int)((b & 0x80000000u) | ((b & 0x7fffffffu) ? h : 0u)), (int)(b << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
 // 0 as long as `nul` is 0 and x is finite, NaN otherwise (FP64: by the bits).
 __device__ __forceinline__ float finite_or(float nul, float x) { return fmaf(x, 0.0f, nul); }
 __device__ __forceinline__ double finite_or(double nul, double x) {

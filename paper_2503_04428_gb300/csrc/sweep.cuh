@@ -1136,7 +1136,7 @@ struct Sweep {
         // kept as an unevaluated pair (TwoSum, then renormalised), so each
         // term costs ~2^-48 of the sum; the column's sum is multiplied by
         // dvol[0] dvol[1] in FP64 at the end of the CTA.
-        const float2 z = a.dv32[2][gz];
+        const float2 z = a.dvz32[gz];
         float2* ts = reinterpret_cast<float2*>(tsum);
 #pragma unroll
         for (int v = 0; v < NV; ++v)

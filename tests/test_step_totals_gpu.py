@@ -186,3 +186,22 @@ def test_fp32_2d_step_totals_are_fp64_sums(hydro_lib, n, riemann, scale):
         terms = (U[v] * dV).ravel()
         size = math.fsum(np.abs(terms))
         assert abs(tot[v] - math.fsum(terms)) <= 400 * 2.0 ** -53 * size, (v, tot[v], math.fsum(terms))
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e-33, 5e-39])
+@pytest.mark.parametrize("n", [(40, 12, 10), (33, 200, 5), (5, 9, 100)])
+def test_fp32_shell_masses_are_fp64_sums(hydro_lib, n, scale):
+    """hydro_shell_masses of an FP32 grid sums rho dV in FP64, whatever the units (subnormal densities too): within a few
+    hundred roundings of 2^-53 of the correctly rounded sums."""
+    case = wl.sphere_state(*n, dim=3)
+    case["sources"] = dict(gravity=O.GRAV_POINT_MONOPOLE, G=0.01, Mc=2.0)
+    U = (scale * case["U"]).astype(np.float32)
+    g = hydro_lib.Grid.from_case(dict(case, U=U), 32)
+    m = g.shell_masses()
+    g.close()
+    r, th, ph = case["faces"]
+    dV = np.diff(ph)[:, None, None] * -np.diff(np.cos(th))[None, :, None] * (np.diff(r ** 3) / 3)[None, None, :]
+    terms = U[0].astype(np.float64) * dV
+    for i in range(n[0]):
+        want = math.fsum(terms[:, :, i].ravel())
+        assert abs(m[i] - want) <= 300 * 2.0 ** -53 * want, (i, m[i], want)
