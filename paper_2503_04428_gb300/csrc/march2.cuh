@@ -275,15 +275,15 @@ __global__ void __launch_bounds__(March2Shape<NSX, SPH>::NT, March2Shape<NSX, SP
             for (int v = 0; v < NV; ++v) Uo[v] = ring[(((i + 1) & 3) * NV + v) * NT];
             new_state2<2, NSX>(a, dt, gx[S::GX_G * 33], s_hfac, Uo, acc, Un);
             if (tsum) {
-              // the thread's sums of U dvol[1], in FP64 (512 x 1536: 42.5 us per
-              // step; compensated FP32 pairs took 36.7 and lost their low
-              // words at densities below ~1e-31)
+              // the thread's sums of U dvol[1] in FP64 (512 x 1536: 38.2 us per
+              // step; with conversions 42.5; compensated FP32 pairs took 36.7
+              // and lost their low words at densities below ~1e-31)
               const double t0 = a.dvol[1][z0 + i - 1], t1 = w1 ? a.dvol[1][zb + i - 1] : 0.0;
 #pragma unroll
               for (int v = 0; v < NV; ++v)
                 if (active(v)) {
-                  double t = fma((double)lo(Un[v]), t0, tsum[v * NT + tid]);
-                  if (w1) t = fma((double)hi(Un[v]), t1, t);
+                  double t = fma(widen(lo(Un[v])), t0, tsum[v * NT + tid]);
+                  if (w1) t = fma(widen(hi(Un[v])), t1, t);
                   tsum[v * NT + tid] = t;
                 }
             }
