@@ -42,16 +42,29 @@ struct Gas {
 // cycles (measured; DFMA, DADD, DMUL and the compares alike, whatever the
 // active lanes), an integer instruction an ALU for about half a cycle.  So
 // the FP64 forms below count FP64 operations: signs and orders are read from
-// the bit patterns, and reciprocals and square roots take one third-order
-// step (error e -> O(e^3); Householder, The Numerical Treatment of a Single
-// Nonlinear Equation, 1970) from the documented PTX approximations, whose
-// relative error is below 2^-18: 3 and 5 FP64 operations against 4.5 and 7.5
-// of the correctly rounded ones, with errors of about 1 ulp.
+// the bit patterns, and reciprocals, quotients and square roots take Newton
+// steps (error e -> O(e^2)) from the documented PTX approximations, whose
+// relative error is below 2^-18, the last one with the residual of the
+// unrounded result (Markstein, Computation of elementary functions on the IBM
+// RISC System/6000 processor, 1990): 4, 5 and 6 FP64 operations against 4.5,
+// 7.5 and 7.5 of the operators, which they equal but for results within ~2^-20
+// of an ulp of the middle between two numbers.  (One third-order step each took
+// 3, 4 and 5, with errors of 0.501, 1.5 and 1 ulp: Sedov 128^3 9.06 ms per 3
+// steps against 9.46, Sod 1000 8.5 us per step against 8.9.)
 
 // FP32 takes the hardware approximations (1-2 ulp; the FP32 bulk's rounding
 // error is ~1e-7 per operation either way) in their .ftz forms: the others
 // guard subnormal arguments with four more instructions each, a fifth of the
 // exact solver's stream.
+
+__device__ __forceinline__ bool is_zero(double x) {
+  return ((__double2hiint(x) & 0x7fffffff) | __double2loint(x)) == 0;
+}
+__device__ __forceinline__ double rcp_estimate(double x) {  // to ~2^-36
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  return fma(r, fma(-x, r, 1.0), r);
+}
 
 // 1/x (x normal; FP32: |x| < 2^126, FP64: |x| < 2^1021).
 template <typename T> __device__ __forceinline__ T rcp(T x);
@@ -61,14 +74,11 @@ template <> __device__ __forceinline__ float rcp<float>(float x) {
   return r;
 }
 template <> __device__ __forceinline__ double rcp<double>(double x) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  double e = fma(-x, r, 1.0);
-  e = fma(e, e, e);
-  return fma(r, e, r);
+  const double r = rcp_estimate(x);
+  return fma(r, fma(-x, r, 1.0), r);
 }
 
-// Square roots of positive x.  The FP32 bulk takes x rsqrt(x) (about 3 ulp):
+// Square roots of 0 and normal numbers (FP64: from 2^-1000).  The FP32 bulk takes x rsqrt(x) (about 3 ulp):
 // the correctly rounded sqrtf sequence cost 2-3 % of the FP32 step's
 // instructions.  rsqrt_fast: 1/sqrt(x), of the smallest normal number if x is
 // less, so that every x >= 0 has a finite root x rsqrt_fast(x).
@@ -80,11 +90,15 @@ __device__ __forceinline__ float rsqrt_fast(float x) {
 template <typename T> __device__ __forceinline__ T dsqrt(T x);
 template <> __device__ __forceinline__ float dsqrt<float>(float x) { return x * rsqrt_fast(x); }
 template <> __device__ __forceinline__ double dsqrt<double>(double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double s = x * y;            // sqrt(x) (1 + d), x y^2 = 1 - e
-  const double e = fma(-s, y, 1.0);
-  return fma(s, e * fma(0.375, e, 0.5), s);
+  double h;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(h) : "d"(x));
+  double s = x * h;                                                      // sqrt(x)
+  h = __hiloint2double(__double2hiint(h) - (1 << 20), __double2loint(h));  // 1/(2 sqrt(x))
+  const double e = fma(-s, h, 0.5);
+  s = fma(s, e, s);
+  h = fma(h, e, h);
+  s = fma(fma(-s, s, x), h, s);
+  return is_zero(x) ? x : s;
 }
 
 // x > 0 (false for NaN).
@@ -114,9 +128,15 @@ template <> __device__ __forceinline__ double dpow<double>(double x, double y) {
 template <> __device__ __forceinline__ float dpow<float>(float x, float y) { return exp2f(y * log2f(x)); }
 
 // Quotient of the state conversions, wave speeds and the exact solver
-// (pressure functions, guess, Newton step, sampling): a times the reciprocal
-// above (Newton corrects its own iterates).  FP64: 4 operations against 7.5.
-template <typename T> __device__ __forceinline__ T qdiv(T a, T b) { return a * rcp<T>(b); }
+// (pressure functions, guess, Newton step, sampling).  FP32: a times the
+// reciprocal above (Newton corrects its own iterates).  FP64: a normal or 0, b
+// as for rcp, the quotient normal.
+template <typename T> __device__ __forceinline__ T qdiv(T a, T b);
+template <> __device__ __forceinline__ float qdiv<float>(float a, float b) { return a * rcp<float>(b); }
+template <> __device__ __forceinline__ double qdiv<double>(double a, double b) {
+  const double r = rcp_estimate(b), q = a * r;
+  return fma(fma(-b, q, a), r, q);
+}
 
 template <typename T> __device__ __forceinline__ T temp_tol();
 template <> __device__ __forceinline__ double temp_tol<double>() { return 1e-13; }
