@@ -160,7 +160,8 @@ __device__ __forceinline__ void hll2(const f2* WL, const f2* WR, f2* F, const Ga
   const f2 auL = a * uL, buR = b * uR;
   const f2 kL = auL + c, kR = buR - c;
   const f2 mL = WL[0] * kL, mR = WR[0] * kR;
-  F[0] = mL + mR;
+  auto carried = [&](f2 qL, f2 qR) { return fma2(c, qL - qR, fma2(buR, qR, auL * qL)); };
+  F[0] = carried(WL[0], WR[0]);
 #pragma unroll
   for (int d = 0; d < D; ++d) {
     F[1 + d] = fma2(mR, WR[1 + d], mL * WL[1 + d]);
@@ -169,7 +170,7 @@ __device__ __forceinline__ void hll2(const f2* WL, const f2* WR, f2* F, const Ga
   const f2 q = fma2(mR, speed_sq<D>(WR), mL * speed_sq<D>(WL));
   F[1 + D] = fma2(gas.half, q, fma2(fma2(kR, gas.igm1, buR), pR, fma2(kL, gas.igm1, auL) * pL));
 #pragma unroll
-  for (int s = 0; s < NSX; ++s) F[2 + D + s] = fma2(mR, WR[2 + D + s], mL * WL[2 + D + s]);
+  for (int s = 0; s < NSX; ++s) F[2 + D + s] = carried(WL[0] * WL[2 + D + s], WR[0] * WR[2 + D + s]);
 }
 
 // hllc_flux of physics.cuh on pairs.
