@@ -66,13 +66,15 @@ __device__ __forceinline__ double rcp_estimate(double x) {  // to ~2^-36
   return fma(r, fma(-x, r, 1.0), r);
 }
 
-// 1/x (x normal; FP32: |x| < 2^126, FP64: |x| < 2^1021).
-template <typename T> __device__ __forceinline__ T rcp(T x);
-template <> __device__ __forceinline__ float rcp<float>(float x) {
+__device__ __forceinline__ float rcp_estimate(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
+
+// 1/x (x normal; FP32: |x| < 2^126, FP64: |x| < 2^1021).
+template <typename T> __device__ __forceinline__ T rcp(T x);
+template <> __device__ __forceinline__ float rcp<float>(float x) { return rcp_estimate(x); }
 template <> __device__ __forceinline__ double rcp<double>(double x) {
   const double r = rcp_estimate(x);
   return fma(r, fma(-x, r, 1.0), r);
@@ -133,10 +135,13 @@ template <> __device__ __forceinline__ float dpow<float>(float x, float y) { ret
 // as for rcp, the quotient normal.
 template <typename T> __device__ __forceinline__ T qdiv(T a, T b);
 template <> __device__ __forceinline__ float qdiv<float>(float a, float b) { return a * rcp<float>(b); }
-template <> __device__ __forceinline__ double qdiv<double>(double a, double b) {
-  const double r = rcp_estimate(b), q = a * r;
+// (quotient: a/b with r = 1/b to ~2^-36 in hand)
+__device__ __forceinline__ float quotient(float a, float, float r) { return a * r; }
+__device__ __forceinline__ double quotient(double a, double b, double r) {
+  const double q = a * r;
   return fma(fma(-b, q, a), r, q);
 }
+template <> __device__ __forceinline__ double qdiv<double>(double a, double b) { return quotient(a, b, rcp_estimate(b)); }
 
 template <typename T> __device__ __forceinline__ T temp_tol();
 template <> __device__ __forceinline__ double temp_tol<double>() { return 1e-13; }
@@ -636,26 +641,49 @@ __device__ __forceinline__ float root_step(float y, float x, int n) {
   const float w = power_n(y, n);
   return fmaf(y * (x - w), rcp<float>(0.5f * (n + 1) * w + 0.5f * (n - 1) * x), y);
 }
-__device__ __forceinline__ double root_step(double y, double x, int n) {
-  const double w = power_n(y, n), den = fma(0.5 * (n + 1), w, 0.5 * (n - 1) * x);
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(den));
-  r = fma(r, fma(-den, r, 1.0), r);
-  return fma(y * (x - w), r, y);
+// FP64: the rounding of the powers is carried along (each product's exact
+// remainder by a fused operation), so that the root is hi + lo, hi its nearest
+// number.  With the plain residual x - y^n the last bit was wrong at times;
+// that and the quotients taken as products with rounded reciprocals (here, in
+// press_fn and in behind_fan) cost the exact solver 2-4 % in accuracy.  512
+// FP64 tubes take 2.01 ms with all of it, 1.83 without.
+struct Root {
+  double hi, lo;
+};
+__device__ __forceinline__ Root root_step(double y, double x, int n) {
+  const double y2 = y * y, e2 = fma(y, y, -y2);
+  const double y4 = y2 * y2, e4 = fma(y2 + y2, e2, fma(y2, y2, -y4));
+  double w = y4, e = e4;
+  if (n == 8) {
+    w = y4 * y4;
+    e = fma(y4 + y4, e4, fma(y4, y4, -w));
+  } else {
+    if (n & 2) {
+      w = y4 * y2;
+      e = fma(y4, e2, fma(e4, y2, fma(y4, y2, -w)));
+    }
+    if (n & 1) {
+      const double v = w * y;
+      e = fma(e, y, fma(w, y, -v));
+      w = v;
+    }
+  }
+  const double d = y * ((x - w) - e) * rcp_estimate(fma(0.5 * (n + 1), w, 0.5 * (n - 1) * x));
+  const double hi = y + d;
+  return {hi, (y - hi) + d};
 }
 // x^z, z = (gamma - 1)/(2 gamma), x > 0 a ratio of pressures.  For the usual
 // gammas 1/z is a small integer and x^z a root: a hardware estimate (relative
-// error ~1e-6) and one root_step, correct to about 1 ulp -- 10 FP64
-// operations, against the ~43 of exp2(z log2 x), whose FP32 form is also
-// twice as long and less exact.
+// error ~1e-6) and one root_step, correct to about 1 ulp (FP64 half of one) --
+// 17 FP64 operations, against the ~43 of exp2(z log2 x), whose FP32 form is
+// also twice as long and less exact.
 __device__ __forceinline__ float pow_z(float x, const Gas<float>& gas) {
   if (gas.root == 0) return dpow<float>(x, gas.z);
   float t;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(__log2f(x) * gas.z));
   return root_step(t, x, gas.root);
 }
-__device__ __forceinline__ double pow_z(double x, const Gas<double>& gas) {
-  if (gas.root == 0) return dpow<double>(x, gas.z);
+__device__ __forceinline__ Root root_z(double x, const Gas<double>& gas) {
   // log2 x from its exponent and leading 23 bits; 2^t scaled back by the exponent
   const int hx = __double2hiint(x), lx = __double2loint(x);
   const float m = __int_as_float(0x3f800000 | ((hx & 0xfffff) << 3) | (int)((unsigned)lx >> 29));
@@ -665,6 +693,28 @@ __device__ __forceinline__ double pow_z(double x, const Gas<double>& gas) {
   double y = (double)f;
   y = __hiloint2double(__double2hiint(y) + ((int)ti << 20), __double2loint(y));
   return root_step(y, x, gas.root);
+}
+__device__ __forceinline__ double pow_z(double x, const Gas<double>& gas) {
+  return gas.root ? root_z(x, gas).hi : dpow<double>(x, gas.z);
+}
+// Behind a rarefaction of pressure ratio q: t = q^z, the ratio of sound
+// speeds, and rho = rK q^(1/g) = rK q^(1 - 2z) (FP64: of a root, the quotient
+// of the exact products, to about half an ulp).
+__device__ __forceinline__ float behind_fan(float rK, float q, const Gas<float>& gas, float& t) {
+  t = pow_z(q, gas);
+  return qdiv(rK * q, t * t);
+}
+__device__ __forceinline__ double behind_fan(double rK, double q, const Gas<double>& gas, double& t) {
+  if (gas.root == 0) {
+    t = dpow<double>(q, gas.z);
+    return rK * dpow<double>(q, gas.ig);
+  }
+  const Root y = root_z(q, gas);
+  t = y.hi;
+  const double b = t * t, eb = fma(t + t, y.lo, fma(t, t, -b));
+  const double a = rK * q, ea = fma(rK, q, -a);
+  const double r = rcp_estimate(b), rho = a * r;
+  return fma(fma(-rho, eb, fma(-rho, b, a) + ea), r, rho);
 }
 // x^(1/z)
 template <typename T>
@@ -690,12 +740,12 @@ struct PressSide {
 template <typename T>
 __device__ __forceinline__ void press_fn(T p, T rp, const PressSide<T>& k, const Gas<T>& gas, T& f, T& df) {
   if (p > k.p) {
-    const T d = p - k.p, r = rcp<T>(p + k.B);
-    const T q = dsqrt(k.A * r);
+    const T d = p - k.p, s = p + k.B, r = rcp_estimate(s);
+    const T q = dsqrt(quotient(k.A, s, r));
     f = d * q;
     df = q * (T(1) - T(0.5) * (d * r));
   } else {
-    const T pz = pow_z(p * k.ip, gas);  // (p/pK)^((g-1)/(2g))
+    const T pz = pow_z(quotient(p, k.p, k.ip), gas);  // (p/pK)^((g-1)/(2g))
     f = k.f0 * (pz - T(1));
     // (p/pK)^(-(g+1)/(2g)) = (p/pK)^z / (p/pK)
     df = pz * (k.p * rp) * k.irc;
@@ -752,11 +802,11 @@ __device__ __forceinline__ int newton_star(T p, T rL, T uL, T pL, T cL, T rR, T 
   bool conv = false;
   for (int it = 1; it <= 100; ++it) {
     T fL, dfL, fR, dfR;
-    const T rp = rcp<T>(p);
+    const T rp = rcp_estimate(p);  // (for the derivatives)
     press_fn(p, rp, L, gas, fL, dfL);
     press_fn(p, rp, R, gas, fR, dfR);
     const T res = fL + fR + du;
-    T pn = p - qdiv(res, dfL + dfR);
+    T pn = p - res * rcp_estimate(dfL + dfR);  // (a correction: its leading digits do)
     if (pn < T(0)) pn = pfloor;
     const T dp = pn - p;
     const bool small = T(2) * fabs(dp) < tol * (pn + p);
@@ -819,9 +869,10 @@ __device__ __forceinline__ bool sample_xi(T S, T rL, T uL, T pL, T cL, T rR, T u
       p = ps;
     }
   } else if (x > uK - cK) {
-    const T pz = pow_z(q, gas);  // c*/c_K
-    if (x >= um - cK * pz) {
-      rho = qdiv(rK * q, pz * pz);  // q^(1/g) = q^(1 - 2z)
+    T t;  // c*/c_K
+    const T rs = behind_fan(rK, q, gas, t);
+    if (x >= um - cK * t) {
+      rho = rs;
       u = um;
       p = ps;
     } else {
