@@ -30,6 +30,9 @@
  *     rho f_1..rho f_S).  In spherical coordinates axes (0,1,2) are
  *     (r, theta, phi) and velocities (u_r, u_theta, u_phi).  Elements are
  *     double for precision 64 and float for precision 32.
+ *   - Densities and pressures, and in HLLC density times sound speed, have to
+ *     be normal numbers of the precision (from 1.2e-38 in FP32): smaller ones
+ *     end a step with an error.
  */
 #ifndef HYDRO_H
 #define HYDRO_H

@@ -29,3 +29,21 @@ def test_small_densities(hydro_lib, n, limiter):
     g.step(dt)
     check(ref.get_state(), g.get_state() * 2.0**80, case["dim"], case["gamma"], 32)
     g.close()
+
+
+@pytest.mark.parametrize("riemann", [O.HLL, O.HLLC, O.EXACT])
+@pytest.mark.parametrize("n", [(37,), (29, 17), (13, 9, 5)])
+def test_subnormal_densities_end_in_an_error(hydro_lib, n, riemann):
+    """Densities of 2^-127 (subnormal in FP32, whose reciprocals take them for 0): the step reports a failure and leaves
+    the state, and does not go on from wrong velocities."""
+    case = wl.smooth_random(len(n), list(n), 1, seed=7, bc=[(O.PERIODIC, O.PERIODIC)] * len(n), riemann=riemann)
+    g = hydro_lib.Grid.from_case(case, 32)
+    dt = g.cfl_dt(0.4)
+    U = (case["U"] * 2.0**-127).astype(np.float32)
+    g.set_state(U)
+    with pytest.raises(hydro_lib.HydroError) as e:
+        g.step(dt)
+    assert e.value.status in (hydro_lib.HYDRO_ERR_NEGATIVE_STATE, hydro_lib.HYDRO_ERR_NONFINITE, hydro_lib.HYDRO_ERR_NEWTON,
+                              hydro_lib.HYDRO_ERR_VACUUM)
+    assert np.array_equal(g.get_state(), U)
+    g.close()
