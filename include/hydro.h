@@ -160,8 +160,9 @@ int hydro_set_sources(hydro_t h, int gravity, const double g0[3], double G, doub
  *
  * hydro_set_exchange: mark side `side` (0 low, 1 high) of `axis` as
  * exchanged; ghost_faces[0..1] are the two face coordinates beyond that side,
- * nearest first (the neighbour's cells' geometry, so that a slab gives
- * bit for bit the arithmetic of the whole grid).  Call before
+ * nearest first (the neighbour's cells' geometry, so that a slab gives the
+ * arithmetic of the whole grid: bit for bit the one of the general sweep, from
+ * which the marching FP32 steps of a whole grid differ by rounding).  Call before
  * hydro_set_state; sides of a second axis are rejected (HYDRO_ERR_ARG).
  * Halos, in the state's precision, are laid out [v][layer][cross section]:
  * layer l is the ghost at distance l+1 from the side, and the cross section

@@ -431,15 +431,15 @@ static SweepArgs<T> sweep_args(hydro_ctx* h, double dt_host, double cfl, double 
 }
 
 // The plain 2D and 3D steps: FP32 with HLL or HLLC marches (march2.cuh,
-// march3.cuh); FP64, which is bound by the FP64 pipe, and the exact solver
-// take the general sweep.
+// march3.cuh; 3D where that pays); FP64, which is bound by the FP64 pipe, and
+// the exact solver take the general sweep.
 template <int DIM>
-static cudaError_t plain_step(const SweepArgs<double>& a, int nsx, int rs, cudaStream_t s, LaunchShape* sh) {
+static cudaError_t plain_step(const SweepArgs<double>& a, int nsx, int rs, int, cudaStream_t s, LaunchShape* sh) {
   return sweep_dispatch<double, DIM>(a, nsx, rs, s, sh);
 }
 template <int DIM>
-static cudaError_t plain_step(const SweepArgs<float>& a, int nsx, int rs, cudaStream_t s, LaunchShape* sh) {
-  if (rs == RS_EXACT) return sweep_dispatch<float, DIM>(a, nsx, rs, s, sh);
+static cudaError_t plain_step(const SweepArgs<float>& a, int nsx, int rs, int sms, cudaStream_t s, LaunchShape* sh) {
+  if (rs == RS_EXACT || (DIM == 3 && !march3_pays(a.n, nsx, sms))) return sweep_dispatch<float, DIM>(a, nsx, rs, s, sh);
   return DIM == 2 ? march2_dispatch(a, nsx, rs, s, sh) : march3_dispatch(a, nsx, rs, s, sh);
 }
 
@@ -484,8 +484,8 @@ static int launch_step_t(hydro_ctx* h, double dt_host, double cfl, double t_end,
   } else {
     switch (h->dim) {
       case 1: e = sweep_dispatch<T, 1>(a, h->nsx, h->riemann, h->stream, sh); break;
-      case 2: e = plain_step<2>(a, h->nsx, h->riemann, h->stream, sh); break;
-      default: e = plain_step<3>(a, h->nsx, h->riemann, h->stream, sh); break;
+      case 2: e = plain_step<2>(a, h->nsx, h->riemann, h->num_sms, h->stream, sh); break;
+      default: e = plain_step<3>(a, h->nsx, h->riemann, h->num_sms, h->stream, sh); break;
     }
   }
   if (e != cudaSuccess) return cuda_fail(e, "sweep launch");

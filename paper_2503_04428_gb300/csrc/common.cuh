@@ -136,17 +136,24 @@ struct LaunchShape {
 // 16 = 4 of 17.5.  A rule rather than a timed trial, so that
 // equal handles take equal chunks and the sums of the totals, grouped by CTA,
 // are the same bits.
-inline int plan_zchunk(long long tiles, int n2, long long slots, int per, double extra, int zmax) {
+struct ChunkPlan {
+  int z = 0;         // planes per CTA
+  double end = 0.0;  // its makespan
+};
+inline ChunkPlan plan_chunks(long long tiles, int n2, long long slots, int per, double extra, int zmax) {
   struct Plan {
     long long tiles = 0, slots = 0;
     int n2 = 0, per = 0;
     double extra = 0.0;
-    int zmax = 0, z = 0;
+    int zmax = 0;
+    ChunkPlan plan;
   };
-  static thread_local Plan last;
-  if (last.tiles == tiles && last.n2 == n2 && last.slots == slots && last.per == per && last.extra == extra &&
-      last.zmax == zmax)
-    return last.z;
+  // (a step may ask for the march's plan and the general sweep's; a few handles in turn)
+  static thread_local Plan kept[8];
+  static thread_local unsigned next = 0;
+  for (const Plan& p : kept)
+    if (p.tiles == tiles && p.n2 == n2 && p.slots == slots && p.per == per && p.extra == extra && p.zmax == zmax)
+      return p.plan;
   double least = 1e300;
   const int top = n2 < zmax ? n2 : zmax, stride = (top + 255) / 256;
   int best = top;
@@ -167,8 +174,11 @@ inline int plan_zchunk(long long tiles, int n2, long long slots, int per, double
       best = z;
     }
   }
-  last = {tiles, slots, n2, per, extra, zmax, best};
-  return best;
+  kept[next++ % 8] = {tiles, slots, n2, per, extra, zmax, {best, least}};
+  return {best, least};
+}
+inline int plan_zchunk(long long tiles, int n2, long long slots, int per, double extra, int zmax) {
+  return plan_chunks(tiles, n2, slots, per, extra, zmax).z;
 }
 
 template <typename T, int DIM>
@@ -182,7 +192,9 @@ struct StepsArgs {
 template <typename T, int DIM>
 cudaError_t steps_dispatch(const SweepArgs<T>& a, const StepsArgs& sa, int nsx, int rs, cudaStream_t s,
                            LaunchShape* sh, bool* taken);
-// The FP32 3D step of the plain ideal gas with HLL or HLLC (march3.cuh).
+// The FP32 3D step of the plain ideal gas with HLL or HLLC (march3.cuh), and
+// whether it is the faster form for a grid of these sizes (else the general sweep is).
+bool march3_pays(const int* n, int nsx, int sms);
 cudaError_t march3_dispatch(const SweepArgs<float>& a, int nsx, int rs, cudaStream_t s, LaunchShape* sh);
 // The FP32 2D step of the plain ideal gas with HLL or HLLC (march2.cuh).
 cudaError_t march2_dispatch(const SweepArgs<float>& a, int nsx, int rs, cudaStream_t s, LaunchShape* sh);

@@ -613,6 +613,36 @@ __global__ void __launch_bounds__(March3Shape<NSX, SPH>::NT, March3Shape<NSX, SP
   finish_step<NT>(a.ctrl, (double)smax, err, (unsigned long long)n_fb, 0ull, s_dt, a.mirror);
 }
 
+// The march's and the general sweep's time in microseconds, from their plans:
+// a CTA's step of two planes costs the march `step` (one CTA per SM), a plane
+// costs the general sweep `plane` alone on its SM and `more` with each further
+// CTA there.  Fitted to 35 grids from 8^3 to 192^3 and 32 x 32 x 2048 to 300 x
+// 300 x 20 (HLL and HLLC; each form within 25 %).  The form it picks is the
+// faster one, or at most 13 % slower, on all of them; the march's tiles of 30 x
+// 14, 10 or 8 owned cells fit widths next above their multiples badly.  HLLC,
+// one scalar, us per step, march and sweep: 64^3 54 and 41, 80^3 52 and 59, 96^3
+// 105 and 89, 128^3 182 and 228, 32 x 32 x 512 111 and 59, 192^3 510 and 572.
+// A single column of the general sweep's tiles (up to 16 x 16 cells) is faster
+// there (2 x 2 x 2000: 59 and 50).  Columns of 4096 planes or more march at any
+// width, so that the same long column gives the same bits in grids of any width
+// (the two forms round differently); they are wide in use, and narrow ones lose
+// (16 x 16 x 6600).
+template <int NSX>
+bool march3_pays(const int* n, int sms) {
+  using M = March3Shape<NSX, false>;
+  using S = SweepShape<float, 3, NSX>;
+  constexpr double step = NSX == 0 ? 6.1 : NSX == 1 ? 5.4 : 5.9;
+  constexpr double plane = NSX == 0 ? 3.9 : NSX == 1 ? 4.4 : 6.0, more = NSX == 0 ? 2.0 : NSX == 1 ? 1.8 : 2.1;
+  auto tiles = [&](int tx, int ty) { return (long long)((n[0] + tx - 1) / tx) * ((n[1] + ty - 1) / ty); };
+  const ChunkPlan m = plan_chunks(tiles(M::TX, M::TY), n[2], (long long)sms * M::MB, 2, 1.8, 2 * M::MAXLEN);
+  const long long t = tiles(S::TX, S::TY);
+  if (n[2] >= 4096) return true;
+  if (t == 1) return false;
+  const ChunkPlan s = plan_chunks(t, n[2], (long long)sms * S::MB, 1, 1.5, n[2]);
+  const double per_sm = (double)(t * ((n[2] + s.z - 1) / s.z)) / sms;
+  return 10.0 + step * m.end <= 8.5 + (plane + more * std::min(std::max(per_sm - 1.0, 0.0), S::MB - 1.0)) * s.end;
+}
+
 template <int NSX, int RS, bool SPH>
 cudaError_t launch_march3(const SweepArgs<float>& args, cudaStream_t s, LaunchShape* sh) {
   using S = March3Shape<NSX, SPH>;

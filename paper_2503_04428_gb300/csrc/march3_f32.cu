@@ -18,4 +18,8 @@ cudaError_t march3_dispatch(const SweepArgs<float>& a, int nsx, int rs, cudaStre
     default: return dispatch<3>(a, rs, s, sh);
   }
 }
+
+bool march3_pays(const int* n, int nsx, int sms) {
+  return nsx == 0 ? march3_pays<0>(n, sms) : nsx == 1 ? march3_pays<1>(n, sms) : march3_pays<3>(n, sms);
+}
 }  // namespace hydro

@@ -1708,7 +1708,7 @@ cudaError_t launch_sweep(const SweepArgs<T>& a, cudaStream_t s, LaunchShape* sh)
     }                                                                                         \
   }
 
-// The exact solver alone (the FP32 2D and 3D forms, whose HLL and HLLC steps march).
+// The exact solver alone (the FP32 2D forms, whose HLL and HLLC steps march).
 #define HYDRO_SWEEP_DISPATCH_EXACT(T, DIM)                                                    \
   template <>                                                                                 \
   cudaError_t sweep_dispatch<T, DIM>(const SweepArgs<T>& a, int nsx, int rs, cudaStream_t s,  \

@@ -1,6 +1,6 @@
-// Fused sweep kernels: float state, 3D grids with the exact Riemann solver (all scalar counts).
+// Fused sweep kernels: float state, 3D grids (all solvers and scalar counts).
 #include "sweep.cuh"
 
 namespace hydro {
-HYDRO_SWEEP_DISPATCH_EXACT(float, 3)
+HYDRO_SWEEP_DISPATCH(float, 3)
 }  // namespace hydro

@@ -75,3 +75,34 @@ def _one_step(hydro_lib, case):
         out.append((g.get_state(), g.step_totals()))
         g.close()
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+
+
+# sizes that the march takes (march3_pays), at and around its tiles' edges, with odd and remaining planes
+MARCHED = [(150, 70, 33), (119, 39, 81), (209, 83, 45), (211, 85, 46), (600, 40, 21), (299, 23, 35), (60, 8, 300),
+           (30, 300, 40), (149, 55, 150), (600, 420, 7), (1200, 2, 40), (899, 3, 31), (2, 3, 4100)]
+
+
+@pytest.mark.parametrize("k", range(len(MARCHED)))
+@pytest.mark.parametrize("ns", [0, 1, 2, 3])
+def test_cartesian_sizes_that_march(hydro_lib, k, ns):
+    case = wl.smooth_random(3, list(MARCHED[k]), ns, seed=70 + k, bc=BCS[(k + ns) % 4],
+                            riemann=[O.HLL, O.HLLC][(k + ns) % 2], limiter=[O.MINMOD, O.VANLEER, O.VANALBADA][k % 3])
+    _marches(hydro_lib, case)
+    _one_step(hydro_lib, case)
+
+
+@pytest.mark.parametrize("n", [(150, 70, 33), (299, 23, 35), (601, 41, 21)])
+@pytest.mark.parametrize("riemann", [O.HLL, O.HLLC])
+@pytest.mark.parametrize("ns", [0, 1, 3])
+def test_spherical_sizes_that_march(hydro_lib, n, riemann, ns):
+    case = wl.sphere_state(*n, n_scalars=ns, dim=3, riemann=riemann)
+    case["sources"] = dict(gravity=O.GRAV_POINT_MONOPOLE, G=0.01, Mc=2.0)
+    _marches(hydro_lib, case)
+    _one_step(hydro_lib, case)
+
+
+def _marches(hydro_lib, case):
+    g = hydro_lib.Grid.from_case(case, 32)
+    g.run(1, 0.4)
+    assert g.stats()["tile_x"] == 30  # (the general sweep's tiles are 16 wide)
+    g.close()
