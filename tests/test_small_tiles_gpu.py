@@ -141,3 +141,49 @@ def test_an_expired_wait_loses_the_state(hydro_lib, n):
     with pytest.raises(H.HydroError):
         g.set_step_wait(-1)
     g.close()
+
+
+def _sourced(kind, n):
+    if kind == "point":
+        case = wl.sphere_state(*n, n_scalars=1, dim=len(n), riemann=O.HLLC)
+        case["sources"] = dict(gravity=O.GRAV_POINT, G=3.0, Mc=2.0)
+    elif kind == "const":
+        case = wl.smooth_random(len(n), n, 1, seed=33, riemann=O.HLL, bc=[(T, R), (P, P)][:len(n)])
+        case["sources"] = dict(gravity=O.GRAV_UNIFORM, g0=(0.3, -0.2, 0.0), heating=O.HEAT_CONST, heat_params=(50.0,))
+    else:  # Ni-56 in CGS units on a grid of 1e14 cm: a run spans days, over which the heating decays
+        case = wl.smooth_random(len(n), n, 2, seed=34, riemann=O.HLLC, bc=[(T, R), (P, P)][:len(n)])
+        case["faces"] = [1e14 * np.asarray(f) for f in case["faces"]]
+        x = np.linspace(0, 1, n[0])[None, None, :] * np.ones((1, n[1] if len(n) > 1 else 1, 1))
+        vel = [1e7 * np.sin(4 * x)] + [np.zeros_like(x)] * (len(n) - 1)
+        case["U"] = wl.conserved(case["gamma"], 1e-9 * (1 + 0.3 * np.sin(6 * x)), vel, 1e5 * (1 + 0.2 * np.cos(5 * x)),
+                                 [np.full_like(x, 0.5), 0.1 + 0.05 * np.sin(3 * x)])
+        case["sources"] = dict(heating=O.HEAT_NI56, heat_params=(1,))
+    return case
+
+
+@pytest.mark.parametrize("precision", [64, 32])
+@pytest.mark.parametrize("n", [[300], [40, 33]])
+@pytest.mark.parametrize("kind", ["point", "const", "ni56"])
+def test_run_with_sources_equals_single_steps(hydro_lib, kind, n, precision):
+    """Gravity and heating in a many-step run, which keeps the time (and so the Ni-56 heating's decay) itself, against
+    single steps, at the bars of test_run_equals_single_steps; and without the sources the run ends elsewhere."""
+    case = _sourced(kind, n)
+    a, b, c = [hydro_lib.Grid.from_case(dict(case, sources=s), precision) for s in (case["sources"], case["sources"], None)]
+    for g in (a, b, c):
+        g.set_time(86400.0 * 5 if kind == "ni56" else 0.0)
+    t = a.run(12, 0.4)
+    c.run(12, 0.4)
+    for _ in range(12):
+        b.step(b.cfl_dt(0.4))
+    sa, sb = a.stats(), b.stats()
+    tol = 3e-13 if precision == 64 else 2e-4
+    assert sa["steps"] == sb["steps"] == 12 and abs(t - sb["t"]) <= tol * sb["t"]
+    A, B, C = [g.get_state().astype(np.float64) for g in (a, b, c)]
+    for v in range(len(A)):
+        assert np.abs(A[v] - B[v]).max() <= tol * max(np.abs(B[v]).max(), 1e-3 * np.abs(B[0]).max() if kind != "ni56" else 0)
+    e = 1 + len(n)
+    assert np.abs(A[e] - C[e]).max() > 100 * tol * np.abs(A[e]).max()  # the sources act
+    if kind == "ni56":
+        assert t - 86400.0 * 5 > 0.5 * 86400  # (of a decay time of 8.8 days)
+    for g in (a, b, c):
+        g.close()
