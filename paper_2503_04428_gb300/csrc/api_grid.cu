@@ -1133,7 +1133,6 @@ int hydro_run(hydro_t h, int nsteps, double cfl, double t_end, double* t_out) {
       cudaGraphExecDestroy(h->graph);
       h->graph = nullptr;
     }
-    // make sure kernel attributes are set outside of capture
     cudaGraph_t g;
     HCK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeRelaxed));
     st = launch_step(h, 0.0, cfl, t_end, h->ctrl);

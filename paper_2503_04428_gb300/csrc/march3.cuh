@@ -24,13 +24,15 @@
 // the Hancock increment and once with it, which costs less than keeping 6 NV
 // values in registers or parking them in shared memory.
 //
-// Measured against the general sweep (one GB300, whole passes of state in,
-// 10 or 5 steps, state out): Sedov 256^3 HLL with totals 13.3 -> 9.75 ms,
-// wedge 1024 x 128^2 (NV = 8, HLLC, monopole) 10.9 -> 8.45 ms; thread
+// Measured against the general sweep, which stays for the sizes that march3_pays
+// leaves it (one GB300, whole passes of state in, 10 or 5 steps, state out):
+// Sedov 256^3 HLL with totals 13.3 -> 9.75 ms, wedge 1024 x 128^2 (NV = 8, HLLC,
+// monopole) 10.9 -> 8.45 ms; thread
 // instructions per cell-update 2210 -> 990 (Sedov), 48 % of issue slots busy
 // with 16 warps per SM.  The two-warp barriers and the halo rows' staging then
 // gave 9.65 -> 9.34 and 7.81 -> 7.50 ms, the totals' widths staged with the
-// other axis-2 factors 9.33 -> 9.25.  Bound now: fixed-latency dependences at
+// other axis-2 factors 9.33 -> 9.25; HLL's mass flux by differences 9.25 -> 9.30.
+// Bound now: fixed-latency dependences at
 // that occupancy (registers: 128 at NV = 5, 168 at NV = 6 and 8): 4 % fewer
 // instructions (the totals' sums of both halves in pairs) gave nothing, and
 // sums by FP64 instructions cost 11.95 ms.
@@ -44,7 +46,7 @@
 namespace hydro {
 
 // Rows of warps per CTA, one CTA per SM: as many as leave the step its
-// registers without spills (NV = 5: 16 rows of 128 registers 9.75 ms, 12 of
+// registers (three scalar slots spill 8-12 bytes; NV = 5: 16 rows of 128 registers 9.75 ms, 12 of
 // 168 10.9; with the two-warp barriers 16 rows 9.49, 8 rows twice per SM
 // 9.73) and fit shared memory
 // with the totals (NV = 6: 12, NV = 8: 10).

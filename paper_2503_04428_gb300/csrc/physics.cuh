@@ -112,7 +112,7 @@ __device__ __forceinline__ bool is_pos(float x) { return x > 0.0f; }
 __device__ __forceinline__ bool is_pos(double x) {
   return (unsigned long long)__double_as_longlong(x) - 1ull < 0x7ff0000000000000ull;
 }
-// x >= 0 up to the sign of zero (-0 counts as negative).
+// x >= 0 (FP64: of the two zeros only +0).
 __device__ __forceinline__ bool is_nonneg(float x) { return x >= 0.0f; }
 __device__ __forceinline__ bool is_nonneg(double x) { return __double2hiint(x) >= 0; }
 // The smaller and the larger of two numbers (neither NaN).

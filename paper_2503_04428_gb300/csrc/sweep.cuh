@@ -1307,7 +1307,8 @@ __device__ __forceinline__ double step_dt(const volatile Ctrl* vc, double dt_hos
 // forms of the radiation EoS and the exact solver wait on their Newton chains:
 // two CTAs of 96 registers instead of one of 130-144 (wedge with radiation
 // 512 x 96^2 8.22 -> 5.6 ms per 5 steps, exact 101 x 67 x 53 2.15 -> 1.49 ms
-// per 10 steps, both with the chunks of plan_zchunk).
+// per 10 steps, both with the chunks of plan_zchunk; the exact form spills 48-88
+// bytes for it).
 template <typename T, int DIM, int NSX, int RS, int MODE, bool SMALL>
 __host__ __device__ constexpr int sweep_ctas() {
   if (SMALL) return 1;
