@@ -133,9 +133,11 @@ struct LaunchShape {
 // Measured: FP64 Sedov 128^3 (64 tiles, 152 slots, per 1, extra 1.5) 2.98 ms
 // at 56 planes (128 CTAs of 56 and 64 of 16 on the free slots: 57.5), 3.13 at
 // 19 = 3 waves of 20.5, 3.28 at 8 = 7 of 9.5, 3.39 at 64 = 1 of 65.5, 3.53 at
-// 16 = 4 of 17.5.  A rule rather than a timed trial, so that
-// equal handles take equal chunks and the sums of the totals, grouped by CTA,
-// are the same bits.
+// 16 = 4 of 17.5.  The other sweeps (radiation, dual energy, moving grids, the
+// exact solver; 64^3 to 128^3 and 96 x 40 x 200, both precisions) took 1.0 to 2.7
+// times as long with chunks chosen by timed trials, in the code of those trials.
+// A rule rather than a timed trial, so that equal handles take equal chunks and
+// the sums of the totals, grouped by CTA, are the same bits.
 struct ChunkPlan {
   int z = 0;         // planes per CTA
   double end = 0.0;  // its makespan
